@@ -182,7 +182,16 @@ typedef struct {
                                if the system's previous solve took at least
                                64 sweeps (or there was none): the grouping
                                costs about as much as ~60 sweeps' saving;
-                               0: every colour its own phase. */
+                               0: every colour its own phase.
+                               Plain systems with 0 or 4, max_sweeps above
+                               128, a global test (or none), no mixed or
+                               domain-wise update and the default block shape
+                               solve by dataflow: the same order with no
+                               phases at all (each update runs once its two
+                               bodies' earlier ones are done), so there is
+                               nothing to merge; results equal those of the
+                               barrier schedule except for the summation
+                               order of the residual. */
 } cd_params;
 
 typedef struct cd_system cd_system;
@@ -197,7 +206,9 @@ typedef struct {
     double wall_force[6];     /* sum of normal impulses on each wall / dt */
     int64_t n_phases;         /* grid-barrier phases per sweep: n_colours, or
                                  M - 1 fewer when the M last colours ran as
-                                 one phase (params.merge_last_colour) */
+                                 one phase (params.merge_last_colour); the
+                                 dataflow solve, which has no phases, counts
+                                 n_colours */
 } cd_solve_stats;
 
 typedef struct {

@@ -28,6 +28,7 @@ struct cd_system {
     int sweep_blocks;
     int sweep_threads;
     int colour_blocks;
+    int flow_records;                  // contacts a block of the dataflow solve keeps in shared memory
     int has_contacts;
     size_t ws_bytes;
     void* ws;
@@ -198,6 +199,16 @@ static size_t layout(cd_system* s, char* base, CdWork* w)
         t.mg_bmin = L.take<int>(base, mg ? nbk : 1);
         t.mg_bmax = L.take<int>(base, mg ? nbk : 1);
     }
+    {
+        const bool fl = s->g.flow != 0;
+        t.fl_V = L.take<char>(base, fl ? (n + 6) * cd_flow_body_bytes((int)s->p.dim, (int)s->p.precision) : 1);
+        t.fl_mask = L.take<unsigned long long>(base, fl ? n + 6 : 1);
+        t.fl_ord = L.take<unsigned>(base, fl ? cap : 1);
+        t.fl_part = L.take<char>(base, fl ? 64 * G : 1);
+        t.fl_P = L.take<char>(base, fl ? cap * (s->p.dim == 2 ? 2 : 4) * real : 1);
+        t.fl_P2 = L.take<char>(base, fl ? cap * (s->p.dim == 2 ? 2 : 4) * real : 1);
+        t.fl_Vprev = L.take<char>(base, fl ? 2 * (n + 6) * vrec : 1);
+    }
     t.rep_top = L.take<int>(base, npk);
     t.rep_dmax = L.take<int>(base, npk);
     t.rep_flag = L.take<int>(base, cap + 1);
@@ -347,6 +358,11 @@ static cd_status launch_solve(cd_system* s, int free_flight, int timed)
     CD_CUDA(s, cd_launch_pack(s->g, s->w, s->vel, s->omega, s->radius, s->inv_m, s->inv_I, s->f_ext, free_flight,
                               (int)s->p.precision, s->stream, &s->launches));
     if (timed && (st = mark(s)) != CD_OK) return st;
+    if (s->g.flow) {
+        CD_CUDA(s, cd_launch_flow(s->g, s->w, s->num_sms, s->flow_records, (int)s->p.precision, (int)s->p.criterion, s->p.alpha,
+                                  (int)s->p.max_sweeps, s->stream, &s->launches));
+        return CD_OK;
+    }
     CD_CUDA(s, cd_launch_sweep(s->g, s->w, s->sweep_blocks, s->sweep_threads, (int)s->p.precision,
                                (int)s->p.criterion, s->p.alpha,
                                (int)s->p.max_sweeps, s->pw, s->stream, &s->launches));
@@ -647,6 +663,20 @@ static cd_status create_impl(const cd_params* params, int64_t npk, const int64_t
                     g.ndom_total == 1 && !g.dyn_walls && p.tape_steps == 0 && cd_merge_label_blocks_per_sm() >= 1)
                        ? (p.merge_last_colour == 2 ? 2 : 3) : 0;
     g.merge_blocks = s->sweep_blocks;
+    // the dataflow solve: wherever its schedule may replace the barriers'.  A
+    // caller who asks for merging (1 to 3) or for another block shape gets the
+    // schedule that was asked for; up to 128 sweeps mode 4 keeps merging, which
+    // n_phases reports (longer solves are faster without it, see cd_flow.cu)
+    s->flow_records = cd_flow_records((int)p.dim, (int)p.precision, s->device);
+    g.flow = (npk == 1 && g.par_p == 0.0 && g.ndom_total == 1 && p.criterion != CD_CONV_LOCAL && p.max_sweeps > 128 &&
+              (p.merge_last_colour == 0 || p.merge_last_colour == 4) && s->sweep_threads == CD_SWEEP_THREADS &&
+              s->sweep_blocks == s->num_sms && s->flow_records >= 0) ? 1 : 0;
+    if (g.flow) {
+        g.merge_last = 0;
+        // records that cannot fit (more particles, so more contacts, than the blocks hold)
+        // leave the shared memory to the L1 cache
+        if (n > (int64_t)s->flow_records * s->num_sms) s->flow_records = 0;
+    }
     if (g.merge_last && !cd_sweep_fits(g, (int)p.precision, s->sweep_threads, s->sweep_blocks / s->num_sms)) {
         delete s;
         return fail(nullptr, CD_ERR_INVALID_ARG, "that many sweep blocks do not fit on one SM");

@@ -1,0 +1,845 @@
+// cd_flow.cu -- the impulse solve as a dataflow over the contacts (plain
+// systems): the colour order without a grid barrier per colour.
+//
+// The colour order says, for every body, in which order its contacts update
+// it.  Nothing else orders the updates: an update may run as soon as both its
+// bodies have had all their earlier ones.  So every body's velocity record
+// carries the number of updates it has had, and a warp (32 contacts of one
+// colour; the block's warps take the block's contacts colour by colour) looks
+// at its bodies' records until they carry the numbers it expects.  The blocks
+// are all resident (cooperative launch) and every warp takes its items in
+// colour order, so the earliest item not yet done can always run: no wait is
+// circular, and each is bounded as well.  The bits are those of the barrier
+// schedule.
+//
+// A block keeps its contacts' records (impulse included) in shared memory for
+// the whole solve where they fit; a system too large for that reads them
+// through L1.  One more warp takes the block's residual terms, publishes their
+// sum, gathers the other blocks' and runs the convergence test.  Its ~5,000
+// cycles stay off the path: after the first sweeps a sweep starts before the
+// test of the one (then two) before it is known.  The impulses of the last
+// three sweeps are kept in turn, and the velocities from before the last two,
+// so the sweeps begun past the last one are taken back.
+//
+// What bounds it: in FP64 the FP64 pipe (19 cycles a warp instruction on an
+// SM, 29 of them a warp of contacts) while the neighbours' records are under
+// way between the SMs; in FP32, and in small systems, the way of a record
+// from SM to SM (~500 cycles on a die, ~850 across) once per colour, plus the
+// update (FP64: ~1,700 cycles for a whole warp of contacts; ~1,100 for 16
+// contacts split over lane pairs, where a block has few).  Per sweep, against
+// the barrier schedule (grid barrier 2,900 cycles a colour, then the velocity
+// loads): 100,000-disc pile FP64 28.4 -> 18.1 us, FP32 18.0 -> 10.2 us;
+// 5,000 discs FP64 20.6 -> 9.9 us; 2,000 discs 20.9 -> 10.1 us.  Tried and not kept: one lane
+// looking for its warp (FP32 7% slower, 5,000 discs 12%), pauses between looks
+// (5,000 discs 2 to 15% slower), 15 or 7 updating warps in place of 11 (FP64 2
+// and 17% slower), records through L1 (FP64 pile 24.3 us a sweep).
+#include "cd_sweep_core.cuh"
+
+// ---------------------------------------------------------------------------
+// Tagged velocity records.  A record is made of 64-bit elements, each 48 bits
+// of velocity and a 16-bit tag, the number of updates its body has had (modulo
+// 2^16).  Every element says by itself which update it belongs to, so a reader
+// that finds the tag it expects in all of them has that update's velocities:
+// no fence, no flag beside the data.  (A reader is at most one pass, 64
+// updates, behind a writer.)  Three numbers make a group: FP64 four elements
+// (one 256-bit access), FP32 two (one 128-bit access); 2D has one group
+// (v_x, v_y, omega), 3D two (v, omega).
+// ---------------------------------------------------------------------------
+typedef unsigned long long u64;
+template <typename T> struct FlowGroup;
+template <> struct FlowGroup<double> { static constexpr int N = 4; };
+template <> struct FlowGroup<float> { static constexpr int N = 2; };
+
+__device__ __forceinline__ void flow_load(const u64* p, u64 (&e)[4])
+{
+    asm volatile("ld.relaxed.gpu.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(e[0]), "=l"(e[1]), "=l"(e[2]), "=l"(e[3]) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void flow_load(const u64* p, u64 (&e)[2])
+{
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(e[0]), "=l"(e[1]) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void flow_store(u64* p, const u64 (&e)[4])
+{
+    asm volatile("st.relaxed.gpu.global.v4.b64 [%0], {%1, %2, %3, %4};"
+                 :: "l"(p), "l"(e[0]), "l"(e[1]), "l"(e[2]), "l"(e[3]) : "memory");
+}
+__device__ __forceinline__ void flow_store(u64* p, const u64 (&e)[2])
+{
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" :: "l"(p), "l"(e[0]), "l"(e[1]) : "memory");
+}
+
+__device__ __forceinline__ u64 flow_pair(unsigned lo, unsigned hi) { return ((u64)hi << 32) | (u64)lo; }
+__device__ __forceinline__ unsigned flow_lo(u64 x) { return (unsigned)x; }
+__device__ __forceinline__ unsigned flow_hi(u64 x) { return (unsigned)(x >> 32); }
+__device__ __forceinline__ unsigned flow_tag(u64 e) { return (unsigned)(e >> 48); }
+
+// Three FP64 numbers: their low 48 bits in elements 0 to 2, their top 16 bits
+// together in element 3.
+__device__ __forceinline__ void flow_pack(double a, double b, double c, unsigned tag, u64 (&e)[4])
+{
+    const u64 x = (u64)__double_as_longlong(a), y = (u64)__double_as_longlong(b), z = (u64)__double_as_longlong(c);
+    e[0] = flow_pair(flow_lo(x), __byte_perm(flow_hi(x), tag, 0x5410));
+    e[1] = flow_pair(flow_lo(y), __byte_perm(flow_hi(y), tag, 0x5410));
+    e[2] = flow_pair(flow_lo(z), __byte_perm(flow_hi(z), tag, 0x5410));
+    e[3] = flow_pair(__byte_perm(flow_hi(x), flow_hi(y), 0x7632), __byte_perm(flow_hi(z), tag, 0x5432));
+}
+__device__ __forceinline__ void flow_unpack(const u64 (&e)[4], double& a, double& b, double& c)
+{
+    a = __hiloint2double((int)__byte_perm(flow_hi(e[0]), flow_lo(e[3]), 0x5410), (int)flow_lo(e[0]));
+    b = __hiloint2double((int)__byte_perm(flow_hi(e[1]), flow_lo(e[3]), 0x7610), (int)flow_lo(e[1]));
+    c = __hiloint2double((int)__byte_perm(flow_hi(e[2]), flow_hi(e[3]), 0x5410), (int)flow_lo(e[2]));
+}
+// Three FP32 numbers: a and b whole, c in two halves.
+__device__ __forceinline__ void flow_pack(float a, float b, float c, unsigned tag, u64 (&e)[2])
+{
+    const unsigned z = __float_as_uint(c);
+    e[0] = flow_pair(__float_as_uint(a), __byte_perm(z, tag, 0x5410));
+    e[1] = flow_pair(__float_as_uint(b), __byte_perm(z, tag, 0x5432));
+}
+__device__ __forceinline__ void flow_unpack(const u64 (&e)[2], float& a, float& b, float& c)
+{
+    a = __uint_as_float(flow_lo(e[0]));
+    b = __uint_as_float(flow_lo(e[1]));
+    c = __uint_as_float(__byte_perm(flow_hi(e[0]), flow_hi(e[1]), 0x5410));
+}
+
+// A body's record.
+template <int DIM, typename T>
+struct FlowBody {
+    static constexpr int G = (DIM == 2) ? 1 : 2;
+    static constexpr int N = FlowGroup<T>::N;
+    u64 e[G][N];
+    __device__ __forceinline__ void load(const u64* p)
+    {
+#pragma unroll
+        for (int q = 0; q < G; ++q) flow_load(p + q * N, e[q]);
+    }
+    __device__ __forceinline__ void store(u64* p) const
+    {
+#pragma unroll
+        for (int q = 0; q < G; ++q) flow_store(p + q * N, e[q]);
+    }
+    __device__ __forceinline__ bool has(unsigned tag) const
+    {
+        unsigned off = 0u;
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+#pragma unroll
+            for (int j = 0; j < N; ++j) off |= flow_hi(e[q][j]) ^ (tag << 16);
+        return (off >> 16) == 0u;
+    }
+    __device__ __forceinline__ void pack(const typename Vec<T>::V4& v, const typename Vec<T>::V4& o, unsigned tag)
+    {
+        flow_pack(v.x, v.y, v.z, tag, e[0]);
+        if constexpr (DIM == 3) flow_pack(o.x, o.y, o.z, tag, e[1]);
+    }
+    __device__ __forceinline__ void unpack(typename Vec<T>::V4& v, typename Vec<T>::V4& o) const
+    {
+        flow_unpack(e[0], v.x, v.y, v.z);
+        v.w = (T)0;
+        if constexpr (DIM == 3) {
+            flow_unpack(e[1], o.x, o.y, o.z);
+            o.w = (T)0;
+        }
+    }
+};
+
+// A block's sum of residual terms, tagged with its pass.
+struct FlowSum { u64 e[2]; };
+__device__ __forceinline__ void flow_sum_store(FlowSum* p, double x, unsigned tag)
+{
+    // 48 bits and 16 bits of the sum, each with a tag
+    const u64 b = (u64)__double_as_longlong(x);
+    const u64 e[2] = {(b & 0xffffffffffffULL) | ((u64)tag << 48), (b >> 48) | ((u64)tag << 48)};
+    flow_store(p->e, e);
+}
+__device__ __forceinline__ bool flow_sum_is(const u64 (&e)[2], unsigned tag)
+{
+    return flow_tag(e[0]) == (tag & 0xffffu) && flow_tag(e[1]) == (tag & 0xffffu);
+}
+__device__ __forceinline__ double flow_sum_of(const u64 (&e)[2])
+{
+    return __longlong_as_double((long long)((e[0] & 0xffffffffffffULL) | (e[1] << 48)));
+}
+
+#define FLOW_WORKERS 11                           // warps that update contacts
+#define FLOW_THREADS (32 * (FLOW_WORKERS + 1))    // and one that runs the convergence test
+#define FLOW_ROWS 4                               // rows of tagged block sums
+#define FLOW_SLOTS 4                              // passes whose residual terms are kept
+#define FLOW_LAG1 16                              // from this pass on one starts before the test of the one before is
+#define FLOW_LAG2 32                              // known, from this one on two do: what they change can be taken back
+// FP64 2D: a block's contacts of a colour up to which two lanes share one.  At 64
+// the pairs fill four warps, one for each of the SM's FP64 quarters, 14
+// instructions deep in place of two warps 24 deep; beyond, a quarter would
+// take two warps of 14, more than one of 24.
+#define FLOW_SPLIT 64
+
+// What the block's warps share.
+struct FlowShared {
+    int lo[CD_KMAX], end[CD_KMAX];   // this block's positions of each colour
+    int base[CD_KMAX + 1];           // first of its warp items (32 contacts, or 16 split over two lanes each)
+    int slot[CD_KMAX + 1];           // contacts of the colours before: place in the block's records
+    int before[CD_KMAX];             // the colour with items before each (in turn), or -1 - the last one
+    int done[CD_KMAX];               // its warp items done, over all passes
+    double acc[FLOW_SLOTS][FLOW_WORKERS][32]; // residual terms of a pass by worker lane
+    int arrived[FLOW_SLOTS];         // workers that have left them (counted over the passes of a slot)
+    int decided;                     // last pass the test is known of
+    int stop;                        // the sweep the iteration ends with, once known (else -1)
+    int dead;                        // a wait gave up
+    double ravg, resid;
+    int converged;
+};
+
+__device__ __forceinline__ int flow_ld(const int* p) { return *(volatile const int*)p; }
+
+// A bounded wait: gives up CD_WAIT_NS after its first look at the clock, or
+// when another block has flagged an error.
+struct FlowBound {
+    unsigned spins = 0;
+    u64 t0 = 0;
+    __device__ __forceinline__ bool look(CdCtrl* ctrl)
+    {
+        if (t0 == 0) t0 = cd_globaltimer();
+        else if (cd_globaltimer() - t0 > CD_WAIT_NS) {
+            atomicCAS(&ctrl->error, CDE_NONE, CDE_TIMEOUT);
+            return false;
+        }
+        return cd_ld_volatile_int(&ctrl->error) == CDE_NONE;
+    }
+    __device__ __forceinline__ bool go(CdCtrl* ctrl) { return (++spins & 255u) != 0u || look(ctrl); }
+};
+
+// Waits in shared memory until *p >= v; false when a wait gave up.
+__device__ __forceinline__ bool flow_wait_shared(CdCtrl* ctrl, FlowShared& sh, const int* p, int v)
+{
+    FlowBound bound;
+    while (flow_ld(p) < v) {
+        if (flow_ld(&sh.dead)) return false;
+        if (!bound.go(ctrl)) {
+            *(volatile int*)&sh.dead = 1;
+            return false;
+        }
+    }
+    __threadfence_block();
+    return true;
+}
+
+// Looks again at the records at pa and pb (null: none) until they carry their
+// tags (the caller has looked once); the lanes of a warp leave together.
+// False when a wait gave up.
+template <int DIM, typename T>
+__device__ __forceinline__ bool flow_wait(CdCtrl* ctrl, FlowShared& sh, const u64* pa, unsigned ta, const u64* pb,
+                                          unsigned tb, FlowBody<DIM, T>& A, FlowBody<DIM, T>& B)
+{
+    FlowBound bound;
+    bool ra = !pa || A.has(ta), rb = !pb || B.has(tb);
+    while (!__all_sync(0xffffffffu, ra && rb)) {
+        if (!ra) A.load(pa);
+        if (!rb) B.load(pb);
+        ra = ra || A.has(ta);
+        rb = rb || B.has(tb);
+        if ((++bound.spins & 63u) == 0u && !__all_sync(0xffffffffu, bound.look(ctrl) && !flow_ld(&sh.dead))) {
+            *(volatile int*)&sh.dead = 1;
+            return false;
+        }
+    }
+    return true;
+}
+
+__device__ __forceinline__ double shfl_pair(double v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
+
+// The control warp's part of a pass: the block's sum, published, every block's
+// sums gathered, the test.  The sums of lanes, then of blocks, are taken in a
+// fixed order, the same in every block.  Returns false when a wait gave up.
+__device__ __forceinline__ bool flow_control(CdCtrl* ctrl, FlowShared& sh, FlowSum* part, int pass, int nb, int nc,
+                                             int crit, double alpha, int max_sweeps, double& xprev)
+{
+    const int lane = threadIdx.x & 31;
+    bool on = true;
+    if (lane == 0) on = flow_wait_shared(ctrl, sh, &sh.arrived[pass % FLOW_SLOTS],
+                                          FLOW_WORKERS * (pass / FLOW_SLOTS + 1));
+    if (!__shfl_sync(0xffffffffu, (int)on, 0)) return false;
+    __syncwarp();
+    double x = 0.0;
+#pragma unroll
+    for (int u = 0; u < FLOW_WORKERS; ++u) {
+        const double y = *(volatile double*)&sh.acc[pass % FLOW_SLOTS][u][lane];
+        if (__any_sync(0xffffffffu, __double_as_longlong(y) != 0)) x += y;
+    }
+    x = warp_sum_nz(x);
+    FlowSum* row = part + (size_t)(pass % FLOW_ROWS) * nb;
+    const unsigned tag = (unsigned)pass + 1u;
+    if (lane == 0) flow_sum_store(row + blockIdx.x, x, tag);
+    x = 0.0;
+    FlowBound bound;
+    for (int b0 = 0; b0 < nb; b0 += 160) {
+        // five blocks a lane at a time, their loads in flight together
+        u64 f[5][2];
+        bool have = false;
+        while (!__all_sync(0xffffffffu, have)) {
+            have = true;
+#pragma unroll
+            for (int u = 0; u < 5; ++u) {
+                const int b = b0 + 32 * u + lane;
+                if (b < nb) flow_load(row[b].e, f[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 5; ++u)
+                if (b0 + 32 * u + lane < nb) have = have && flow_sum_is(f[u], tag);
+            on = bound.go(ctrl) && !flow_ld(&sh.dead);
+            if (!__all_sync(0xffffffffu, on)) return false;
+        }
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+            if (b0 + 32 * u + lane < nb) x += flow_sum_of(f[u]);
+    }
+    x = warp_sum(x);
+    if (lane == 0) {
+        // the ratio of the test against its threshold by products; only where
+        // that is within rounding of the threshold (or at the end) the test
+        // itself, whose FP64 divisions take longer than the rest
+        bool end = pass >= max_sweeps;
+        if (pass > 0 && crit != CD_CONV_NONE && !end) {
+            const double a = (crit == CD_CONV_GLOBAL_SQ) ? sqrt(alpha) : alpha;
+            const double s = x + xprev, off = fabs(x - xprev) - a * s;
+            end = !(off > s * (1e-15 * (1.0 + a)));
+        }
+        if (end) {
+            const double ra = x / (double)nc;
+            double rs = 0.0;
+            int cv = 0;
+            if (pass > 0) global_test(ra, xprev / (double)nc, crit, alpha, rs, cv);
+            *(volatile double*)&sh.ravg = ra;
+            *(volatile double*)&sh.resid = rs;
+            *(volatile int*)&sh.converged = cv;
+            if (cv || pass >= max_sweeps) *(volatile int*)&sh.stop = pass;
+        }
+        __threadfence_block();
+        *(volatile int*)&sh.decided = pass;
+        xprev = x;
+    }
+    return true;
+}
+
+// The block's contact records kept in shared memory for the solve (structure
+// of arrays over `cap` contacts): all that an update needs except velocities.
+template <int DIM, typename T>
+struct FlowRecords {
+    typedef typename Vec<T>::V4 T4;
+    typedef typename Vec<T>::V2 T2;
+    typedef typename std::conditional<DIM == 2, T2, T4>::type TP;    // impulse record
+    typedef typename std::conditional<DIM == 2, T, T2>::type TM;     // m_t, or (m_n, m_t)
+    static constexpr int BYTES = (int)(sizeof(T4) + sizeof(TP) + 3 * sizeof(T2) + sizeof(TM) + sizeof(int2) +
+                                       sizeof(unsigned));
+    T4* geo;
+    TP* P;
+    T2* s0;   // (1/m_a, r_a)
+    T2* s1;   // (r_a/I_a, 1/m_b)
+    T2* s2;   // (r_b, r_b/I_b)
+    TM* m;
+    int2* ab;
+    unsigned* ord;
+    __device__ __forceinline__ FlowRecords(char* base, int cap)
+    {
+        geo = (T4*)base;
+        P = (TP*)(geo + cap);
+        s0 = (T2*)(P + cap);
+        s1 = s0 + cap;
+        s2 = s1 + cap;
+        m = (TM*)(s2 + cap);
+        ab = (int2*)(m + cap);
+        ord = (unsigned*)(ab + cap);
+    }
+};
+
+// The FP64 2D update of core2d by two lanes a contact: the even one takes the
+// normal row and the y components, the odd one the tangential row and the x
+// components; the same operations with the same rounding, 14 in a row instead
+// of 24.  What differs between the lanes are operands chosen before the
+// velocities are there: between two FP64 instructions a select or a shuffle
+// costs ~44 cycles beyond their own 64 each.
+struct FlowHalf {
+    double c1, c2, c3, c4, c5, bias, Pold;
+    __device__ __forceinline__ void choose(bool odd, const Rec<2, double>& r)
+    {
+        c1 = odd ? -r.geo.y : r.geo.x;
+        c2 = odd ? r.geo.x : r.geo.y;
+        c3 = odd ? -r.sa.y : 1.0;
+        c4 = odd ? -r.sb.y : 0.0;
+        c5 = odd ? -r.mt : -r.geo.w;
+        bias = r.geo.z;
+        Pold = odd ? r.P.y : r.P.x;
+    }
+    // Returns this lane's impulse component, and in v1 the new velocity record
+    // of body a (even lane) or b (odd).  wall_k: b - n (>= 0: b is the
+    // force-controlled wall wall_k, which moves along its normal only).
+    __device__ __forceinline__ double update(bool odd, const Rec<2, double>& r, const Vec<double>::V4& va,
+                                             const Vec<double>::V4& vb, int wall_k, bool apply_only,
+                                             Vec<double>::V4& v1) const
+    {
+        const double xa = odd ? va.x : va.y, xb = odd ? vb.x : vb.y;
+        double Pnew = Pold, d = Pold;
+        if (!apply_only) {
+            const double u3 = odd ? va.z : bias, u4 = odd ? vb.z : 0.0;
+            const double dvx = __dsub_rn(vb.x, va.x), dvy = __dsub_rn(vb.y, va.y);
+            double u = __fma_rn(dvy, c2, __dmul_rn(dvx, c1));     // u_n | (dv x n)
+            u = __fma_rn(c3, u3, u);                              // b + u_n | - r_a w_a
+            u = __fma_rn(c4, u4, u);                              //         | - r_b w_b
+            const double Ps = __fma_rn(c5, u, Pold);
+            const double lim = pos_part(shfl_pair(__dmul_rn(r.mu, Ps)));   // mu max(P_n*, 0)
+            Pnew = odd ? clamp_sym(Ps, lim) : pos_part(Ps);
+            d = __dsub_rn(Pnew, Pold);
+        }
+        const double e = shfl_pair(d);
+        const double dPn = odd ? e : d, dPt = odd ? d : e;
+        const double dP = __fma_rn(dPn, c2, __dmul_rn(dPt, c1));  // y | x
+        const double xa1 = __fma_rn(-r.sa.x, dP, xa);
+        double xb1 = __fma_rn(r.sb.x, dP, xb);
+        double om = __fma_rn(odd ? -r.sb.z : -r.sa.z, dPt, odd ? vb.z : va.z);   // of this lane's body
+        if (wall_k >= 0) {
+            if (((wall_k >> 1) == 0) != odd) xb1 = 0.0;
+            if (odd) om = 0.0;
+        }
+        const double other = shfl_pair(odd ? xa1 : xb1);
+        v1.x = odd ? xb1 : other;
+        v1.y = odd ? other : xa1;
+        v1.z = om;
+        v1.w = 0.0;
+        return Pnew;
+    }
+};
+
+__device__ __forceinline__ void* flow_impulses(const CdWork& w, int pass)
+{
+    const int u = pass % 3;
+    return u == 0 ? w.c_P : u == 1 ? w.fl_P : w.fl_P2;
+}
+
+template <int DIM, typename T>
+__global__ void __launch_bounds__(FLOW_THREADS, 1)
+k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
+{
+    typedef FlowBody<DIM, T> Body;
+    typedef FlowRecords<DIM, T> Records;
+    typedef typename Vec<T>::V4 T4;
+    typedef typename Vec<T>::V2 T2;
+    typedef typename Records::TP TP;
+    typedef typename Records::TM TM;
+    constexpr int EB = Body::G * Body::N;   // elements of a body's record
+    constexpr bool F64_2D = (DIM == 2) && std::is_same<T, double>::value;
+    // |P| of an update is taken while the warp's next one waits (3D FP64 has no registers left for it)
+    constexpr bool DEFER = (DIM == 2) || std::is_same<T, float>::value;
+    extern __shared__ __align__(128) char s_rec[];
+    __shared__ FlowShared sh;
+    __shared__ double s_red[FLOW_WORKERS + 1][3];
+    __shared__ double s_bc;
+    CdCtrl* ctrl = w.ctrl;
+    if (ctrl->skip) return;
+    const int nc = ctrl->nc, K = ctrl->ncolours, nb = gridDim.x;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    u64 epoch = 0;
+    u64* VT = (u64*)w.fl_V;
+    FlowSum* part = (FlowSum*)w.fl_part;
+    T4* V = (T4*)w.V;
+    T4* Vprev = (T4*)w.fl_Vprev;
+    constexpr int RW = (DIM == 2) ? 1 : 2;
+    const int nbody = g.n + (g.dyn_walls ? 6 : 0);
+
+    // this block's positions of each colour, and their warp items
+    if (threadIdx.x < 32) {
+        int run = 0, srun = 0;
+        for (int k0 = 0; k0 < K; k0 += 32) {
+            const int k = k0 + lane;
+            int m = 0, c = 0;
+            if (k < K) {
+                const int lo = w.colour_off[k], hi = w.colour_off[k + 1];
+                const int chunk = (hi - lo + nb - 1) / nb;
+                const int b0 = min(lo + (int)blockIdx.x * chunk, hi), e = min(b0 + chunk, hi);
+                sh.lo[k] = b0;
+                sh.end[k] = e;
+                c = e - b0;
+                m = (F64_2D && c <= FLOW_SPLIT) ? (c + 15) >> 4 : (c + 31) >> 5;
+            }
+            int incl = m, ci = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o), z = __shfl_up_sync(0xffffffffu, ci, o);
+                if (lane >= o) { incl += y; ci += z; }
+            }
+            if (k < K) { sh.base[k + 1] = run + incl; sh.slot[k + 1] = srun + ci; }
+            run += __shfl_sync(0xffffffffu, incl, 31);
+            srun += __shfl_sync(0xffffffffu, ci, 31);
+        }
+        if (lane == 0) sh.base[0] = sh.slot[0] = 0;
+        __syncwarp();
+        if (lane == 0) {
+            for (int u = 0; u < FLOW_SLOTS; ++u) sh.arrived[u] = 0;
+            int prev = -1;
+            for (int k = 0; k < K; ++k) {
+                sh.before[k] = prev;
+                sh.done[k] = 0;
+                if (sh.base[k + 1] > sh.base[k]) prev = k;
+            }
+            for (int k = 0; k < K && sh.before[k] < 0; ++k) sh.before[k] = -1 - prev;
+            sh.decided = -1;
+            sh.stop = (nc == 0) ? 0 : -1;
+            sh.dead = 0;
+            sh.ravg = sh.resid = 0.0;
+            sh.converged = (nc == 0);
+        }
+    }
+    // tagged records (tag 0), cleared block sums
+    for (int i = tid; i < nbody; i += stride) {
+        if (i >= g.n && !cd_is_body(g, i)) continue;
+        Body x;
+        T4 o;
+        o.x = o.y = o.z = o.w = (T)0;
+        if constexpr (DIM == 3) o = V[RW * i + 1];
+        x.pack(V[RW * i], o, 0u);
+        x.store(VT + (size_t)EB * i);
+    }
+    for (int i = tid; i < FLOW_ROWS * nb; i += stride) flow_sum_store(part + i, 0.0, 0u);
+    __syncthreads();
+    const int Q = sh.base[K];
+    const bool res = sh.slot[K] <= rec_cap;   // the block's records fit its shared memory
+    Records rec(s_rec, rec_cap);
+    // the colours each body has
+    for (int k = 0; k < K; ++k)
+        for (int p = sh.lo[k] + (int)threadIdx.x; p < sh.end[k]; p += blockDim.x) {
+            const int2 ab = w.c_ab[p];
+            atomicOr(&w.fl_mask[ab.x], 1ULL << k);
+            if (cd_is_body(g, ab.y)) atomicOr(&w.fl_mask[ab.y], 1ULL << k);
+        }
+    if (!cd_grid_sync(ctrl, nb, epoch)) return;
+    // a contact's place among each body's contacts and their number (8 bits
+    // each), and the resident records
+    for (int k = 0; k < K; ++k)
+        for (int p = sh.lo[k] + (int)threadIdx.x; p < sh.end[k]; p += blockDim.x) {
+            Rec<DIM, T> r;
+            r.ab = w.c_ab[p];
+            const u64 below = (1ULL << k) - 1ULL;
+            const u64 ma = w.fl_mask[r.ab.x], mb = cd_is_body(g, r.ab.y) ? w.fl_mask[r.ab.y] : 0ULL;
+            const unsigned ord = (unsigned)__popcll(ma & below) | ((unsigned)__popcll(ma) << 8) |
+                                 ((unsigned)__popcll(mb & below) << 16) | ((unsigned)__popcll(mb) << 24);
+            if (res) {
+                const int i = sh.slot[k] + p - sh.lo[k];
+                load_static<DIM, T>(g, w, r);
+                T2 t;
+                t.x = r.sa.x; t.y = r.sa.y; rec.s0[i] = t;
+                t.x = r.sa.z; t.y = r.sb.x; rec.s1[i] = t;
+                t.x = r.sb.y; t.y = r.sb.z; rec.s2[i] = t;
+                rec.geo[i] = ((const T4*)w.c_geo)[p];
+                rec.m[i] = ((const TM*)w.c_m)[p];
+                rec.P[i] = ((const TP*)w.c_P)[p];
+                rec.ab[i] = r.ab;
+                rec.ord[i] = ord;
+            } else {
+                w.fl_ord[p] = ord;
+            }
+        }
+    __syncthreads();
+
+    int last = 0;   // last pass this warp has run
+    // FP32 with more items than warps: wait for the block's own colour before
+    // looking.  The looks that find nothing fill the L1's request queue and hold
+    // up everything else there (100,000 discs: 15.4 -> 10.9 us a sweep).  FP64
+    // items take longer than that and gain from starting early (gated: 18.7 ->
+    // 21.3 us), and with one item a warp there is no queue.
+    const bool gate = sizeof(T) == 4 && Q > FLOW_WORKERS;
+    if (nc > 0 && wid == FLOW_WORKERS) {
+        double xprev = 0.0;
+        for (int pass = 0; ; ++pass) {
+            if (!flow_control(ctrl, sh, part, pass, nb, nc, crit, alpha, max_sweeps, xprev)) {
+                *(volatile int*)&sh.dead = 1;
+                break;
+            }
+            __syncwarp();
+            if (flow_ld(&sh.stop) >= 0) break;
+        }
+    } else if (nc > 0) {
+        TP pend;   // impulse of the warp's last update whose magnitude is not summed yet
+        for (int pass = 0; ; ++pass) {   // pass 0: the starting impulses; pass s: sweep s
+            const bool apply_only = (pass == 0);
+            const int known = pass - 1 - (pass >= FLOW_LAG1) - (pass >= FLOW_LAG2);
+            bool on = known < 0 || flow_wait_shared(ctrl, sh, &sh.decided, known);
+            on = on && pass <= max_sweeps && !flow_ld(&sh.dead);
+            // (a stop after `known` is not looked at: every warp of the grid runs the same passes)
+            if (on) {
+                const int st = flow_ld(&sh.stop);
+                on = !(st >= 0 && st <= known);
+            }
+            if (!__all_sync(0xffffffffu, on)) break;
+            last = pass;
+            // the impulses after pass s are in array s % 3
+            const TP* Pin = (const TP*)flow_impulses(w, apply_only ? 0 : pass - 1);
+            TP* Pout = (TP*)flow_impulses(w, pass);
+            const bool save = pass >= FLOW_LAG1;
+            T4* Vsave = Vprev + (size_t)(pass & 1) * RW * (g.n + 6);
+            double acc = 0.0;
+            bool owed = false;
+            bool dead = false;
+            int k = 0;
+            auto settle = [&]() {   // the magnitude owed
+                if constexpr (DEFER) {
+                    if (owed) {
+                        if constexpr (F64_2D) acc += abs_of_pair(pend.x, pend.y);
+                        else if constexpr (DIM == 2) acc += abs_of_sq<T>((double)fma_of<T>(pend.y, pend.y, mul_of<T>(pend.x, pend.x)));
+                        else acc += abs_of_sq<T>((double)fma_of<T>(pend.w, pend.w, fma_of<T>(pend.z, pend.z, fma_of<T>(pend.y, pend.y, mul_of<T>(pend.x, pend.x)))));
+                    }
+                    owed = false;
+                }
+            };
+            for (int q = wid; q < Q; q += FLOW_WORKERS) {
+                while (q >= sh.base[k + 1]) ++k;
+                const int first = sh.lo[k], cnt = sh.end[k] - first;
+                const bool split = F64_2D && cnt <= FLOW_SPLIT;
+                const int at = split ? 16 * (q - sh.base[k]) + (lane >> 1) : 32 * (q - sh.base[k]) + lane;
+                const bool act = at < cnt;
+                const int p = first + at, i = sh.slot[k] + at;
+                Rec<DIM, T> r;
+                u64 *pa = nullptr, *pb = nullptr;
+                unsigned ta = 0, tb = 0, ord = 0;
+                bool wall = true;
+                Body A, B;
+                if (act) {
+                    if (res) {
+                        r.ab = rec.ab[i];
+                        ord = rec.ord[i];
+                    } else {
+                        r.ab = w.c_ab[p];
+                        ord = w.fl_ord[p];
+                    }
+                    wall = !cd_is_body(g, r.ab.y);
+                    ta = (unsigned)pass * ((ord >> 8) & 255u) + (ord & 255u);
+                    tb = (unsigned)pass * (ord >> 24) + ((ord >> 16) & 255u);
+                    pa = VT + (size_t)EB * r.ab.x;
+                    if (!wall) pb = VT + (size_t)EB * r.ab.y;
+                    if (!gate) {
+                        A.load(pa);
+                        if (!wall) B.load(pb);
+                    }
+                    // the rest of the record while the velocities are on their way
+                    TM m;
+                    if (res) {
+                        const T2 t0 = rec.s0[i], t1 = rec.s1[i], t2 = rec.s2[i];
+                        r.sa.x = t0.x; r.sa.y = t0.y; r.sa.z = t1.x; r.sa.w = (T)0;
+                        r.sb.x = t1.y; r.sb.y = t2.x; r.sb.z = t2.y; r.sb.w = (T)0;
+                        r.geo = rec.geo[i];
+                        m = rec.m[i];
+                        r.P = rec.P[i];
+                    } else {
+                        load_static<DIM, T>(g, w, r);
+                        r.geo = ((const T4*)w.c_geo)[p];
+                        m = ((const TM*)w.c_m)[p];
+                        r.P = Pin[p];
+                    }
+                    if constexpr (DIM == 2) r.mt = m;
+                    else r.m = m;
+                    r.pk = 0;
+                    r.mu = (T)g.mu;
+                }
+                FlowHalf half;
+                if constexpr (F64_2D) {
+                    if (split) {
+                        if (!act) {
+                            r.geo.x = r.geo.y = r.geo.z = r.geo.w = 0.0;
+                            r.sa = r.sb = r.geo;
+                            r.P.x = r.P.y = r.mt = r.mu = 0.0;
+                        }
+                        half.choose(lane & 1, r);
+                    }
+                }
+                settle();
+                if (gate) {
+                    // not before the block's items of the colour before are done: the records are
+                    // hardly there earlier, and looks that find nothing delay every other access
+                    const int kb = sh.before[k] >= 0 ? sh.before[k] : -1 - sh.before[k];
+                    const int need = (sh.base[kb + 1] - sh.base[kb]) * (pass + (sh.before[k] >= 0));
+                    if (!__all_sync(0xffffffffu, flow_wait_shared(ctrl, sh, &sh.done[kb], need))) { dead = true; break; }
+                    if (pa) A.load(pa);
+                    if (pb) B.load(pb);
+                }
+                if (!flow_wait<DIM, T>(ctrl, sh, pa, ta, pb, tb, A, B)) { dead = true; break; }
+                T4 va, oa, vb, ob;
+                if constexpr (F64_2D) {
+                    if (split) {
+                        const bool odd = lane & 1;
+                        if (act) {
+                            A.unpack(va, oa);
+                            if (!wall) B.unpack(vb, ob);
+                            else wall_vel2<T>(g, w, r.ab.y, vb);
+                        } else {
+                            va.x = va.y = va.z = 0.0;
+                            vb = va;
+                        }
+                        T4 v1;
+                        const double Pnew = half.update(odd, r, va, vb, wall ? -1 : r.ab.y - g.n, apply_only, v1);
+                        if (act && !(odd && wall)) {
+                            A.pack(v1, v1, (odd ? tb : ta) + 1u);
+                            A.store(odd ? pb : pa);
+                        }
+                        if (act) {
+                            if (!apply_only) {
+                                reinterpret_cast<double*>(Pout + p)[odd] = Pnew;
+                                if (res) reinterpret_cast<double*>(rec.P + i)[odd] = Pnew;
+                            }
+                            // the records of the pass start, for taking the sweep back
+                            const int mine = odd ? (int)((ord >> 16) & 255u) : (int)(ord & 255u);
+                            if (save && mine == 0 && !(odd && wall)) Vsave[odd ? r.ab.y : r.ab.x] = odd ? vb : va;
+                        }
+                        const double Pother = shfl_pair(Pnew);
+                        pend.x = Pnew;
+                        pend.y = Pother;
+                        owed = act && !odd;
+                        __syncwarp();
+                        if (gate && lane == 0) atomicAdd(&sh.done[k], 1);
+                        continue;
+                    }
+                }
+                if (act) {
+                    A.unpack(va, oa);
+                    if (!wall) B.unpack(vb, ob);
+                    else if constexpr (DIM == 2) wall_vel2<T>(g, w, r.ab.y, vb);
+                    else wall_vel3<T>(g, w, r.ab.y, vb, ob);
+                    if (save) {
+                        if ((ord & 255u) == 0u) {
+                            Vsave[RW * r.ab.x] = va;
+                            if constexpr (DIM == 3) Vsave[RW * r.ab.x + 1] = oa;
+                        }
+                        if (!wall && ((ord >> 16) & 255u) == 0u) {
+                            Vsave[RW * r.ab.y] = vb;
+                            if constexpr (DIM == 3) Vsave[RW * r.ab.y + 1] = ob;
+                        }
+                    }
+                    TP Pn;
+                    UpdOut o;
+                    if constexpr (DIM == 2) {
+                        o = core2d<T, true>(g, r, va, vb, wall, apply_only, crit, alpha, 0.0, Pn);
+                        if (!wall && r.ab.y >= g.n) {
+                            if (((r.ab.y - g.n) >> 1) == 0) vb.y = (T)0; else vb.x = (T)0;
+                            vb.z = (T)0;
+                        }
+                    } else {
+                        o = core3d<T, DEFER>(g, r, va, oa, vb, ob, wall, apply_only, crit, alpha, 0.0, Pn);
+                        if (!wall && r.ab.y >= g.n) {
+                            const int ax = (r.ab.y - g.n) >> 1;
+                            if (ax != 0) vb.x = (T)0;
+                            if (ax != 1) vb.y = (T)0;
+                            if (ax != 2) vb.z = (T)0;
+                            ob.x = ob.y = ob.z = (T)0;
+                        }
+                    }
+                    A.pack(va, oa, ta + 1u);
+                    A.store(pa);
+                    if (!wall) {
+                        B.pack(vb, ob, tb + 1u);
+                        B.store(pb);
+                    }
+                    if (!apply_only) {
+                        Pout[p] = Pn;
+                        if (res) rec.P[i] = Pn;
+                    }
+                    if constexpr (DEFER) {
+                        pend = Pn;
+                        owed = true;
+                    } else {
+                        acc += o.pabs;
+                    }
+                }
+                if (gate) {
+                    __syncwarp();
+                    if (lane == 0) atomicAdd(&sh.done[k], 1);
+                }
+            }
+            if (dead) break;
+            settle();
+            *(volatile double*)&sh.acc[pass % FLOW_SLOTS][wid][lane] = acc;
+            __syncwarp();
+            if (lane == 0) {
+                __threadfence_block();
+                atomicAdd(&sh.arrived[pass % FLOW_SLOTS], 1);
+            }
+        }
+    }
+    __syncthreads();
+    if (sh.dead) return;
+    const int sweeps = sh.stop;
+    // final impulses of this block's contacts in c_P
+    if (sweeps % 3) {
+        const TP* P = (const TP*)flow_impulses(w, sweeps);
+        for (int k = 0; k < K; ++k)
+            for (int p = sh.lo[k] + (int)threadIdx.x; p < sh.end[k]; p += blockDim.x)
+                ((TP*)w.c_P)[p] = P[p];
+    }
+    // sweeps past the last: the velocities from before them
+    const bool back = __syncthreads_or(last > sweeps);
+    if (!cd_grid_sync(ctrl, nb, epoch)) return;
+    for (int i = tid; i < nbody; i += stride) {
+        if (i >= g.n && !cd_is_body(g, i)) continue;
+        T4 v, o;
+        if (back && w.fl_mask[i] != 0ULL) {
+            const T4* Vsave = Vprev + (size_t)((sweeps + 1) & 1) * RW * (g.n + 6);
+            v = Vsave[RW * i];
+            v.w = (T)0;
+            if constexpr (DIM == 3) o = Vsave[RW * i + 1];
+        } else {
+            Body x;
+            x.load(VT + (size_t)EB * i);
+            x.unpack(v, o);
+        }
+        V[RW * i] = v;
+        if constexpr (DIM == 3) V[RW * i + 1] = o;
+    }
+    finish_solve<DIM, T>(g, w, nc, nb, tid, stride, epoch, sweeps, sh.converged, sh.resid, sh.ravg, s_red, s_bc);
+}
+
+struct FlowKernel { const void* fn; int body_bytes, record_bytes; };
+static FlowKernel flow_kernel(int dim, int precision)
+{
+#define FLOW_K(D, T) FlowKernel{(const void*)k_flow<D, T>, (int)sizeof(FlowBody<D, T>), FlowRecords<D, T>::BYTES}
+    if (dim == 2) return precision == CD_FP64 ? FLOW_K(2, double) : FLOW_K(2, float);
+    return precision == CD_FP64 ? FLOW_K(3, double) : FLOW_K(3, float);
+#undef FLOW_K
+}
+
+size_t cd_flow_body_bytes(int dim, int precision) { return (size_t)flow_kernel(dim, precision).body_bytes; }
+
+// Contacts a block keeps in shared memory (a multiple of 16, so that every
+// array of the records stays aligned), or -1 if the kernel does not fit.
+int cd_flow_records(int dim, int precision, int device)
+{
+    const FlowKernel f = flow_kernel(dim, precision);
+    int most = 0;
+    cudaFuncAttributes a;
+    if (cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
+        cudaFuncGetAttributes(&a, f.fn) != cudaSuccess)
+        return -1;
+    const int room = most - (int)a.sharedSizeBytes - 256;
+    const int recs = room > 0 ? room / f.record_bytes / 16 * 16 : 0;
+    if (cudaFuncSetAttribute(f.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, recs * f.record_bytes) != cudaSuccess)
+        return -1;
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, f.fn, FLOW_THREADS, (size_t)(recs * f.record_bytes)) !=
+            cudaSuccess || b < 1)
+        return -1;
+    return recs;
+}
+
+cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int criterion,
+                           double alpha, int max_sweeps, cudaStream_t s, int* nl)
+{
+    cudaError_t e = cudaMemsetAsync(w.ctrl, 0, 2 * sizeof(u64), s);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(w.fl_mask, 0, sizeof(u64) * (size_t)(g.n + 6), s)) != cudaSuccess) return e;
+    const FlowKernel f = flow_kernel(g.dim, precision);
+    CdGeom ga = g;
+    CdWork wa = w;
+    int crit = criterion, ms = max_sweeps, rc = records;
+    double al = alpha;
+    void* args[] = {&ga, &wa, &crit, &al, &ms, &rc};
+    ++*nl;
+    return cudaLaunchCooperativeKernel(f.fn, dim3(blocks), dim3(FLOW_THREADS), args,
+                                       (size_t)(records * f.record_bytes), s);
+}

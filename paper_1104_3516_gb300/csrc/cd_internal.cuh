@@ -176,6 +176,14 @@ struct CdWork {
     int* mg_boff;       // CD_MG_MAXC G + 1: exclusive scan of mg_bcnt
     int* mg_bmin;       // CD_MG_MAXC G: lowest position of the bucket
     int* mg_bmax;       // CD_MG_MAXC G: highest position of the bucket
+    // dataflow solve (cd_flow.cu)
+    void* fl_V;         // n + 6 tagged velocity records
+    unsigned long long* fl_mask; // n + 6: colours of each body's contacts
+    unsigned* fl_ord;   // cap (colour order): place of the contact among its bodies' contacts
+    void* fl_part;      // 4 G tagged block sums
+    void* fl_P;         // cap: impulses after the sweeps s with s % 3 = 1 (c_P: 0)
+    void* fl_P2;        // cap: ... = 2
+    void* fl_Vprev;     // 2 (n + 6) velocity records from before the latest two sweeps
     // repair of the highest colour (global colour order)
     int* rep_top;       // npk: highest colour of each packing
     int* rep_dmax;      // npk: most contacts of one body of the packing
@@ -276,6 +284,7 @@ struct CdGeom {
     int merge_last;     // params.merge_last_colour (0 off, 2: at most two colours, 3: three, else two)
     int merge_auto;     // merge only after a solve of at least CD_MG_MIN_SWEEPS sweeps (or none yet)
     int merge_blocks;   // blocks of the sweep grid the chains are assigned to
+    int flow;           // 1: the solve runs as a dataflow (cd_flow.cu)
 };
 
 // Velocity records of the domain views start after the particles' and the
@@ -475,6 +484,10 @@ cudaError_t cd_launch_stress(const CdGeom& g, const CdWork& w, const double* pos
                              double lo, double width, int ns, double* sig, cudaStream_t stream, int* nl);
 cudaError_t cd_launch_sweep(const CdGeom& g, const CdWork& w, int coop_blocks, int threads, int precision,
                             int criterion, double alpha, int max_sweeps, int pw, cudaStream_t stream, int* nl);
+cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int criterion,
+                           double alpha, int max_sweeps, cudaStream_t stream, int* nl);
+size_t cd_flow_body_bytes(int dim, int precision);
+int cd_flow_records(int dim, int precision, int device);
 int cd_sweep_fits(const CdGeom& g, int precision, int threads, int per_sm);
 cudaError_t cd_launch_unpack(const CdGeom& g, const CdWork& w, double* pos, double* vel, double* omega,
                              double* theta, int integrate, int precision, cudaStream_t stream, int* nl);

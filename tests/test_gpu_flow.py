@@ -1,0 +1,76 @@
+"""The dataflow solve (plain systems whose sweep cap exceeds 128, without an
+asked-for merge) against the barrier schedule on the same system: the order of
+the updates is the same, so impulses, velocities and positions are bit-equal,
+and the stopping sweep is the same (a solve that stops after sweeps that were
+started before their test was known takes them back).  merge_last_colour = 1
+keeps the barrier schedule."""
+import numpy as np
+import pytest
+
+from gpu_common import gpu_system, needs_gpu
+from paper_1104_3516_gb300 import workloads as W
+
+pytestmark = [pytest.mark.gpu, needs_gpu]
+
+
+def both(wl, steps=2, **kw):
+    a = gpu_system(wl, merge_last_colour=1, **kw)
+    b = gpu_system(wl, merge_last_colour=4, **kw)
+    sa = [a.step(1) for _ in range(steps)]
+    sb = [b.step(1) for _ in range(steps)]
+    for x, y in zip(sa, sb):
+        for k in ("sweeps", "converged", "n_contacts", "n_colours"):
+            assert x["last"][k] == y["last"][k], k
+        # the sums of |P| over the contacts differ in their order only
+        assert abs(x["last"]["r_avg"] - y["last"]["r_avg"]) <= 1e-13 * x["last"]["r_avg"]
+        assert np.allclose(x["last"]["wall_force"], y["last"]["wall_force"], rtol=1e-13, atol=0)
+        assert y["last"]["n_phases"] == y["last"]["n_colours"]
+    ca, cb = a.contacts(), b.contacts()
+    for k in ("pairs", "colour", "impulse"):
+        assert np.array_equal(ca[k], cb[k]), k
+    xa, xb = a.state(), b.state()
+    for k in ("x", "v", "w"):
+        assert np.array_equal(xa[k], xb[k]), k
+    return sb
+
+
+# discs per block of 152 from one lane pair (a few contacts a colour in some
+# blocks, none in others) over whole warps to several items a warp; 300,000
+# exceed what the blocks' shared memory holds
+@pytest.mark.parametrize("n", [3, 40, 700, 4999, 20011, 40000, 300000])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_pile_is_bit_identical(n, precision):
+    from paper_1104_3516_gb300 import cd
+    wl = W.dense_biaxial_discs(seed=5, n=n) if n > 3 else W.settling_discs(seed=5, n=3)
+    both(wl, steps=1 if n > 100000 else 2, criterion=cd.CD_CONV_NONE, max_sweeps=131, precision=precision,
+         max_contacts=4 * n + 64)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_spheres_are_bit_identical(precision):
+    from paper_1104_3516_gb300 import cd
+    for wl in (W.sphere_gas(n=3000, floor=20.0, vsig=0.5), W.sphere_gas(seed=3, n=20011, floor=40.0, vsig=0.5)):
+        both(wl, criterion=cd.CD_CONV_NONE, max_sweeps=131, precision=precision)
+
+
+# thresholds whose stopping sweep falls before, at and after the sweeps from
+# which on one and two sweeps are started ahead of their test
+@pytest.mark.parametrize("criterion", [0, 1])
+@pytest.mark.parametrize("alpha", [1e-1, 3e-2, 1e-2, 5e-3, 2e-3, 1e-3, 3e-4, 1e-4])
+def test_stops_at_the_same_sweep(alpha, criterion):
+    wl = W.dense_biaxial_discs(seed=9, n=2000)
+    sb = both(wl, steps=3, criterion=criterion, alpha=alpha if criterion == 0 else alpha * alpha, max_sweeps=5000)
+    assert sb[0]["last"]["converged"]
+
+
+def test_cap_reached_and_few_contacts():
+    wl = W.dense_biaxial_discs(seed=2, n=1000)
+    sb = both(wl, criterion=0, alpha=0.0, max_sweeps=129)
+    assert sb[0]["last"]["sweeps"] == 129 and not sb[0]["last"]["converged"]
+    both(W.dilute_discs(seed=4, n=200, width=20.0), steps=4)   # a handful of contacts, most colours empty in most blocks
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_force_controlled_lid_is_bit_identical(precision):
+    """The lid is a body of many colours (its contacts conflict)."""
+    both(W.pressure_column(seed=6, n=600), steps=3, precision=precision)
