@@ -17,9 +17,7 @@
 // histograms, one exclusive scan, a rank within the chunk from warp match
 // masks), then the contact data is gathered into colour order in the sweep's
 // real type.
-#include <type_traits>
-
-#include "cd_internal.cuh"
+#include "cd_colour_core.cuh"
 
 __global__ void k_p2c_count(CdGeom g, CdWork w)
 {
@@ -67,200 +65,15 @@ __global__ void k_p2c_sort(CdGeom g, CdWork w)
     }
 }
 
-// Persistent cooperative kernel: Jones-Plassmann rounds separated by the
-// bounded grid barrier.  `prio` scratch lives in the chunk buffer (8 bytes per
-// contact is reserved there by the workspace layout).
-//
-// Worklist form: every contact first counts its neighbours of higher
-// priority (contacts sharing a body); those with
-// none start the first list.  A round colours the contacts of its list (the
-// smallest colour no higher-priority neighbour has; all of those are
-// coloured by then) and decrements the counts of their lower-priority
-// neighbours; a contact whose count reaches zero joins the next list.  Each
-// contact is coloured exactly once, from the same neighbours as in the
-// round-by-round scan, so the colouring is the same greedy fixed point, at a
-// cost proportional to the contacts and their neighbours instead of to
-// rounds x contacts.  Scratch: the colour repair's arrays (used only after
-// the colouring): rep_flag holds the counts, rep_list and rep_path the lists
-// of even and odd rounds; round_cnt[r % 3] is the length of round r's list
-// (three counters, so that one grid barrier per round suffices: round r
-// clears the counter of round r + 2, last read in round r - 1).
-__device__ __forceinline__ bool jp_higher(const CdWork& w, const unsigned long long* prio, int d, int c,
-                                          unsigned long long pc, unsigned long long kc)
-{
-    const unsigned long long pd = prio[d];
-    if (pd != pc) return pd > pc;
-    const int2 dd = w.pairs[d];
-    return cd_key(dd.x, dd.y) < kc;
-}
-
-// Appends c to list (length at *len) with one atomic per warp.
-__device__ __forceinline__ void jp_append(int* list, int* len, int c, bool take)
-{
-    const unsigned m = __ballot_sync(0xffffffffu, take);
-    if (!m) return;
-    const int lane = threadIdx.x & 31;
-    int base = 0;
-    if (lane == __ffs(m) - 1) base = atomicAdd(len, __popc(m));
-    base = __shfl_sync(0xffffffffu, base, __ffs(m) - 1);
-    if (take) list[base + __popc(m & ((1u << lane) - 1u))] = c;
-}
-
-// Appends each lane's up to four entries c[u] (take[u]) with one atomic per
-// warp: the lane's offset is the exclusive prefix sum of the lanes' counts.
-__device__ __forceinline__ void jp_append4(int* list, int* len, const int (&c)[4], const bool (&take)[4])
-{
-    const int lane = threadIdx.x & 31;
-    int k = 0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) k += take[u] ? 1 : 0;
-    int incl = k;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    if (total == 0) return;
-    int base = 0;
-    if (lane == 31) base = atomicAdd(len, total);
-    base = __shfl_sync(0xffffffffu, base, 31) + incl - k;
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-        if (take[u]) list[base++] = c[u];
-}
-
-__global__ void __launch_bounds__(CD_SWEEP_THREADS) k_jp(CdGeom g, CdWork w, unsigned long long* prio,
-                                                          int* round_cnt)
+// Persistent cooperative kernel.
+__global__ void __launch_bounds__(CD_SWEEP_THREADS) k_jp(CdGeom g, CdWork w, unsigned long long* prio)
 {
     CdCtrl* ctrl = w.ctrl;
     if (ctrl->skip) return;
-    const int nc = ctrl->nc;
-    const unsigned long long nb = gridDim.x;
     unsigned long long epoch = 0;
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int stride = gridDim.x * blockDim.x;
-    int* cnt = w.rep_flag;
-    for (int c = tid; c < nc; c += stride) {
-        int2 ab = w.pairs[c];
-        unsigned long long h;
-        if (g.npk > 1) {
-            // a packing of a batch is coloured with its own seed and local
-            // ids (walls n_b + k), exactly as if it were a system alone
-            const CdPack& P = w.pk[w.pack_of[ab.x]];
-            const int al = ab.x - P.first;
-            const int bl = (ab.y < g.n) ? ab.y - P.first : P.count + (ab.y - g.n) % 6;
-            h = cd_splitmix64(P.seed ^ cd_key(al, bl));
-        } else {
-            h = cd_splitmix64(g.seed ^ cd_key(ab.x, ab.y));
-        }
-        // largest degree first (contacts of both ends, capped at 255), then the hash
-        unsigned long long ds = (unsigned long long)(w.p2c_off[ab.x + 1] - w.p2c_off[ab.x]);
-        if (cd_is_body(g, ab.y)) ds += (unsigned long long)(w.p2c_off[ab.y + 1] - w.p2c_off[ab.y]);
-        if (ds > 255ULL) ds = 255ULL;
-        prio[c] = (ds << 56) | (h >> 8);
-        w.colour[c] = -1;
-    }
-    if (tid == 0) { round_cnt[0] = 0; round_cnt[1] = 0; round_cnt[2] = 0; ctrl->ncolours = 0; }
-    if (!cd_grid_sync(ctrl, nb, epoch)) return;
-    // higher-priority neighbours of every contact; the free ones start the first list
-    for (int c0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); c0 < nc; c0 += stride) {
-        const int c = c0 + (threadIdx.x & 31);
-        int k = 0;
-        if (c < nc) {
-            const unsigned long long pc = prio[c];
-            const int2 ab = w.pairs[c];
-            const unsigned long long kc = cd_key(ab.x, ab.y);
-            for (int side = 0; side < 2; ++side) {
-                const int q = side ? ab.y : ab.x;
-                if (!cd_is_body(g, q)) continue;
-                const int f0 = w.p2c_off[q], f1 = w.p2c_off[q + 1];
-                for (int t = f0; t < f1; t += 4) {
-                    int d[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) d[u] = (t + u < f1) ? w.p2c[t + u] : -1;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (d[u] >= 0 && d[u] != c &&
-                            jp_higher(w, prio, d[u], c, pc, kc))
-                            ++k;
-                }
-            }
-            cnt[c] = k;
-        }
-        jp_append(w.rep_list, &round_cnt[0], c, c < nc && k == 0);   // round 0's list
-    }
-    if (!cd_grid_sync(ctrl, nb, epoch)) return;
-    for (int round = 0; round < (1 << 20); ++round) {
-        // even rounds read rep_list and fill rep_path, odd rounds the reverse
-        // (selected, not indexed: an indexed pair of pointers lives in local memory)
-        int* const list_cur = (round & 1) ? w.rep_path : w.rep_list;
-        int* const list_nxt = (round & 1) ? w.rep_list : w.rep_path;
-        const int len = cd_ld_volatile_int(&round_cnt[round % 3]);
-        if (len == 0) break;
-        if (tid == 0) round_cnt[(round + 2) % 3] = 0;
-        for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < len; i0 += stride) {
-            const int i = i0 + (threadIdx.x & 31);
-            const int c = (i < len) ? list_cur[i] : -1;
-            int2 ab = make_int2(0, 0);
-            unsigned long long pc = 0ULL, kc = 0ULL;
-            if (c >= 0) {
-                pc = prio[c];
-                ab = w.pairs[c];
-                kc = cd_key(ab.x, ab.y);
-            }
-            // one pass over both bodies' contacts: the colours of the higher-priority
-            // neighbours (all final), and the release of the lower-priority ones (they
-            // read c's colour only in a later round, after the grid barrier)
-            unsigned long long used = 0ULL;
-            for (int side = 0; side < 2; ++side) {
-                const int q = side ? ab.y : ab.x;
-                const bool on = c >= 0 && cd_is_body(g, q);
-                const int f0 = on ? w.p2c_off[q] : 0, f1 = on ? w.p2c_off[q + 1] : 0;
-                int most = f1 - f0;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
-                // four neighbours at a time: their loads and atomics are in flight together
-                for (int t = 0; t < most; t += 4) {
-                    int d[4], v[4];
-                    bool hi[4], lo[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) d[u] = (f0 + t + u < f1) ? w.p2c[f0 + t + u] : -1;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const bool nb_ok = d[u] >= 0 && d[u] != c;
-                        const bool h = nb_ok && jp_higher(w, prio, d[u], c, pc, kc);
-                        hi[u] = h;
-                        lo[u] = nb_ok && !h;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        v[u] = hi[u] ? cd_ld_volatile_int(&w.colour[d[u]]) : (lo[u] ? atomicSub(&cnt[d[u]], 1) : 0);
-                    bool rel[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        if (hi[u] && v[u] >= 0) used |= 1ULL << v[u];
-                        rel[u] = lo[u] && v[u] == 1;   // its last higher-priority neighbour: next round
-                    }
-                    jp_append4(list_nxt, &round_cnt[(round + 1) % 3], d, rel);
-                }
-            }
-            int top = 0;
-            if (c >= 0) {
-                const int col = (used == ~0ULL) ? 64 : __ffsll((long long)~used) - 1;
-                if (col >= CD_KMAX) {
-                    atomicCAS(&ctrl->error, CDE_NONE, CDE_COLOURS);
-                } else {
-                    *(volatile int*)&w.colour[c] = col;
-                    top = col + 1;
-                }
-            }
-            top = __reduce_max_sync(0xffffffffu, top);   // one atomic per warp
-            if ((threadIdx.x & 31) == 0 && top > 0) atomicMax(&ctrl->ncolours, top);
-        }
-        if (!cd_grid_sync(ctrl, nb, epoch)) return;
-        if (cd_ld_volatile_int(&ctrl->error) != CDE_NONE) break;
-    }
+    const unsigned long long nb = gridDim.x;
+    auto sync = [&]() { return cd_grid_sync(ctrl, nb, epoch); };
+    jp_colour(g, w, ctrl->nc, prio, sync);
 }
 
 // ---------------------------------------------------------------------------
@@ -343,110 +156,16 @@ __global__ void k_rep_fill(CdWork w)
         if (w.rep_flag[c]) w.rep_list[w.rep_pos[c]] = c;
 }
 
-// The repair runs one warp per packing: every step is sequential, but the
-// lanes read a body's contact list together, so a step costs a few L2 round
-// trips instead of one per contact of the body.  All lanes follow the same
-// control flow; lane 0 writes.
-
-// Colours below t that body x has on no contact other than c (all of them
-// for a wall that is not a body).
-__device__ __forceinline__ unsigned long long rep_free(const CdGeom& g, const CdWork& w, int x, int c, int t)
-{
-    const unsigned long long all = (1ULL << t) - 1ULL;
-    if (!cd_is_body(g, x)) return all;
-    const int lane = threadIdx.x & 31;
-    const int f0 = w.p2c_off[x], f1 = w.p2c_off[x + 1];
-    unsigned long long used = 0ULL;
-    for (int f = f0; f < f1; f += 32) {
-        unsigned long long bit = 0ULL;
-        if (f + lane < f1) {
-            const int d = w.p2c[f + lane];
-            const int k = w.colour[d];
-            if (d != c && k >= 0 && k < t) bit = 1ULL << k;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) bit |= __shfl_xor_sync(0xffffffffu, bit, o);
-        used |= bit;
-    }
-    return all & ~used;
-}
-
-// Body x's contact of colour cur (at most one in a proper colouring), or -1.
-__device__ __forceinline__ int rep_find(const CdWork& w, int x, int cur)
-{
-    const int lane = threadIdx.x & 31;
-    const int f0 = w.p2c_off[x], f1 = w.p2c_off[x + 1];
-    for (int f = f0; f < f1; f += 32) {
-        int d = -1;
-        if (f + lane < f1) {
-            const int dd = w.p2c[f + lane];
-            if (w.colour[dd] == cur) d = dd;
-        }
-        const unsigned hit = __ballot_sync(0xffffffffu, d >= 0);
-        if (hit) return __shfl_sync(0xffffffffu, d, __ffs(hit) - 1);
-    }
-    return -1;
-}
-
+// One warp per packing.
 __global__ void k_rep_run(CdGeom g, CdWork w)
 {
     if (w.ctrl->skip || w.ctrl->error != CDE_NONE) return;   // e.g. an uncoloured contact
     const int nc = w.ctrl->nc;
-    const int lane = threadIdx.x & 31;
-    const int b = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);   // one warp per packing
+    const int b = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (b >= g.npk) return;
     const int c0 = (g.npk > 1) ? w.pk_coff[b] : 0, c1 = (g.npk > 1) ? w.pk_coff[b + 1] : nc;
-    const int ncb = c1 - c0, t = w.rep_top[b];
-    if (ncb <= 0 || t <= 0 || t > 63 || t + 1 <= w.rep_dmax[b]) return;
-    const int l0 = w.rep_pos[c0], l1 = w.rep_pos[c1];
-    int limit = ncb / 256;
-    if (limit > 1024) limit = 1024;
-    if (limit < 1) limit = 1;
-    if (l1 - l0 > limit) return;
-    int* path = w.rep_path + c0;
-    for (int l = l0; l < l1; ++l) {
-        const int c = w.rep_list[l];
-        const int2 uv = w.pairs[c];
-        const int u = uv.x, v = uv.y;
-        const unsigned long long mu = rep_free(g, w, u, c, t), mv = rep_free(g, w, v, c, t);
-        if (mu & mv) {
-            if (lane == 0) w.colour[c] = __ffsll((long long)(mu & mv)) - 1;
-            __syncwarp();
-            continue;
-        }
-        if (!cd_is_body(g, v)) continue;
-        bool done = false;
-        for (int a = 0; a < t && !done; ++a) {
-            if (!((mu >> a) & 1ULL)) continue;
-            for (int bb = 0; bb < t && !done; ++bb) {
-                if (!((mv >> bb) & 1ULL)) continue;
-                int len = 0, x = v, cur = a;
-                bool fail = false;
-                for (;;) {
-                    const int e = rep_find(w, x, cur);
-                    if (e < 0) break;
-                    const int2 pe = w.pairs[e];
-                    const int y = (pe.x == x) ? pe.y : pe.x;
-                    if (lane == 0) path[len] = e;
-                    ++len;
-                    if (y == u) { fail = true; break; }
-                    if (!cd_is_body(g, y)) break;
-                    x = y;
-                    cur = (cur == a) ? bb : a;
-                    if (len >= ncb) { fail = true; break; }
-                }
-                __syncwarp();
-                if (fail) continue;
-                for (int i = lane; i < len; i += 32) {
-                    const int e = path[i];
-                    w.colour[e] = (w.colour[e] == a) ? bb : a;
-                }
-                if (lane == 0) w.colour[c] = a;
-                __syncwarp();
-                done = true;
-            }
-        }
-    }
+    const int t = w.rep_top[b], l0 = w.rep_pos[c0], l1 = w.rep_pos[c1];
+    if (rep_wanted(c1 - c0, t, w.rep_dmax[b], l1 - l0)) rep_run(g, w, t, l0, l1, c1 - c0, w.rep_path + c0);
 }
 
 __global__ void k_rep_ncolours_reset(CdCtrl* ctrl)
@@ -536,44 +255,7 @@ __global__ void k_colour_scatter(CdGeom g, CdWork w, int pw)
     if (c >= nc || k < 0) return;
     for (int v = 0; v < wid; ++v) rank += s_wcnt[v][k];
     int pos = w.chunk_cnt[k * ncl + blockIdx.x] + rank;
-    w.perm[pos] = c;
-    int2 ab = w.pairs[c];
-    w.c_ab[pos] = ab;
-    double b = __ddiv_rn(w.gap[c], g.dt);
-    if (DIM == 2) {
-        typedef typename std::conditional<sizeof(T) == 8, double4_32a, float4>::type T4;
-        typedef typename std::conditional<sizeof(T) == 8, double2, float2>::type T2;
-        T4 geo;
-        geo.x = (T)w.nrm[3 * c];
-        geo.y = (T)w.nrm[3 * c + 1];
-        geo.z = (T)b;
-        geo.w = (T)w.mn[c];
-        ((T4*)w.c_geo)[pos] = geo;
-        ((T*)w.c_m)[pos] = (T)w.mt[c];
-        T2 P;
-        P.x = (T)w.Pk[2 * c];
-        P.y = (T)w.Pk[2 * c + 1];
-        ((T2*)w.c_P)[pos] = P;
-    } else {
-        typedef typename std::conditional<sizeof(T) == 8, double4_32a, float4>::type T4;
-        typedef typename std::conditional<sizeof(T) == 8, double2, float2>::type T2;
-        T4 geo;
-        geo.x = (T)w.nrm[3 * c];
-        geo.y = (T)w.nrm[3 * c + 1];
-        geo.z = (T)w.nrm[3 * c + 2];
-        geo.w = (T)b;
-        ((T4*)w.c_geo)[pos] = geo;
-        T2 m;
-        m.x = (T)w.mn[c];
-        m.y = (T)w.mt[c];
-        ((T2*)w.c_m)[pos] = m;
-        T4 P;
-        P.x = (T)w.Pk[4 * c];
-        P.y = (T)w.Pk[4 * c + 1];
-        P.z = (T)w.Pk[4 * c + 2];
-        P.w = (T)w.Pk[4 * c + 3];
-        ((T4*)w.c_P)[pos] = P;
-    }
+    colour_record<DIM, T>(g, w, c, pos);
 }
 
 __global__ void k_colour_offsets(CdWork w)
@@ -655,8 +337,7 @@ cudaError_t cd_launch_colour(const CdGeom& g, const CdWork& w, int coop_blocks, 
         CdGeom ga = g;
         CdWork wa = w;
         unsigned long long* prio = w.prio;
-        int* rc = w.round_cnt;
-        void* args[] = {&ga, &wa, &prio, &rc};
+        void* args[] = {&ga, &wa, &prio};
         if ((e = cudaMemsetAsync(w.ctrl, 0, 2 * sizeof(unsigned long long), s)) != cudaSuccess) return e;
         e = cudaLaunchCooperativeKernel((const void*)k_jp, dim3(coop_blocks), dim3(CD_SWEEP_THREADS), args, 0, s);
         if (e != cudaSuccess) return e;
