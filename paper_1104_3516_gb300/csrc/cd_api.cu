@@ -28,6 +28,7 @@ struct cd_system {
     int sweep_blocks;
     int sweep_threads;
     int colour_blocks;
+    CdPrepPlan prep = {0, 0};          // one-kernel preparation (no blocks: separate kernels)
     int flow_records;                  // contacts a block of the dataflow solve keeps in shared memory
     int has_contacts;
     size_t ws_bytes;
@@ -199,6 +200,8 @@ static size_t layout(cd_system* s, char* base, CdWork* w)
         t.mg_bmin = L.take<int>(base, mg ? nbk : 1);
         t.mg_bmax = L.take<int>(base, mg ? nbk : 1);
     }
+    t.prep_tot = L.take<int>(base, s->prep.blocks ? 4 * CD_PREP_MAX_BLOCKS : 1);
+    t.prep_hist = L.take<int>(base, s->prep.blocks ? CD_KMAX * CD_PREP_MAX_BLOCKS : 1);
     {
         const bool fl = s->g.flow != 0;
         t.fl_V = L.take<char>(base, fl ? (n + 6) * cd_flow_body_bytes((int)s->p.dim, (int)s->p.precision) : 1);
@@ -324,18 +327,9 @@ static cd_status need_ready(cd_system* s)
     return CD_OK;
 }
 
-static cd_status launch_detect_chain(cd_system* s, int timed)
+// What follows the colour order: domains, merging.
+static cd_status launch_after_colour(cd_system* s)
 {
-    cd_status st;
-    CD_CUDA(s, cd_launch_detect(s->g, s->w, s->pos, s->radius, s->inv_m, s->inv_I, (int)s->p.warm_start, s->pw,
-                                s->stream, &s->launches));
-    if (s->g.npk > 1) CD_CUDA(s, cd_launch_pk_ranges(s->g, s->w, s->stream, &s->launches));
-    if (timed && (st = mark(s)) != CD_OK) return st;
-    CD_CUDA(s, cd_launch_colour(s->g, s->w, s->colour_blocks, (int)s->p.precision, s->pw, s->stream, &s->launches,
-                                s->pos));
-    k_error_gate<<<1, 1, 0, s->stream>>>(s->w.ctrl);
-    ++s->launches;
-    CD_CUDA(s, cudaGetLastError());
     if (s->g.ndom_total > 1)
         CD_CUDA(s, cd_launch_domains(s->g, s->w, s->pos, s->radius, s->stream, &s->launches));
     if (s->g.merge_last) {
@@ -351,12 +345,43 @@ static cd_status launch_detect_chain(cd_system* s, int timed)
     return CD_OK;
 }
 
+// pack: the velocities are packed as well (with the free flight) where one
+// kernel prepares the step.
+static cd_status launch_detect_chain(cd_system* s, int timed, int pack)
+{
+    cd_status st;
+    if (s->prep.blocks) {
+        CdPrepIO io = {};
+        io.pos = s->pos; io.radius = s->radius; io.inv_m = s->inv_m; io.inv_I = s->inv_I;
+        io.vel = s->vel; io.omega = s->omega; io.f_ext = s->f_ext;
+        io.warm = (int)s->p.warm_start;
+        io.pw = s->pw;
+        io.pack = pack;
+        io.free_flight = 1;
+        CD_CUDA(s, cd_launch_prepare(s->g, s->w, io, s->prep.blocks, s->prep.cluster, (int)s->p.precision, s->stream,
+                                     &s->launches));
+        return launch_after_colour(s);
+    }
+    CD_CUDA(s, cd_launch_detect(s->g, s->w, s->pos, s->radius, s->inv_m, s->inv_I, (int)s->p.warm_start, s->pw,
+                                s->stream, &s->launches));
+    if (s->g.npk > 1) CD_CUDA(s, cd_launch_pk_ranges(s->g, s->w, s->stream, &s->launches));
+    if (timed && (st = mark(s)) != CD_OK) return st;
+    CD_CUDA(s, cd_launch_colour(s->g, s->w, s->colour_blocks, (int)s->p.precision, s->pw, s->stream, &s->launches,
+                                s->pos));
+    k_error_gate<<<1, 1, 0, s->stream>>>(s->w.ctrl);
+    ++s->launches;
+    CD_CUDA(s, cudaGetLastError());
+    return launch_after_colour(s);
+}
+
 static cd_status launch_solve(cd_system* s, int free_flight, int timed)
 {
     cd_status st;
     s->mg_hint_valid = false;   // this solve's sweeps are unknown to the host until read back
-    CD_CUDA(s, cd_launch_pack(s->g, s->w, s->vel, s->omega, s->radius, s->inv_m, s->inv_I, s->f_ext, free_flight,
-                              (int)s->p.precision, s->stream, &s->launches));
+    // (a step's velocities are packed by the one-kernel preparation)
+    if (!(free_flight && s->prep.blocks))
+        CD_CUDA(s, cd_launch_pack(s->g, s->w, s->vel, s->omega, s->radius, s->inv_m, s->inv_I, s->f_ext, free_flight,
+                                  (int)s->p.precision, s->stream, &s->launches));
     if (timed && (st = mark(s)) != CD_OK) return st;
     if (s->g.flow) {
         CD_CUDA(s, cd_launch_flow(s->g, s->w, s->num_sms, s->flow_records, (int)s->p.precision, (int)s->p.criterion, s->p.alpha,
@@ -681,6 +706,9 @@ static cd_status create_impl(const cd_params* params, int64_t npk, const int64_t
         delete s;
         return fail(nullptr, CD_ERR_INVALID_ARG, "that many sweep blocks do not fit on one SM");
     }
+    // one-kernel preparation of small plain systems (with timing the phases are
+    // launched, and timed, one by one)
+    if (npk == 1 && !p.timing && n <= CD_PREP_MAX_N) s->prep = cd_prepare_plan((int)p.dim, (int)p.precision, n, s->device);
     *out = s;
     return CD_OK;
 }
@@ -752,7 +780,7 @@ extern "C" cd_status cd_detect_contacts(cd_system* s, int64_t* n_contacts)
     cd_status st = need_ready(s);
     if (st != CD_OK) return st;
     k_begin_call<<<1, 1, 0, s->stream>>>(s->w.ctrl, 0);
-    if ((st = launch_detect_chain(s, 0)) != CD_OK) return st;
+    if ((st = launch_detect_chain(s, 0, 0)) != CD_OK) return st;
     CdCtrl h;
     if ((st = read_ctrl(s, &h)) != CD_OK) return st;
     if (n_contacts) *n_contacts = h.overflow ? h.nc_needed : h.nc;
@@ -807,7 +835,7 @@ static cd_status launch_step(cd_system* s, int timed)
 {
     cd_status st;
     if (timed && (st = mark(s)) != CD_OK) return st;
-    if ((st = launch_detect_chain(s, timed)) != CD_OK) return st;
+    if ((st = launch_detect_chain(s, timed, 1)) != CD_OK) return st;
     if ((st = launch_solve(s, 1, timed)) != CD_OK) return st;
     if (timed && (st = mark(s)) != CD_OK) return st;
     CD_CUDA(s, cd_launch_unpack(s->g, s->w, s->pos, s->vel, s->omega, s->theta, 1, (int)s->p.precision, s->stream,

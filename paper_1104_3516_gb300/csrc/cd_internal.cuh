@@ -176,6 +176,9 @@ struct CdWork {
     int* mg_boff;       // CD_MG_MAXC G + 1: exclusive scan of mg_bcnt
     int* mg_bmin;       // CD_MG_MAXC G: lowest position of the bucket
     int* mg_bmax;       // CD_MG_MAXC G: highest position of the bucket
+    // one-kernel preparation of small systems (cd_prepare.cu)
+    int* prep_tot;      // 4 values per block
+    int* prep_hist;     // CD_KMAX x blocks: contacts of each colour in each block's range
     // dataflow solve (cd_flow.cu)
     void* fl_V;         // n + 6 tagged velocity records
     unsigned long long* fl_mask; // n + 6: colours of each body's contacts
@@ -451,6 +454,28 @@ cudaError_t cd_launch_set_contacts(const CdGeom& g, const CdWork& w, const doubl
                                    const double* impulses, int pw, cudaStream_t stream, int* nl);
 cudaError_t cd_launch_colour(const CdGeom& g, const CdWork& w, int coop_blocks, int precision, int pw,
                              cudaStream_t stream, int* nl, const double* pos);
+// What the one-kernel preparation reads (cd_prepare.cu).
+struct CdPrepIO {
+    const double* pos;
+    const double* radius;
+    const double* inv_m;
+    const double* inv_I;
+    const double* vel;
+    const double* omega;
+    const double* f_ext;
+    int warm, pw;
+    int detect_only;    // stop once the contact set is current
+    int pack;           // 1: the velocities too, free_flight as cd_launch_pack
+    int free_flight;
+};
+#define CD_PREP_MAX_BLOCKS 256
+cudaError_t cd_launch_prepare(const CdGeom& g, const CdWork& w, const CdPrepIO& io, int blocks, int cluster,
+                              int precision, cudaStream_t stream, int* nl);
+// Blocks of the one-kernel preparation for n particles (0: it does not fit the
+// device), and whether they form one cluster.
+struct CdPrepPlan { int blocks, cluster; };
+CdPrepPlan cd_prepare_plan(int dim, int precision, int64_t n, int device);
+#define CD_PREP_MAX_N 500000   // see cd_prepare.cu
 cudaError_t cd_launch_pack(const CdGeom& g, const CdWork& w, const double* vel, const double* omega,
                            const double* radius, const double* inv_m, const double* inv_I, const double* f_ext,
                            int free_flight, int precision, cudaStream_t stream, int* nl);

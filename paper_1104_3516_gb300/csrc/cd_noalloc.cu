@@ -46,7 +46,8 @@
 #define NA_PK (NA_MT + NA_ALIGN(sizeof(double) * CD_NOALLOC_MAX_CONTACTS))
 #define NA_CAND (NA_PK + NA_ALIGN(sizeof(double) * 4 * CD_NOALLOC_MAX_CONTACTS))
 #define NA_RMAX (NA_CAND + NA_I32((size_t)CD_NOALLOC_MAX_N * CD_CAND))
-#define NA_BYTES (NA_RMAX + 256)
+#define NA_TOT (NA_RMAX + 256)
+#define NA_BYTES (NA_TOT + NA_I32(4 * CD_PREP_MAX_BLOCKS))
 
 static __device__ __align__(256) unsigned char cd_noalloc_scratch[NA_BYTES];
 
@@ -137,6 +138,8 @@ extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t
     unsigned long long* rbits = (unsigned long long*)(base + NA_RMAX);
     k_noalloc_begin<<<1, 1, 0, s>>>(ctrl, rbits, p.wall_pos[0], p.wall_pos[1], p.wall_pos[2], p.wall_pos[3],
                                     p.wall_pos[4], p.wall_pos[5]);
+    const CdPrepPlan plan = cd_prepare_plan((int)p.dim, CD_FP64, n, dev);
+    if (!plan.blocks) return na_error(CD_ERR_CUDA, "the detection kernel does not fit on this device");
     int gb = (int)((n + CD_BLOCK - 1) / CD_BLOCK);
     k_noalloc_radii<<<gb, CD_BLOCK, 0, s>>>((int)n, radius, rbits);
     unsigned long long hb[2] = {0ULL, 0ULL};
@@ -207,7 +210,12 @@ extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t
     w.pk_wall_pos = ctrl->wall_pos;   // device address inside the scratch
     const int pw = (p.dim == 2) ? 2 : 4;
     int nl = 0;
-    if ((e = cd_launch_detect(g, w, pos, radius, inv_mass, inv_inertia, 0, pw, s, &nl)) != cudaSuccess)
+    w.prep_tot = (int*)(base + NA_TOT);
+    CdPrepIO io = {};
+    io.pos = pos; io.radius = radius; io.inv_m = inv_mass; io.inv_I = inv_inertia;
+    io.pw = pw;
+    io.detect_only = 1;
+    if ((e = cd_launch_prepare(g, w, io, plan.blocks, plan.cluster, CD_FP64, s, &nl)) != cudaSuccess)
         return na_cuda(e, "detection launch");
     CdCtrl h;
     if ((e = cudaMemcpyAsync(&h, ctrl, sizeof h, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
