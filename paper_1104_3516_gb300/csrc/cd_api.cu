@@ -211,6 +211,11 @@ static size_t layout(cd_system* s, char* base, CdWork* w)
         t.fl_P = L.take<char>(base, fl ? cap * (s->p.dim == 2 ? 2 : 4) * real : 1);
         t.fl_P2 = L.take<char>(base, fl ? cap * (s->p.dim == 2 ? 2 : 4) * real : 1);
         t.fl_Vprev = L.take<char>(base, fl ? 2 * (n + 6) * vrec : 1);
+        t.fl_plan = L.take<FlowPlan>(base, fl && npk > 1 ? 1 : 0);
+        t.fl_list = L.take<int>(base, fl && npk > 1 ? npk : 1);
+        t.fl_start = L.take<int>(base, fl && npk > 1 ? npk + 1 : 1);
+        t.fl_mail = L.take<int>(base, fl && npk > 1 ? 2 * npk + 1 : 1);
+        t.fl_word = L.take<unsigned>(base, fl && npk > 1 ? 2 * npk + 1 : 1);
     }
     t.rep_top = L.take<int>(base, npk);
     t.rep_dmax = L.take<int>(base, npk);
@@ -383,6 +388,12 @@ static cd_status launch_solve(cd_system* s, int free_flight, int timed)
         CD_CUDA(s, cd_launch_pack(s->g, s->w, s->vel, s->omega, s->radius, s->inv_m, s->inv_I, s->f_ext, free_flight,
                                   (int)s->p.precision, s->stream, &s->launches));
     if (timed && (st = mark(s)) != CD_OK) return st;
+    if (s->g.flow && s->g.npk > 1) {
+        CD_CUDA(s, cd_launch_flow_batch(s->g, s->w, s->num_sms, s->flow_records, (int)s->p.precision,
+                                        (int)s->p.criterion, s->p.alpha, (int)s->p.max_sweeps, s->stream,
+                                        &s->launches));
+        return CD_OK;
+    }
     if (s->g.flow) {
         CD_CUDA(s, cd_launch_flow(s->g, s->w, s->num_sms, s->flow_records, (int)s->p.precision, (int)s->p.criterion, s->p.alpha,
                                   (int)s->p.max_sweeps, s->stream, &s->launches));
@@ -692,15 +703,18 @@ static cd_status create_impl(const cd_params* params, int64_t npk, const int64_t
     // caller who asks for merging (1 to 3) or for another block shape gets the
     // schedule that was asked for; up to 128 sweeps mode 4 keeps merging, which
     // n_phases reports (longer solves are faster without it, see cd_flow.cu)
-    s->flow_records = cd_flow_records((int)p.dim, (int)p.precision, s->device);
-    g.flow = (npk == 1 && g.par_p == 0.0 && g.ndom_total == 1 && p.criterion != CD_CONV_LOCAL && p.max_sweeps > 128 &&
+    s->flow_records = cd_flow_records((int)p.dim, (int)p.precision, npk > 1, s->device);
+    g.flow = (npk > 1) ? (p.criterion != CD_CONV_LOCAL && s->sweep_threads == CD_SWEEP_THREADS &&
+                          s->sweep_blocks == s->num_sms && s->num_sms <= FLOW_MAX_BLOCKS &&
+                          s->flow_records >= 2 * CD_KMAX) :
+             (g.par_p == 0.0 && g.ndom_total == 1 && p.criterion != CD_CONV_LOCAL && p.max_sweeps > 128 &&
               (p.merge_last_colour == 0 || p.merge_last_colour == 4) && s->sweep_threads == CD_SWEEP_THREADS &&
               s->sweep_blocks == s->num_sms && s->flow_records >= 0) ? 1 : 0;
     if (g.flow) {
         g.merge_last = 0;
         // records that cannot fit (more particles, so more contacts, than the blocks hold)
         // leave the shared memory to the L1 cache
-        if (n > (int64_t)s->flow_records * s->num_sms) s->flow_records = 0;
+        if (npk == 1 && n > (int64_t)s->flow_records * s->num_sms) s->flow_records = 0;
     }
     if (g.merge_last && !cd_sweep_fits(g, (int)p.precision, s->sweep_threads, s->sweep_blocks / s->num_sms)) {
         delete s;

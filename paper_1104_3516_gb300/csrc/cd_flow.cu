@@ -165,6 +165,7 @@ __device__ __forceinline__ double flow_sum_of(const u64 (&e)[2])
 
 #define FLOW_WORKERS 11                           // warps that update contacts
 #define FLOW_THREADS (32 * (FLOW_WORKERS + 1))    // and one that runs the convergence test
+#define FLOW_LEAST 112                            // contacts that a block of a batched system is given at least
 #define FLOW_ROWS 4                               // rows of tagged block sums
 #define FLOW_SLOTS 4                              // passes whose residual terms are kept
 #define FLOW_LAG1 16                              // from this pass on one starts before the test of the one before is
@@ -175,9 +176,25 @@ __device__ __forceinline__ double flow_sum_of(const u64 (&e)[2])
 // take two warps of 14, more than one of 24.
 #define FLOW_SPLIT 64
 
+// The blocks that solve a system (or a packing) together: nb of the grid from
+// block `start` on, this one the blk-th, with a barrier word of their own.
+struct FlowTeam {
+    unsigned* word;
+    int start, nb, blk;
+    __device__ __forceinline__ bool sync(CdCtrl* ctrl) const
+    {
+        if (nb == 1) {
+            __syncthreads();
+            return true;
+        }
+        return cd_team_sync(ctrl, word, (unsigned)nb, blk == 0);
+    }
+};
+
 // What the block's warps share.
 struct FlowShared {
     int lo[CD_KMAX], end[CD_KMAX];   // this block's positions of each colour
+    int half[CD_KMAX];               // 1: its contacts are split over two lanes each
     int base[CD_KMAX + 1];           // first of its warp items (32 contacts, or 16 split over two lanes each)
     int slot[CD_KMAX + 1];           // contacts of the colours before: place in the block's records
     int before[CD_KMAX];             // the colour with items before each (in turn), or -1 - the last one
@@ -252,8 +269,8 @@ __device__ __forceinline__ double shfl_pair(double v) { return __shfl_xor_sync(0
 // The control warp's part of a pass: the block's sum, published, every block's
 // sums gathered, the test.  The sums of lanes, then of blocks, are taken in a
 // fixed order, the same in every block.  Returns false when a wait gave up.
-__device__ __forceinline__ bool flow_control(CdCtrl* ctrl, FlowShared& sh, FlowSum* part, int pass, int nb, int nc,
-                                             int crit, double alpha, int max_sweeps, double& xprev)
+__device__ __forceinline__ bool flow_control(CdCtrl* ctrl, FlowShared& sh, FlowSum* part, const FlowTeam& tm, int pass,
+                                             int nc, int crit, double alpha, int max_sweeps, double& xprev)
 {
     const int lane = threadIdx.x & 31;
     bool on = true;
@@ -268,9 +285,10 @@ __device__ __forceinline__ bool flow_control(CdCtrl* ctrl, FlowShared& sh, FlowS
         if (__any_sync(0xffffffffu, __double_as_longlong(y) != 0)) x += y;
     }
     x = warp_sum_nz(x);
-    FlowSum* row = part + (size_t)(pass % FLOW_ROWS) * nb;
+    const int nb = tm.nb;
+    FlowSum* row = part + (size_t)(pass % FLOW_ROWS) * gridDim.x + tm.start;
     const unsigned tag = (unsigned)pass + 1u;
-    if (lane == 0) flow_sum_store(row + blockIdx.x, x, tag);
+    if (lane == 0) flow_sum_store(row + tm.blk, x, tag);
     x = 0.0;
     FlowBound bound;
     for (int b0 = 0; b0 < nb; b0 += 160) {
@@ -416,9 +434,15 @@ __device__ __forceinline__ void* flow_impulses(const CdWork& w, int pass)
     return u == 0 ? w.c_P : u == 1 ? w.fl_P : w.fl_P2;
 }
 
-template <int DIM, typename T>
-__global__ void __launch_bounds__(FLOW_THREADS, 1)
-k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
+// The solve of nc contacts by a team of blocks: K colours, colour k at the
+// colour-order positions [sh.lo[k], sh.end[k]) (narrowed to this block's), on
+// the particles body0 .. body1 - 1 (and the force-controlled walls).  Leaves
+// the velocities in w.V, the impulses in colour order (c_P) or key order (Pk),
+// the sweeps and the test in sh.  False when a wait gave up.
+template <int DIM, typename T, bool BATCH>
+__device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, FlowShared& sh, char* s_rec, int rec_cap,
+                                           const FlowTeam& tm, int K, int nc, T mu, int body0, int body1, int crit,
+                                           double alpha, int max_sweeps)
 {
     typedef FlowBody<DIM, T> Body;
     typedef FlowRecords<DIM, T> Records;
@@ -430,22 +454,15 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
     constexpr bool F64_2D = (DIM == 2) && std::is_same<T, double>::value;
     // |P| of an update is taken while the warp's next one waits (3D FP64 has no registers left for it)
     constexpr bool DEFER = (DIM == 2) || std::is_same<T, float>::value;
-    extern __shared__ __align__(128) char s_rec[];
-    __shared__ FlowShared sh;
-    __shared__ double s_red[FLOW_WORKERS + 1][3];
-    __shared__ double s_bc;
     CdCtrl* ctrl = w.ctrl;
-    if (ctrl->skip) return;
-    const int nc = ctrl->nc, K = ctrl->ncolours, nb = gridDim.x;
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    const int nb = tm.nb;
+    const int tid = tm.blk * blockDim.x + threadIdx.x, stride = nb * blockDim.x;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    u64 epoch = 0;
     u64* VT = (u64*)w.fl_V;
     FlowSum* part = (FlowSum*)w.fl_part;
     T4* V = (T4*)w.V;
     T4* Vprev = (T4*)w.fl_Vprev;
     constexpr int RW = (DIM == 2) ? 1 : 2;
-    const int nbody = g.n + (g.dyn_walls ? 6 : 0);
 
     // this block's positions of each colour, and their warp items
     if (threadIdx.x < 32) {
@@ -454,13 +471,19 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
             const int k = k0 + lane;
             int m = 0, c = 0;
             if (k < K) {
-                const int lo = w.colour_off[k], hi = w.colour_off[k + 1];
-                const int chunk = (hi - lo + nb - 1) / nb;
-                const int b0 = min(lo + (int)blockIdx.x * chunk, hi), e = min(b0 + chunk, hi);
-                sh.lo[k] = b0;
-                sh.end[k] = e;
-                c = e - b0;
-                m = (F64_2D && c <= FLOW_SPLIT) ? (c + 15) >> 4 : (c + 31) >> 5;
+                // whole warp items, dealt so that the blocks' totals over the colours
+                // are even: colour k's remainder starts at another block
+                const int lo = sh.lo[k], hi = sh.end[k];
+                const int half = F64_2D && hi - lo <= FLOW_SPLIT * nb;
+                const int sh_item = half ? 4 : 5;
+                const long long items = (hi - lo + (1 << sh_item) - 1) >> sh_item;
+                const int r = (int)(((long long)k * 5 * nb >> 3) % nb);
+                const int i0 = (int)((items * tm.blk + r) / nb), i1 = (int)((items * (tm.blk + 1) + r) / nb);
+                sh.lo[k] = min(lo + (i0 << sh_item), hi);
+                sh.end[k] = min(lo + (i1 << sh_item), hi);
+                sh.half[k] = half;
+                c = sh.end[k] - sh.lo[k];
+                m = i1 - i0;
             }
             int incl = m, ci = c;
 #pragma unroll
@@ -491,8 +514,8 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
         }
     }
     // tagged records (tag 0), cleared block sums
-    for (int i = tid; i < nbody; i += stride) {
-        if (i >= g.n && !cd_is_body(g, i)) continue;
+    for (int i = body0 + tid; i < body1; i += stride) {
+        if (!cd_is_body(g, i)) continue;
         Body x;
         T4 o;
         o.x = o.y = o.z = o.w = (T)0;
@@ -500,7 +523,7 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
         x.pack(V[RW * i], o, 0u);
         x.store(VT + (size_t)EB * i);
     }
-    for (int i = tid; i < FLOW_ROWS * nb; i += stride) flow_sum_store(part + i, 0.0, 0u);
+    if (threadIdx.x < FLOW_ROWS) flow_sum_store(part + threadIdx.x * gridDim.x + blockIdx.x, 0.0, 0u);
     __syncthreads();
     const int Q = sh.base[K];
     const bool res = sh.slot[K] <= rec_cap;   // the block's records fit its shared memory
@@ -512,7 +535,7 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
             atomicOr(&w.fl_mask[ab.x], 1ULL << k);
             if (cd_is_body(g, ab.y)) atomicOr(&w.fl_mask[ab.y], 1ULL << k);
         }
-    if (!cd_grid_sync(ctrl, nb, epoch)) return;
+    if (!tm.sync(ctrl)) return false;
     // a contact's place among each body's contacts and their number (8 bits
     // each), and the resident records
     for (int k = 0; k < K; ++k)
@@ -551,7 +574,7 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
     if (nc > 0 && wid == FLOW_WORKERS) {
         double xprev = 0.0;
         for (int pass = 0; ; ++pass) {
-            if (!flow_control(ctrl, sh, part, pass, nb, nc, crit, alpha, max_sweeps, xprev)) {
+            if (!flow_control(ctrl, sh, part, tm, pass, nc, crit, alpha, max_sweeps, xprev)) {
                 *(volatile int*)&sh.dead = 1;
                 break;
             }
@@ -594,7 +617,7 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
             for (int q = wid; q < Q; q += FLOW_WORKERS) {
                 while (q >= sh.base[k + 1]) ++k;
                 const int first = sh.lo[k], cnt = sh.end[k] - first;
-                const bool split = F64_2D && cnt <= FLOW_SPLIT;
+                const bool split = F64_2D && sh.half[k];
                 const int at = split ? 16 * (q - sh.base[k]) + (lane >> 1) : 32 * (q - sh.base[k]) + lane;
                 const bool act = at < cnt;
                 const int p = first + at, i = sh.slot[k] + at;
@@ -638,7 +661,7 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
                     if constexpr (DIM == 2) r.mt = m;
                     else r.m = m;
                     r.pk = 0;
-                    r.mu = (T)g.mu;
+                    r.mu = mu;
                 }
                 FlowHalf half;
                 if constexpr (F64_2D) {
@@ -764,20 +787,32 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
         }
     }
     __syncthreads();
-    if (sh.dead) return;
+    if (sh.dead) return false;
     const int sweeps = sh.stop;
-    // final impulses of this block's contacts in c_P
-    if (sweeps % 3) {
+    // final impulses of this block's contacts
+    if (BATCH || sweeps % 3) {
         const TP* P = (const TP*)flow_impulses(w, sweeps);
         for (int k = 0; k < K; ++k)
-            for (int p = sh.lo[k] + (int)threadIdx.x; p < sh.end[k]; p += blockDim.x)
-                ((TP*)w.c_P)[p] = P[p];
+            for (int p = sh.lo[k] + (int)threadIdx.x; p < sh.end[k]; p += blockDim.x) {
+                const TP x = P[p];
+                if constexpr (BATCH) {
+                    const size_t c = (size_t)w.perm[p];
+                    if constexpr (DIM == 2) {
+                        w.Pk[2 * c] = (double)x.x; w.Pk[2 * c + 1] = (double)x.y;
+                    } else {
+                        w.Pk[4 * c] = (double)x.x; w.Pk[4 * c + 1] = (double)x.y;
+                        w.Pk[4 * c + 2] = (double)x.z; w.Pk[4 * c + 3] = (double)x.w;
+                    }
+                } else {
+                    ((TP*)w.c_P)[p] = x;
+                }
+            }
     }
     // sweeps past the last: the velocities from before them
     const bool back = __syncthreads_or(last > sweeps);
-    if (!cd_grid_sync(ctrl, nb, epoch)) return;
-    for (int i = tid; i < nbody; i += stride) {
-        if (i >= g.n && !cd_is_body(g, i)) continue;
+    if (!tm.sync(ctrl)) return false;
+    for (int i = body0 + tid; i < body1; i += stride) {
+        if (!cd_is_body(g, i)) continue;
         T4 v, o;
         if (back && w.fl_mask[i] != 0ULL) {
             const T4* Vsave = Vprev + (size_t)((sweeps + 1) & 1) * RW * (g.n + 6);
@@ -792,25 +827,276 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
         V[RW * i] = v;
         if constexpr (DIM == 3) V[RW * i + 1] = o;
     }
-    finish_solve<DIM, T>(g, w, nc, nb, tid, stride, epoch, sweeps, sh.converged, sh.resid, sh.ravg, s_red, s_bc);
+    return true;
+}
+
+// A plain system: the whole grid is one team.
+template <int DIM, typename T>
+__global__ void __launch_bounds__(FLOW_THREADS, 1)
+k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
+{
+    extern __shared__ __align__(128) char s_rec[];
+    __shared__ FlowShared sh;
+    __shared__ double s_red[FLOW_WORKERS + 1][3];
+    __shared__ double s_bc;
+    CdCtrl* ctrl = w.ctrl;
+    if (ctrl->skip) return;
+    const int nc = ctrl->nc, K = ctrl->ncolours, nb = gridDim.x;
+    const FlowTeam tm{reinterpret_cast<unsigned*>(&ctrl->bar_count), 0, nb, (int)blockIdx.x};
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+        sh.lo[k] = w.colour_off[k];
+        sh.end[k] = w.colour_off[k + 1];
+    }
+    __syncthreads();
+    if (!flow_solve<DIM, T, false>(g, w, sh, s_rec, rec_cap, tm, K, nc, (T)g.mu, 0, g.n + (g.dyn_walls ? 6 : 0), crit,
+                                   alpha, max_sweeps))
+        return;
+    u64 epoch = 0;
+    finish_solve<DIM, T>(g, w, nc, nb, blockIdx.x * blockDim.x + threadIdx.x, nb * blockDim.x, epoch, sh.stop,
+                         sh.converged, sh.resid, sh.ravg, s_red, s_bc);
+}
+
+// ---------------------------------------------------------------------------
+// Batched systems.  Packings share nothing, so each is solved by a team of its
+// own and stops by itself: no barrier and no residual pass over the others.  A
+// packing asks for a block per `target` contacts.  The largest packings' teams
+// are laid out in advance until the grid is full; a team that is done takes
+// the largest packing left that asks for no more blocks than it has, with as
+// many as that asks for, and what is left of the team the one after, if that
+// is half as many or more.  (The first part of a team so keeps at least as many
+// blocks as any packing left asks for: none is left over.)  One step from zero
+// forces against the barrier schedule, which swept all packings together and
+// summed each one's |P| in a single block: 8 packings 45.5 -> 12.8 ms, 23 57.8
+// -> 18.0, 64 94 -> 53, 128 144 -> 102, 300 352 -> 238; from 64 on the FP64 pipe
+// bounds it (128: 67 ms).  Cut always, or only for a whole half: 300 packings
+// 370 and 252 ms, 128 106 and 110.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ int flow_ask(const CdWork& w, int b, int target, int blocks)
+{
+    const int nc = w.pk_coff[b + 1] - w.pk_coff[b];
+    const int ask = (nc + target - 1) / target;
+    return ask < 1 ? 1 : (ask > blocks ? blocks : ask);
+}
+
+__global__ void k_flow_plan(CdGeom g, CdWork w, int blocks, int records)
+{
+    __shared__ int s_at[FLOW_MAX_BLOCKS + 1];   // packings that ask for i blocks, then the next place of theirs
+    if (w.ctrl->skip) return;
+    FlowPlan* plan = w.fl_plan;
+    // all packings at once if the blocks' records can hold them so
+    const int room = blocks > 2 * g.npk ? blocks - g.npk : blocks / 2;
+    int target = (w.ctrl->nc + room - 1) / room;
+    // (dealt in warp items, a block may get one more than its share of every colour)
+    if (target > records - 32 * w.ctrl->ncolours) target = records - 32 * w.ctrl->ncolours;
+    if (target < FLOW_LEAST) target = FLOW_LEAST;
+    for (int i = threadIdx.x; i < 2 * g.npk + 1; i += blockDim.x) w.fl_word[i] = 0u;
+    for (int i = threadIdx.x; i <= blocks; i += blockDim.x) s_at[i] = 0;
+    __syncthreads();
+    for (int b = threadIdx.x; b < g.npk; b += blockDim.x) atomicAdd(&s_at[flow_ask(w, b, target, blocks)], 1);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int i = 0, run = 0, used = 0;
+        bool full = false;
+        for (int ask = blocks; ask >= 1; --ask) {
+            const int n = s_at[ask];
+            s_at[ask] = run;
+            int placed = 0;   // of these
+            while (placed < n && !full) {
+                if (used + ask > blocks) { full = true; break; }
+                w.fl_start[i++] = used;
+                used += ask;
+                ++placed;
+            }
+            plan->head[ask] = run + placed;
+            run += n;
+            plan->end[ask] = run;
+        }
+        w.fl_start[i] = used;
+        plan->target = target;
+        plan->placed = i;
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < g.npk; b += blockDim.x)
+        w.fl_list[atomicAdd(&s_at[flow_ask(w, b, target, blocks)], 1)] = b;
+}
+
+// Takes the packing that asks for most blocks, but no more than nb: its place
+// in fl_list, or -1 if none is left.  One warp.
+__device__ __forceinline__ int flow_take(FlowPlan* plan, int nb)
+{
+    const int lane = threadIdx.x & 31;
+    for (int g0 = nb; g0 >= 1; g0 -= 32) {
+        const int ask = g0 - lane;
+        const int end = ask >= 1 ? plan->end[ask] : 0;
+        unsigned m = __ballot_sync(0xffffffffu, ask >= 1 && cd_ld_volatile_int(&plan->head[ask]) < end);
+        while (m) {
+            const int at = __ffs(m) - 1;
+            int x = (lane == at) ? atomicAdd(&plan->head[ask], 1) : 0;
+            if (lane == at && x >= end) x = -1;
+            x = __shfl_sync(0xffffffffu, x, at);
+            if (x >= 0) return x;
+            m &= m - 1u;
+        }
+    }
+    return -1;
+}
+
+// First position in [lo, hi) (one colour, key order) whose contact's body a is
+// at least `particle`.
+__device__ __forceinline__ int flow_lower(const CdWork& w, int lo, int hi, int particle)
+{
+    while (lo < hi) {
+        const int mid = lo + ((hi - lo) >> 1);
+        if (w.c_ab[mid].x < particle) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+template <int DIM, typename T>
+__global__ void __launch_bounds__(FLOW_THREADS, 1)
+k_flow_batch(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
+{
+    extern __shared__ __align__(128) char s_rec[];
+    __shared__ FlowShared sh;
+    __shared__ double s_red[FLOW_WORKERS + 1][3];
+    CdCtrl* ctrl = w.ctrl;
+    if (ctrl->skip) return;
+    FlowPlan* plan = w.fl_plan;
+    const int K = ctrl->ncolours, me = blockIdx.x, target = plan->target, placed = plan->placed;
+    // the block's first team
+    int at = 0, start = w.fl_start[placed], nb = (int)gridDim.x - start, slot = 2 * g.npk;
+    bool given = me < start;
+    if (given) {
+        int hi = placed - 1;   // the last team that starts at or before this block
+        while (at < hi) {
+            const int mid = (at + hi + 1) >> 1;
+            if (w.fl_start[mid] <= me) at = mid; else hi = mid - 1;
+        }
+        start = w.fl_start[at];
+        nb = w.fl_start[at + 1] - start;
+    }
+    for (;;) {
+        while (!given) {
+            // the team of `slot` takes the next packing
+            const FlowTeam tm{&w.fl_word[slot], start, nb, me - start};
+            if (tm.blk == 0 && threadIdx.x < 32) {
+                const int x = flow_take(plan, nb);
+                if (threadIdx.x == 0) *(volatile int*)&w.fl_mail[slot] = x;
+            }
+            if (!tm.sync(ctrl)) return;
+            at = cd_ld_volatile_int(&w.fl_mail[slot]);
+            if (at < 0) return;
+            int ask = flow_ask(w, w.fl_list[at], target, (int)gridDim.x);
+            if (2 * nb < 3 * ask) ask = nb;   // not worth a team of its own
+            given = me < start + ask;
+            if (given) {
+                nb = ask;
+            } else {
+                start += ask;
+                nb -= ask;
+                slot = g.npk + at;
+            }
+        }
+        given = false;
+        slot = at;
+        const FlowTeam tm{&w.fl_word[slot], start, nb, me - start};
+        const int b = w.fl_list[at];
+        const int first = w.pk[b].first, count = w.pk[b].count;
+        const int c0 = w.pk_coff[b], nc = w.pk_coff[b + 1] - c0;
+        for (int k = threadIdx.x; k < K; k += blockDim.x) {
+            const int lo = flow_lower(w, w.colour_off[k], w.colour_off[k + 1], first);
+            sh.lo[k] = lo;
+            sh.end[k] = flow_lower(w, lo, w.colour_off[k + 1], first + count);
+        }
+        __syncthreads();
+        if (!flow_solve<DIM, T, true>(g, w, sh, s_rec, rec_cap, tm, K, nc, (T)w.pk[b].mu, first, first + count, crit,
+                                      alpha, max_sweeps))
+            return;
+        if (tm.blk == 0) {
+            // the packing's wall forces and statistics
+            const int pw = (DIM == 2) ? 2 : 4;
+            double lo3[3] = {0.0, 0.0, 0.0}, hi3[3] = {0.0, 0.0, 0.0};
+            for (int i = c0 + (int)threadIdx.x; i < c0 + nc; i += blockDim.x) {
+                const int bb = w.pairs[i].y;
+                if (bb < g.n) continue;
+                const int k = (bb - g.n) % 6;
+                const double pn = w.Pk[pw * i];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    if (q == k) lo3[q] += pn;
+                    if (q + 3 == k) hi3[q] += pn;
+                }
+            }
+            block_sum<3>(lo3, s_red);
+            block_sum<3>(hi3, s_red);
+            if (threadIdx.x == 0) {
+                double* st = w.pk_stats + CD_PKSTATS * b;
+                st[PKS_SWEEPS] = (double)sh.stop;
+                st[PKS_CONV] = (double)sh.converged;
+                st[PKS_RESID] = sh.resid;
+                st[PKS_RAVG] = sh.ravg;
+                st[PKS_RPREV] = sh.ravg;
+                st[PKS_NC] = (double)nc;
+                for (int q = 0; q < 3; ++q) {
+                    st[PKS_WF0 + q] = lo3[q] / g.dt;
+                    st[PKS_WF0 + 3 + q] = hi3[q] / g.dt;
+                }
+            }
+        }
+    }
+}
+
+// The call's totals over the packings.
+__global__ void k_flow_totals(CdGeom g, CdWork w)
+{
+    __shared__ long long s_sum, s_upd, s_open;
+    __shared__ int s_max;
+    CdCtrl* ctrl = w.ctrl;
+    if (ctrl->skip || ctrl->error != CDE_NONE) return;
+    if (threadIdx.x == 0) { s_sum = 0; s_upd = 0; s_open = 0; s_max = 0; }
+    __syncthreads();
+    for (int b = threadIdx.x; b < g.npk; b += blockDim.x) {
+        const double* st = w.pk_stats + CD_PKSTATS * b;
+        const long long sw = (long long)st[PKS_SWEEPS];
+        atomicAdd((unsigned long long*)&s_sum, (unsigned long long)sw);
+        atomicAdd((unsigned long long*)&s_upd, (unsigned long long)(sw * (long long)st[PKS_NC]));
+        if (st[PKS_CONV] == 0.0) atomicAdd((unsigned long long*)&s_open, 1ULL);
+        atomicMax(&s_max, (int)sw);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const double* st = w.pk_stats;
+        for (int q = 0; q < 6; ++q) ctrl->wall_force[q] = st[PKS_WF0 + q];
+        ctrl->r_avg = st[PKS_RAVG];
+        ctrl->residual = st[PKS_RESID];
+        ctrl->steps_done += 1;
+        ctrl->total_sweeps += s_sum;
+        ctrl->total_updates += s_upd;
+        ctrl->n_not_conv += s_open;
+        if (s_max > ctrl->max_sweeps_step) ctrl->max_sweeps_step = s_max;
+        ctrl->sweeps = s_max;
+        ctrl->converged = (s_open == 0);
+    }
 }
 
 struct FlowKernel { const void* fn; int body_bytes, record_bytes; };
-static FlowKernel flow_kernel(int dim, int precision)
+static FlowKernel flow_kernel(int dim, int precision, int batch)
 {
-#define FLOW_K(D, T) FlowKernel{(const void*)k_flow<D, T>, (int)sizeof(FlowBody<D, T>), FlowRecords<D, T>::BYTES}
+#define FLOW_K(D, T) \
+    FlowKernel{batch ? (const void*)k_flow_batch<D, T> : (const void*)k_flow<D, T>, (int)sizeof(FlowBody<D, T>), \
+               FlowRecords<D, T>::BYTES}
     if (dim == 2) return precision == CD_FP64 ? FLOW_K(2, double) : FLOW_K(2, float);
     return precision == CD_FP64 ? FLOW_K(3, double) : FLOW_K(3, float);
 #undef FLOW_K
 }
 
-size_t cd_flow_body_bytes(int dim, int precision) { return (size_t)flow_kernel(dim, precision).body_bytes; }
+size_t cd_flow_body_bytes(int dim, int precision) { return (size_t)flow_kernel(dim, precision, 0).body_bytes; }
 
 // Contacts a block keeps in shared memory (a multiple of 16, so that every
 // array of the records stays aligned), or -1 if the kernel does not fit.
-int cd_flow_records(int dim, int precision, int device)
+int cd_flow_records(int dim, int precision, int batch, int device)
 {
-    const FlowKernel f = flow_kernel(dim, precision);
+    const FlowKernel f = flow_kernel(dim, precision, batch);
     int most = 0;
     cudaFuncAttributes a;
     if (cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
@@ -827,13 +1113,13 @@ int cd_flow_records(int dim, int precision, int device)
     return recs;
 }
 
-cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int criterion,
-                           double alpha, int max_sweeps, cudaStream_t s, int* nl)
+static cudaError_t flow_launch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int batch,
+                               int criterion, double alpha, int max_sweeps, cudaStream_t s, int* nl)
 {
     cudaError_t e = cudaMemsetAsync(w.ctrl, 0, 2 * sizeof(u64), s);
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(w.fl_mask, 0, sizeof(u64) * (size_t)(g.n + 6), s)) != cudaSuccess) return e;
-    const FlowKernel f = flow_kernel(g.dim, precision);
+    const FlowKernel f = flow_kernel(g.dim, precision, batch);
     CdGeom ga = g;
     CdWork wa = w;
     int crit = criterion, ms = max_sweeps, rc = records;
@@ -842,4 +1128,22 @@ cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, int blocks, int rec
     ++*nl;
     return cudaLaunchCooperativeKernel(f.fn, dim3(blocks), dim3(FLOW_THREADS), args,
                                        (size_t)(records * f.record_bytes), s);
+}
+
+cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int criterion,
+                           double alpha, int max_sweeps, cudaStream_t s, int* nl)
+{
+    return flow_launch(g, w, blocks, records, precision, 0, criterion, alpha, max_sweeps, s, nl);
+}
+
+cudaError_t cd_launch_flow_batch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision,
+                                 int criterion, double alpha, int max_sweeps, cudaStream_t s, int* nl)
+{
+    k_flow_plan<<<1, 512, 0, s>>>(g, w, blocks, records);
+    ++*nl;
+    cudaError_t e = flow_launch(g, w, blocks, records, precision, 1, criterion, alpha, max_sweeps, s, nl);
+    if (e != cudaSuccess) return e;
+    k_flow_totals<<<1, 256, 0, s>>>(g, w);
+    ++*nl;
+    return cudaGetLastError();
 }

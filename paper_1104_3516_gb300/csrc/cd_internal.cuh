@@ -85,6 +85,15 @@ struct CdPack {
     unsigned long long seed;  // colouring seed of the packing
 };
 
+// Batched systems by dataflow (cd_flow.cu): how the blocks form teams.
+#define FLOW_MAX_BLOCKS 512
+struct FlowPlan {
+    int target;                     // contacts a block is given
+    int placed;                     // packings whose teams are laid out in advance
+    int head[FLOW_MAX_BLOCKS + 1];  // packings that ask for g blocks: the next one of them to be taken,
+    int end[FLOW_MAX_BLOCKS + 1];   // and the end of them, in fl_list
+};
+
 // Pointers into the caller's workspace.
 struct CdWork {
     CdCtrl* ctrl;
@@ -187,6 +196,11 @@ struct CdWork {
     void* fl_P;         // cap: impulses after the sweeps s with s % 3 = 1 (c_P: 0)
     void* fl_P2;        // cap: ... = 2
     void* fl_Vprev;     // 2 (n + 6) velocity records from before the latest two sweeps
+    FlowPlan* fl_plan;  // batched systems: which blocks solve which packings
+    int* fl_list;       // npk: packings by the blocks they ask for, most first
+    int* fl_start;      // npk + 1: first block of each team laid out in advance
+    int* fl_mail;       // 2 npk + 1: the packing taken next, by the team that takes it
+    unsigned* fl_word;  // 2 npk + 1: barrier words of the teams
     // repair of the highest colour (global colour order)
     int* rep_top;       // npk: highest colour of each packing
     int* rep_dmax;      // npk: most contacts of one body of the packing
@@ -370,13 +384,12 @@ __device__ __forceinline__ int cd_ld_volatile_int(const int* p)
 // arrival (thread 0 gets the counter's old value); the block may then issue
 // work that touches nothing another block reads before the barrier (loads of
 // read-only records) while the others arrive; cd_grid_wait completes it.
-__device__ __forceinline__ unsigned cd_grid_arrive(CdCtrl* ctrl, unsigned long long nblocks)
+__device__ __forceinline__ unsigned cd_bar_arrive(unsigned* word, unsigned nblocks, bool first)
 {
     __syncthreads();
     unsigned old = 0;
     if (threadIdx.x == 0) {
-        unsigned* word = reinterpret_cast<unsigned*>(&ctrl->bar_count);
-        const unsigned add = (blockIdx.x == 0) ? (0x80000000u - (unsigned)(nblocks - 1)) : 1u;
+        const unsigned add = first ? (0x80000000u - (nblocks - 1u)) : 1u;
         // release: the block's writes (ordered before this thread by the block
         // barrier above) are visible to whoever acquires the flipped word
         asm volatile("atom.add.release.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(word), "r"(add) : "memory");
@@ -384,11 +397,10 @@ __device__ __forceinline__ unsigned cd_grid_arrive(CdCtrl* ctrl, unsigned long l
     return old;
 }
 
-__device__ __forceinline__ bool cd_grid_wait(CdCtrl* ctrl, unsigned old, unsigned long long& epoch)
+__device__ __forceinline__ bool cd_bar_wait(CdCtrl* ctrl, const unsigned* word, unsigned old)
 {
     __shared__ int s_ok;
     if (threadIdx.x == 0) {
-        const unsigned* word = reinterpret_cast<const unsigned*>(&ctrl->bar_count);
         int ok = 1;
         unsigned long long t0 = 0;
         unsigned spins = 0;
@@ -406,10 +418,28 @@ __device__ __forceinline__ bool cd_grid_wait(CdCtrl* ctrl, unsigned old, unsigne
         // the acquire load that saw the flip orders thread 0's later accesses;
         // the block barrier below extends that to the other threads
         s_ok = ok;
-        ++epoch;
     }
     __syncthreads();
     return s_ok != 0;
+}
+
+// The barrier of `nblocks` blocks of a cooperative grid on a word of their
+// own (first: the block that adds the flip).
+__device__ __forceinline__ bool cd_team_sync(CdCtrl* ctrl, unsigned* word, unsigned nblocks, bool first)
+{
+    const unsigned old = cd_bar_arrive(word, nblocks, first);
+    return cd_bar_wait(ctrl, word, old);
+}
+
+__device__ __forceinline__ unsigned cd_grid_arrive(CdCtrl* ctrl, unsigned long long nblocks)
+{
+    return cd_bar_arrive(reinterpret_cast<unsigned*>(&ctrl->bar_count), (unsigned)nblocks, blockIdx.x == 0);
+}
+
+__device__ __forceinline__ bool cd_grid_wait(CdCtrl* ctrl, unsigned old, unsigned long long& epoch)
+{
+    ++epoch;
+    return cd_bar_wait(ctrl, reinterpret_cast<const unsigned*>(&ctrl->bar_count), old);
 }
 
 __device__ __forceinline__ bool cd_grid_sync(CdCtrl* ctrl, unsigned long long nblocks, unsigned long long& epoch)
@@ -511,8 +541,10 @@ cudaError_t cd_launch_sweep(const CdGeom& g, const CdWork& w, int coop_blocks, i
                             int criterion, double alpha, int max_sweeps, int pw, cudaStream_t stream, int* nl);
 cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int criterion,
                            double alpha, int max_sweeps, cudaStream_t stream, int* nl);
+cudaError_t cd_launch_flow_batch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision,
+                                 int criterion, double alpha, int max_sweeps, cudaStream_t stream, int* nl);
 size_t cd_flow_body_bytes(int dim, int precision);
-int cd_flow_records(int dim, int precision, int device);
+int cd_flow_records(int dim, int precision, int batch, int device);
 int cd_sweep_fits(const CdGeom& g, int precision, int threads, int per_sm);
 cudaError_t cd_launch_unpack(const CdGeom& g, const CdWork& w, double* pos, double* vel, double* omega,
                              double* theta, int integrate, int precision, cudaStream_t stream, int* nl);

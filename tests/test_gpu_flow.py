@@ -1,4 +1,4 @@
-"""The dataflow solve (plain systems whose sweep cap exceeds 128, without an
+"""The dataflow solve (batches, and plain systems whose sweep cap exceeds 128, without an
 asked-for merge) against the barrier schedule on the same system: the order of
 the updates is the same, so impulses, velocities and positions are bit-equal,
 and the stopping sweep is the same (a solve that stops after sweeps that were
@@ -74,3 +74,46 @@ def test_cap_reached_and_few_contacts():
 def test_force_controlled_lid_is_bit_identical(precision):
     """The lid is a body of many colours (its contacts conflict)."""
     both(W.pressure_column(seed=6, n=600), steps=3, precision=precision)
+
+
+@pytest.mark.parametrize("count", [2, 7, 40, 200])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_batches_are_bit_identical(count, precision):
+    """Packings solved by teams of blocks (one round of teams, several rounds,
+    packings without a contact among them) against the barrier schedule, which
+    another block shape keeps."""
+    batch = [W.settled_pile(seed=50 + b, n=int(n), mu=0.1 + 0.5 * b / count)
+             for b, n in enumerate(W.batch_sizes(seed=3, n_packings=count, nmin=20, nmax=3000))]
+    batch[1] = W.dilute_discs(seed=1, n=5, width=40.0)
+    kw = dict(batch=batch, precision=precision, alpha=1e-3, max_sweeps=150, max_contacts=4 * sum(b.n for b in batch))
+    a = gpu_system(batch[0], sweep_threads=256, sweep_blocks_per_sm=2, **kw)
+    b = gpu_system(batch[0], **kw)
+    for _ in range(2):
+        sa, sb = a.step(1), b.step(1)
+        for k in ("total_sweeps", "total_contact_updates", "max_sweeps_in_step", "n_not_converged"):
+            assert sa[k] == sb[k], k
+        for p, q in zip(a.packing_stats(), b.packing_stats()):
+            for k in ("sweeps", "converged", "n_contacts", "wall_pos"):
+                assert p[k] == q[k], k
+            assert abs(p["r_avg"] - q["r_avg"]) <= 1e-13 * p["r_avg"]
+            assert np.allclose(p["wall_force"], q["wall_force"], rtol=1e-13, atol=0)
+        ca, cb = a.contacts(), b.contacts()
+        for k in ("pairs", "colour", "impulse"):
+            assert np.array_equal(ca[k], cb[k]), k
+        xa, xb = a.state(), b.state()
+        for k in ("x", "v", "w"):
+            assert np.array_equal(xa[k], xb[k]), k
+
+
+def test_batch_of_sphere_gases_is_bit_identical():
+    batch = [W.sphere_gas(seed=b, n=300 + 900 * b, floor=16.0, vsig=0.5) for b in range(4)]
+    a = gpu_system(batch[0], batch=batch, sweep_threads=256, sweep_blocks_per_sm=2)
+    b = gpu_system(batch[0], batch=batch)
+    for _ in range(3):
+        assert a.step(1)["total_sweeps"] == b.step(1)["total_sweeps"]
+    ca, cb = a.contacts(), b.contacts()
+    for k in ca:
+        assert np.array_equal(ca[k], cb[k]), k
+    xa, xb = a.state(), b.state()
+    for k in ("x", "v", "w"):
+        assert np.array_equal(xa[k], xb[k]), k
