@@ -21,18 +21,21 @@
 // three sweeps are kept in turn, and the velocities from before the last two,
 // so the sweeps begun past the last one are taken back.
 //
-// What bounds it: in FP64 the FP64 pipe (19 cycles a warp instruction on an
-// SM, 29 of them a warp of contacts) while the neighbours' records are under
-// way between the SMs; in FP32, and in small systems, the way of a record
+// What bounds it: in FP64 the FP64 pipe (64 cycles a warp instruction on each
+// quarter of an SM, 24 of them a warp of contacts: ~3,200 cycles a colour of the
+// 100,000-disc pile) and then the way of the records to the next colour (~1,700)
+// in turn, since neighbouring blocks move in step; in FP32, and in small systems, the way of a record
 // from SM to SM (~500 cycles on a die, ~850 across) once per colour, plus the
 // update (FP64: ~1,700 cycles for a whole warp of contacts; ~1,100 for 16
 // contacts split over lane pairs, where a block has few).  Per sweep, against
 // the barrier schedule (grid barrier 2,900 cycles a colour, then the velocity
-// loads): 100,000-disc pile FP64 28.4 -> 18.1 us, FP32 18.0 -> 10.2 us;
+// loads): 100,000-disc pile FP64 28.4 -> 17.2 us, FP32 18.0 -> 10.2 us;
 // 5,000 discs FP64 20.6 -> 9.9 us; 2,000 discs 20.9 -> 10.1 us.  Tried and not kept: one lane
 // looking for its warp (FP32 7% slower, 5,000 discs 12%), pauses between looks
 // (5,000 discs 2 to 15% slower), 15 or 7 updating warps in place of 11 (FP64 2
-// and 17% slower), records through L1 (FP64 pile 24.3 us a sweep).
+// and 17% slower), records through L1 (FP64 pile 24.3 us a sweep), two far-apart
+// regions a block on four warps each, to run one while the other waits (they
+// fall into step: FP64 10% slower, FP32 19%).
 #include "cd_sweep_core.cuh"
 
 // ---------------------------------------------------------------------------
@@ -243,14 +246,13 @@ __device__ __forceinline__ bool flow_wait_shared(CdCtrl* ctrl, FlowShared& sh, c
 }
 
 // Looks again at the records at pa and pb (null: none) until they carry their
-// tags (the caller has looked once); the lanes of a warp leave together.
-// False when a wait gave up.
+// tags (the caller has looked once: ra, rb); the lanes of a warp leave
+// together.  False when a wait gave up.
 template <int DIM, typename T>
 __device__ __forceinline__ bool flow_wait(CdCtrl* ctrl, FlowShared& sh, const u64* pa, unsigned ta, const u64* pb,
-                                          unsigned tb, FlowBody<DIM, T>& A, FlowBody<DIM, T>& B)
+                                          unsigned tb, FlowBody<DIM, T>& A, FlowBody<DIM, T>& B, bool ra, bool rb)
 {
     FlowBound bound;
-    bool ra = !pa || A.has(ta), rb = !pb || B.has(tb);
     while (!__all_sync(0xffffffffu, ra && rb)) {
         if (!ra) A.load(pa);
         if (!rb) B.load(pb);
@@ -378,15 +380,15 @@ struct FlowRecords {
 // velocities are there: between two FP64 instructions a select or a shuffle
 // costs ~44 cycles beyond their own 64 each.
 struct FlowHalf {
-    double c1, c2, c3, c4, c5, bias, Pold;
+    double c0, c1, c2, c3, c4, c5, Pold;
     __device__ __forceinline__ void choose(bool odd, const Rec<2, double>& r)
     {
         c1 = odd ? -r.geo.y : r.geo.x;
         c2 = odd ? r.geo.x : r.geo.y;
-        c3 = odd ? -r.sa.y : 1.0;
+        c0 = odd ? -0.0 : r.geo.z;   // (adding -0 to a product leaves it as it is)
+        c3 = odd ? -r.sa.y : 0.0;
         c4 = odd ? -r.sb.y : 0.0;
         c5 = odd ? -r.mt : -r.geo.w;
-        bias = r.geo.z;
         Pold = odd ? r.P.y : r.P.x;
     }
     // Returns this lane's impulse component, and in v1 the new velocity record
@@ -399,10 +401,10 @@ struct FlowHalf {
         const double xa = odd ? va.x : va.y, xb = odd ? vb.x : vb.y;
         double Pnew = Pold, d = Pold;
         if (!apply_only) {
-            const double u3 = odd ? va.z : bias, u4 = odd ? vb.z : 0.0;
+            const double u3 = odd ? va.z : 0.0, u4 = odd ? vb.z : 0.0;
             const double dvx = __dsub_rn(vb.x, va.x), dvy = __dsub_rn(vb.y, va.y);
-            double u = __fma_rn(dvy, c2, __dmul_rn(dvx, c1));     // u_n | (dv x n)
-            u = __fma_rn(c3, u3, u);                              // b + u_n | - r_a w_a
+            double u = __fma_rn(dvy, c2, __fma_rn(dvx, c1, c0));  // b + u_n | (dv x n)
+            u = __fma_rn(c3, u3, u);                              //         | - r_a w_a
             u = __fma_rn(c4, u4, u);                              //         | - r_b w_b
             const double Ps = __fma_rn(c5, u, Pold);
             const double lim = pos_part(shfl_pair(__dmul_rn(r.mu, Ps)));   // mu max(P_n*, 0)
@@ -674,8 +676,8 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                         half.choose(lane & 1, r);
                     }
                 }
-                settle();
                 if (gate) {
+                    settle();
                     // not before the block's items of the colour before are done: the records are
                     // hardly there earlier, and looks that find nothing delay every other access
                     const int kb = sh.before[k] >= 0 ? sh.before[k] : -1 - sh.before[k];
@@ -684,7 +686,11 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                     if (pa) A.load(pa);
                     if (pb) B.load(pb);
                 }
-                if (!flow_wait<DIM, T>(ctrl, sh, pa, ta, pb, tb, A, B)) { dead = true; break; }
+                bool ra = !pa || A.has(ta), rb = !pb || B.has(tb);
+                if (!__all_sync(0xffffffffu, ra && rb)) {
+                    settle();   // in the wait, or else after this item's records are stored
+                    if (!flow_wait<DIM, T>(ctrl, sh, pa, ta, pb, tb, A, B, ra, rb)) { dead = true; break; }
+                }
                 T4 va, oa, vb, ob;
                 if constexpr (F64_2D) {
                     if (split) {
@@ -712,6 +718,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                             const int mine = odd ? (int)((ord >> 16) & 255u) : (int)(ord & 255u);
                             if (save && mine == 0 && !(odd && wall)) Vsave[odd ? r.ab.y : r.ab.x] = odd ? vb : va;
                         }
+                        settle();
                         const double Pother = shfl_pair(Pnew);
                         pend.x = Pnew;
                         pend.y = Pother;
@@ -764,6 +771,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                         Pout[p] = Pn;
                         if (res) rec.P[i] = Pn;
                     }
+                    settle();
                     if constexpr (DEFER) {
                         pend = Pn;
                         owed = true;

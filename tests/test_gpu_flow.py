@@ -117,3 +117,17 @@ def test_batch_of_sphere_gases_is_bit_identical():
     xa, xb = a.state(), b.state()
     for k in ("x", "v", "w"):
         assert np.array_equal(xa[k], xb[k]), k
+
+
+def test_residual_magnitudes_match_64_bits():
+    """R_avg against the mean of sqrt(P_n^2 + P_t^2) of the impulses, for
+    magnitudes over many decades (the masses scale the impulses): within the
+    rounding of the integer root (7.3e-15 a contact) and of the sum."""
+    for scale in (1e-30, 1e-3, 1.0, 1e25):
+        wl = W.dense_biaxial_discs(seed=4, n=3000)
+        wl.inv_m, wl.inv_I = wl.inv_m / scale, wl.inv_I / scale
+        g = gpu_system(wl, criterion=-1, max_sweeps=200)
+        r = g.step(1)["last"]["r_avg"]
+        P = g.contacts()["impulse"].astype(np.longdouble)
+        exact = np.sqrt((P * P).sum(1)).mean()
+        assert abs(np.longdouble(r) - exact) <= 2e-14 * exact
