@@ -155,10 +155,9 @@ typedef struct {
                                velocity changes are summed at the end of the
                                sweep: what a multi-processor run of the paper
                                computes, on one GPU.  The workspace grows by
-                               2 velocity records (and their start copies) per
-                               contact of capacity.  Plain systems with the
-                               colour-barrier schedule, kinematic walls, no
-                               mixed update, no tape.  All 1: Gauss-Seidel. */
+                               2 velocity records (with their start copies and
+                               tagged forms) per contact of capacity.  Plain systems,
+                               kinematic walls, no mixed update, no tape.  All 1: Gauss-Seidel. */
     int64_t parallel_redraw; /* mixed update (parallel_p): 0 the parallel subset
                                is fixed per contact key; 1 it is drawn afresh
                                in every iteration step (the step's number

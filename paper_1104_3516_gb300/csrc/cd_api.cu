@@ -204,8 +204,10 @@ static size_t layout(cd_system* s, char* base, CdWork* w)
     t.prep_hist = L.take<int>(base, s->prep.blocks ? CD_KMAX * CD_PREP_MAX_BLOCKS : 1);
     {
         const bool fl = s->g.flow != 0;
-        t.fl_V = L.take<char>(base, fl ? (n + 6) * cd_flow_body_bytes((int)s->p.dim, (int)s->p.precision) : 1);
-        t.fl_mask = L.take<unsigned long long>(base, fl ? n + 6 : 1);
+        const size_t nrec = n + 6 + vcap;
+        t.fl_nrec = (int)nrec;
+        t.fl_V = L.take<char>(base, fl ? nrec * cd_flow_body_bytes((int)s->p.dim, (int)s->p.precision) : 1);
+        t.fl_mask = L.take<unsigned long long>(base, fl ? nrec : 1);
         t.fl_ord = L.take<unsigned>(base, fl ? cap : 1);
         t.fl_part = L.take<char>(base, fl ? 64 * G : 1);
         t.fl_P = L.take<char>(base, fl ? cap * (s->p.dim == 2 ? 2 : 4) * real : 1);
@@ -703,13 +705,14 @@ static cd_status create_impl(const cd_params* params, int64_t npk, const int64_t
     // caller who asks for merging (1 to 3) or for another block shape gets the
     // schedule that was asked for; up to 128 sweeps mode 4 keeps merging, which
     // n_phases reports (longer solves are faster without it, see cd_flow.cu)
-    s->flow_records = cd_flow_records((int)p.dim, (int)p.precision, npk > 1, s->device);
+    s->flow_records = cd_flow_records(g, (int)p.precision, s->device);
     g.flow = (npk > 1) ? (p.criterion != CD_CONV_LOCAL && s->sweep_threads == CD_SWEEP_THREADS &&
                           s->sweep_blocks == s->num_sms && s->num_sms <= FLOW_MAX_BLOCKS &&
                           s->flow_records >= 2 * CD_KMAX) :
-             (g.par_p == 0.0 && g.ndom_total == 1 && p.criterion != CD_CONV_LOCAL && p.max_sweeps > 128 &&
-              (p.merge_last_colour == 0 || p.merge_last_colour == 4) && s->sweep_threads == CD_SWEEP_THREADS &&
-              s->sweep_blocks == s->num_sms && s->flow_records >= 0) ? 1 : 0;
+             (g.par_p == 0.0 && p.criterion != CD_CONV_LOCAL && s->sweep_threads == CD_SWEEP_THREADS &&
+              s->sweep_blocks == s->num_sms && s->flow_records >= 0 &&
+              (g.ndom_total > 1 ||   // (nothing to merge there)
+               (p.max_sweeps > 128 && (p.merge_last_colour == 0 || p.merge_last_colour == 4)))) ? 1 : 0;
     if (g.flow) {
         g.merge_last = 0;
         // records that cannot fit (more particles, so more contacts, than the blocks hold)

@@ -10,7 +10,7 @@
 // after the walls' records for the others).  The sweep kernel updates every
 // contact on its domain's records, and after each sweep adds the records'
 // changes into the particle's velocity and copies the sum back into every
-// view (cd_sweep.cu).  This file assigns contacts to domains and builds the
+// view (cd_flow.cu; cd_sweep.cu with a barrier per colour).  This file assigns contacts to domains and builds the
 // record map.
 #include "cd_internal.cuh"
 

@@ -194,14 +194,17 @@ struct FlowTeam {
     }
 };
 
+#define FLOW_KINDS (CD_KMAX + 1)
+
 // What the block's warps share.
 struct FlowShared {
-    int lo[CD_KMAX], end[CD_KMAX];   // this block's positions of each colour
-    int half[CD_KMAX];               // 1: its contacts are split over two lanes each
-    int base[CD_KMAX + 1];           // first of its warp items (32 contacts, or 16 split over two lanes each)
-    int slot[CD_KMAX + 1];           // contacts of the colours before: place in the block's records
-    int before[CD_KMAX];             // the colour with items before each (in turn), or -1 - the last one
-    int done[CD_KMAX];               // its warp items done, over all passes
+    // by colour (and the shared particles' sums as one more)
+    int lo[FLOW_KINDS], end[FLOW_KINDS];   // this block's positions
+    int half[FLOW_KINDS];                  // 1: its contacts are split over two lanes each
+    int base[FLOW_KINDS + 1];              // first of its warp items (32 contacts, or 16 split over two lanes each)
+    int slot[FLOW_KINDS + 1];              // contacts of the colours before: place in the block's records
+    int before[FLOW_KINDS];                // the colour with items before each (in turn), or -1 - the last one
+    int done[FLOW_KINDS];                  // its warp items done, over all passes
     double acc[FLOW_SLOTS][FLOW_WORKERS][32]; // residual terms of a pass by worker lane
     int arrived[FLOW_SLOTS];         // workers that have left them (counted over the passes of a slot)
     int decided;                     // last pass the test is known of
@@ -436,12 +439,97 @@ __device__ __forceinline__ void* flow_impulses(const CdWork& w, int pass)
     return u == 0 ? w.c_P : u == 1 ? w.fl_P : w.fl_P2;
 }
 
+// Record r of a contact's second body moves: a particle's, a view's or a
+// force-controlled wall's, not a kinematic wall's.
+template <bool VIEWS>
+__device__ __forceinline__ bool flow_moves(const CdGeom& g, int r)
+{
+    return VIEWS ? (r < g.n || r >= cd_view_base(g)) : cd_is_body(g, r);
+}
+
+// 1 if record r belongs to a particle with several.
+__device__ __forceinline__ unsigned flow_shared(const CdWork& w, int vbase, int n, int r)
+{
+    return r >= vbase || (r < n && w.view_off[r + 1] > w.view_off[r]) ? 1u : 0u;
+}
+
+// The sums after a pass's contacts (dom_combine's, in its order): a lane for
+// each view, the particle's first one works.
+template <int DIM, typename T>
+__device__ __forceinline__ bool flow_sum_views(const CdGeom& g, const CdWork& w, CdCtrl* ctrl, FlowShared& sh, u64* VT,
+                                               int vbase, int q, bool act, int pass)
+{
+    typedef FlowBody<DIM, T> Body;
+    typedef typename Vec<T>::V4 T4;
+    constexpr int EB = Body::G * Body::N;
+    constexpr int RW = (DIM == 2) ? 1 : 2;
+    T4* V0 = (T4*)w.V0;
+    const int i = act ? w.view_owner[q] : 0;
+    const bool lead = act && q == w.view_off[i];
+    const int e = lead ? w.view_off[i + 1] : q;
+    const unsigned ni = lead ? (unsigned)__popcll(w.fl_mask[i]) : 0u;
+    FlowBound bound;
+    bool ready = !lead;
+    while (!__all_sync(0xffffffffu, ready)) {
+        if (!ready) {
+            Body x;
+            x.load(VT + (size_t)EB * i);
+            ready = x.has((unsigned)pass * (ni + 1u) + ni);
+            for (int u = q; u < e && ready; ++u) {
+                const unsigned nu = (unsigned)__popcll(w.fl_mask[vbase + u]);
+                x.load(VT + (size_t)EB * (vbase + u));
+                ready = x.has((unsigned)pass * (nu + 1u) + nu);
+            }
+        }
+        if ((++bound.spins & 63u) == 0u && !__all_sync(0xffffffffu, bound.look(ctrl) && !flow_ld(&sh.dead))) {
+            *(volatile int*)&sh.dead = 1;
+            return false;
+        }
+    }
+    if (lead) {
+        Body x;
+        T4 v, o, a, b, s0 = V0[RW * q], o0 = s0;
+        x.load(VT + (size_t)EB * i);
+        x.unpack(v, o);
+        v.x = s0.x + (v.x - s0.x); v.y = s0.y + (v.y - s0.y); v.z = s0.z + (v.z - s0.z);
+        if constexpr (DIM == 3) {
+            o0 = V0[RW * q + 1];
+            o.x = o0.x + (o.x - o0.x); o.y = o0.y + (o.y - o0.y); o.z = o0.z + (o.z - o0.z);
+        }
+        for (int u = q; u < e; ++u) {
+            x.load(VT + (size_t)EB * (vbase + u));
+            x.unpack(a, b);
+            v.x = v.x + (a.x - s0.x); v.y = v.y + (a.y - s0.y); v.z = v.z + (a.z - s0.z);
+            if constexpr (DIM == 3) {
+                o.x = o.x + (b.x - o0.x); o.y = o.y + (b.y - o0.y); o.z = o.z + (b.z - o0.z);
+            }
+        }
+        V0[RW * q] = v;
+        if constexpr (DIM == 3) V0[RW * q + 1] = o;
+        x.pack(v, o, (unsigned)(pass + 1) * (ni + 1u));
+        x.store(VT + (size_t)EB * i);
+        for (int u = q; u < e; ++u) {
+            x.pack(v, o, (unsigned)(pass + 1) * ((unsigned)__popcll(w.fl_mask[vbase + u]) + 1u));
+            x.store(VT + (size_t)EB * (vbase + u));
+        }
+    }
+    __syncwarp();
+    return true;
+}
+
 // The solve of nc contacts by a team of blocks: K colours, colour k at the
 // colour-order positions [sh.lo[k], sh.end[k]) (narrowed to this block's), on
 // the particles body0 .. body1 - 1 (and the force-controlled walls).  Leaves
 // the velocities in w.V, the impulses in colour order (c_P) or key order (Pk),
 // the sweeps and the test in sh.  False when a wait gave up.
-template <int DIM, typename T, bool BATCH>
+//
+// VIEWS: the domain-wise update (Sec. 3.1).  Contacts work on the velocity
+// records of their domain (c_vab); after a pass's contacts one lane for each
+// particle with several records adds up their changes and stores the sum to
+// all of them, one more update of each: the sums are a colour after the last.
+// (A barrier after each colour and after the sums took 28.9 ms for a step of
+// 20,000 discs in 4 x 4 domains at FP64, this 13.2.)
+template <int DIM, typename T, bool BATCH, bool VIEWS>
 __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, FlowShared& sh, char* s_rec, int rec_cap,
                                            const FlowTeam& tm, int K, int nc, T mu, int body0, int body1, int crit,
                                            double alpha, int max_sweeps)
@@ -465,18 +553,22 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
     T4* V = (T4*)w.V;
     T4* Vprev = (T4*)w.fl_Vprev;
     constexpr int RW = (DIM == 2) ? 1 : 2;
+    const int nprev = g.n + 6;                        // records in Vprev (a view is taken back with its particle)
+    const int nview = VIEWS ? w.view_off[g.n] : 0;    // records of the domains past the particles' own
+    const int vbase = cd_view_base(g);
+    const int KX = VIEWS ? K + 1 : K;
 
     // this block's positions of each colour, and their warp items
     if (threadIdx.x < 32) {
         int run = 0, srun = 0;
-        for (int k0 = 0; k0 < K; k0 += 32) {
+        for (int k0 = 0; k0 < KX; k0 += 32) {
             const int k = k0 + lane;
             int m = 0, c = 0;
-            if (k < K) {
+            if (k < KX) {
                 // whole warp items, dealt so that the blocks' totals over the colours
                 // are even: colour k's remainder starts at another block
-                const int lo = sh.lo[k], hi = sh.end[k];
-                const int half = F64_2D && hi - lo <= FLOW_SPLIT * nb;
+                const int lo = k < K ? sh.lo[k] : 0, hi = k < K ? sh.end[k] : nview;
+                const int half = F64_2D && k < K && hi - lo <= FLOW_SPLIT * nb;
                 const int sh_item = half ? 4 : 5;
                 const long long items = (hi - lo + (1 << sh_item) - 1) >> sh_item;
                 const int r = (int)(((long long)k * 5 * nb >> 3) % nb);
@@ -484,7 +576,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                 sh.lo[k] = min(lo + (i0 << sh_item), hi);
                 sh.end[k] = min(lo + (i1 << sh_item), hi);
                 sh.half[k] = half;
-                c = sh.end[k] - sh.lo[k];
+                c = k < K ? sh.end[k] - sh.lo[k] : 0;
                 m = i1 - i0;
             }
             int incl = m, ci = c;
@@ -493,7 +585,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                 const int y = __shfl_up_sync(0xffffffffu, incl, o), z = __shfl_up_sync(0xffffffffu, ci, o);
                 if (lane >= o) { incl += y; ci += z; }
             }
-            if (k < K) { sh.base[k + 1] = run + incl; sh.slot[k + 1] = srun + ci; }
+            if (k < KX) { sh.base[k + 1] = run + incl; sh.slot[k + 1] = srun + ci; }
             run += __shfl_sync(0xffffffffu, incl, 31);
             srun += __shfl_sync(0xffffffffu, ci, 31);
         }
@@ -502,12 +594,12 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
         if (lane == 0) {
             for (int u = 0; u < FLOW_SLOTS; ++u) sh.arrived[u] = 0;
             int prev = -1;
-            for (int k = 0; k < K; ++k) {
+            for (int k = 0; k < KX; ++k) {
                 sh.before[k] = prev;
                 sh.done[k] = 0;
                 if (sh.base[k + 1] > sh.base[k]) prev = k;
             }
-            for (int k = 0; k < K && sh.before[k] < 0; ++k) sh.before[k] = -1 - prev;
+            for (int k = 0; k < KX && sh.before[k] < 0; ++k) sh.before[k] = -1 - prev;
             sh.decided = -1;
             sh.stop = (nc == 0) ? 0 : -1;
             sh.dead = 0;
@@ -525,17 +617,31 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
         x.pack(V[RW * i], o, 0u);
         x.store(VT + (size_t)EB * i);
     }
+    if constexpr (VIEWS) {
+        T4* V0 = (T4*)w.V0;   // the pass start of each particle with views, by its first view
+        for (int q = tid; q < nview; q += stride) {
+            const int i = w.view_owner[q];
+            Body x;
+            T4 o;
+            o.x = o.y = o.z = o.w = (T)0;
+            if constexpr (DIM == 3) { o = V[RW * i + 1]; V0[RW * q + 1] = o; }
+            const T4 v = V[RW * i];
+            V0[RW * q] = v;
+            x.pack(v, o, 0u);
+            x.store(VT + (size_t)EB * (vbase + q));
+        }
+    }
     if (threadIdx.x < FLOW_ROWS) flow_sum_store(part + threadIdx.x * gridDim.x + blockIdx.x, 0.0, 0u);
     __syncthreads();
-    const int Q = sh.base[K];
+    const int Q = sh.base[KX];
     const bool res = sh.slot[K] <= rec_cap;   // the block's records fit its shared memory
     Records rec(s_rec, rec_cap);
     // the colours each body has
     for (int k = 0; k < K; ++k)
         for (int p = sh.lo[k] + (int)threadIdx.x; p < sh.end[k]; p += blockDim.x) {
-            const int2 ab = w.c_ab[p];
+            const int2 ab = VIEWS ? w.c_vab[p] : w.c_ab[p];   // (a wall's place in c_vab is its own)
             atomicOr(&w.fl_mask[ab.x], 1ULL << k);
-            if (cd_is_body(g, ab.y)) atomicOr(&w.fl_mask[ab.y], 1ULL << k);
+            if (flow_moves<VIEWS>(g, ab.y)) atomicOr(&w.fl_mask[ab.y], 1ULL << k);
         }
     if (!tm.sync(ctrl)) return false;
     // a contact's place among each body's contacts and their number (8 bits
@@ -544,10 +650,16 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
         for (int p = sh.lo[k] + (int)threadIdx.x; p < sh.end[k]; p += blockDim.x) {
             Rec<DIM, T> r;
             r.ab = w.c_ab[p];
+            const int2 rr = VIEWS ? w.c_vab[p] : r.ab;   // the bodies' records
             const u64 below = (1ULL << k) - 1ULL;
-            const u64 ma = w.fl_mask[r.ab.x], mb = cd_is_body(g, r.ab.y) ? w.fl_mask[r.ab.y] : 0ULL;
-            const unsigned ord = (unsigned)__popcll(ma & below) | ((unsigned)__popcll(ma) << 8) |
-                                 ((unsigned)__popcll(mb & below) << 16) | ((unsigned)__popcll(mb) << 24);
+            const u64 ma = w.fl_mask[rr.x], mb = flow_moves<VIEWS>(g, rr.y) ? w.fl_mask[rr.y] : 0ULL;
+            unsigned na = (unsigned)__popcll(ma), nbd = (unsigned)__popcll(mb);
+            if constexpr (VIEWS) {   // the sum is an update too
+                na += flow_shared(w, vbase, g.n, rr.x);
+                if (mb) nbd += flow_shared(w, vbase, g.n, rr.y);
+            }
+            const unsigned ord = (unsigned)__popcll(ma & below) | (na << 8) | ((unsigned)__popcll(mb & below) << 16) |
+                                 (nbd << 24);
             if (res) {
                 const int i = sh.slot[k] + p - sh.lo[k];
                 load_static<DIM, T>(g, w, r);
@@ -558,7 +670,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                 rec.geo[i] = ((const T4*)w.c_geo)[p];
                 rec.m[i] = ((const TM*)w.c_m)[p];
                 rec.P[i] = ((const TP*)w.c_P)[p];
-                rec.ab[i] = r.ab;
+                rec.ab[i] = rr;
                 rec.ord[i] = ord;
             } else {
                 w.fl_ord[p] = ord;
@@ -601,7 +713,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
             const TP* Pin = (const TP*)flow_impulses(w, apply_only ? 0 : pass - 1);
             TP* Pout = (TP*)flow_impulses(w, pass);
             const bool save = pass >= FLOW_LAG1;
-            T4* Vsave = Vprev + (size_t)(pass & 1) * RW * (g.n + 6);
+            T4* Vsave = Vprev + (size_t)(pass & 1) * RW * nprev;
             double acc = 0.0;
             bool owed = false;
             bool dead = false;
@@ -622,6 +734,16 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                 const bool split = F64_2D && sh.half[k];
                 const int at = split ? 16 * (q - sh.base[k]) + (lane >> 1) : 32 * (q - sh.base[k]) + lane;
                 const bool act = at < cnt;
+                if constexpr (VIEWS) {
+                    if (k == K) {
+                        if (!flow_sum_views<DIM, T>(g, w, ctrl, sh, VT, vbase, first + at, act, pass)) { dead = true; break; }
+                        if (gate) {
+                            __syncwarp();
+                            if (lane == 0) atomicAdd(&sh.done[k], 1);
+                        }
+                        continue;
+                    }
+                }
                 const int p = first + at, i = sh.slot[k] + at;
                 Rec<DIM, T> r;
                 u64 *pa = nullptr, *pb = nullptr;
@@ -630,13 +752,13 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                 Body A, B;
                 if (act) {
                     if (res) {
-                        r.ab = rec.ab[i];
+                        r.ab = rec.ab[i];   // (the records)
                         ord = rec.ord[i];
                     } else {
-                        r.ab = w.c_ab[p];
+                        r.ab = VIEWS ? w.c_vab[p] : w.c_ab[p];
                         ord = w.fl_ord[p];
                     }
-                    wall = !cd_is_body(g, r.ab.y);
+                    wall = !flow_moves<VIEWS>(g, r.ab.y);
                     ta = (unsigned)pass * ((ord >> 8) & 255u) + (ord & 255u);
                     tb = (unsigned)pass * (ord >> 24) + ((ord >> 16) & 255u);
                     pa = VT + (size_t)EB * r.ab.x;
@@ -655,7 +777,14 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                         m = rec.m[i];
                         r.P = rec.P[i];
                     } else {
-                        load_static<DIM, T>(g, w, r);
+                        if constexpr (VIEWS) {
+                            const int2 rr = r.ab;
+                            r.ab = w.c_ab[p];
+                            load_static<DIM, T>(g, w, r);
+                            r.ab = rr;
+                        } else {
+                            load_static<DIM, T>(g, w, r);
+                        }
                         r.geo = ((const T4*)w.c_geo)[p];
                         m = ((const TM*)w.c_m)[p];
                         r.P = Pin[p];
@@ -704,7 +833,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                             vb = va;
                         }
                         T4 v1;
-                        const double Pnew = half.update(odd, r, va, vb, wall ? -1 : r.ab.y - g.n, apply_only, v1);
+                        const double Pnew = half.update(odd, r, va, vb, (wall || VIEWS) ? -1 : r.ab.y - g.n, apply_only, v1);
                         if (act && !(odd && wall)) {
                             A.pack(v1, v1, (odd ? tb : ta) + 1u);
                             A.store(odd ? pb : pa);
@@ -716,7 +845,8 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                             }
                             // the records of the pass start, for taking the sweep back
                             const int mine = odd ? (int)((ord >> 16) & 255u) : (int)(ord & 255u);
-                            if (save && mine == 0 && !(odd && wall)) Vsave[odd ? r.ab.y : r.ab.x] = odd ? vb : va;
+                            const int body = odd ? r.ab.y : r.ab.x;
+                            if (save && mine == 0 && !(odd && wall) && (!VIEWS || body < nprev)) Vsave[body] = odd ? vb : va;
                         }
                         settle();
                         const double Pother = shfl_pair(Pnew);
@@ -734,11 +864,11 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                     else if constexpr (DIM == 2) wall_vel2<T>(g, w, r.ab.y, vb);
                     else wall_vel3<T>(g, w, r.ab.y, vb, ob);
                     if (save) {
-                        if ((ord & 255u) == 0u) {
+                        if ((ord & 255u) == 0u && (!VIEWS || r.ab.x < nprev)) {
                             Vsave[RW * r.ab.x] = va;
                             if constexpr (DIM == 3) Vsave[RW * r.ab.x + 1] = oa;
                         }
-                        if (!wall && ((ord >> 16) & 255u) == 0u) {
+                        if (!wall && ((ord >> 16) & 255u) == 0u && (!VIEWS || r.ab.y < nprev)) {
                             Vsave[RW * r.ab.y] = vb;
                             if constexpr (DIM == 3) Vsave[RW * r.ab.y + 1] = ob;
                         }
@@ -747,13 +877,13 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                     UpdOut o;
                     if constexpr (DIM == 2) {
                         o = core2d<T, true>(g, r, va, vb, wall, apply_only, crit, alpha, 0.0, Pn);
-                        if (!wall && r.ab.y >= g.n) {
+                        if (!VIEWS && !wall && r.ab.y >= g.n) {
                             if (((r.ab.y - g.n) >> 1) == 0) vb.y = (T)0; else vb.x = (T)0;
                             vb.z = (T)0;
                         }
                     } else {
                         o = core3d<T, DEFER>(g, r, va, oa, vb, ob, wall, apply_only, crit, alpha, 0.0, Pn);
-                        if (!wall && r.ab.y >= g.n) {
+                        if (!VIEWS && !wall && r.ab.y >= g.n) {
                             const int ax = (r.ab.y - g.n) >> 1;
                             if (ax != 0) vb.x = (T)0;
                             if (ax != 1) vb.y = (T)0;
@@ -823,7 +953,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
         if (!cd_is_body(g, i)) continue;
         T4 v, o;
         if (back && w.fl_mask[i] != 0ULL) {
-            const T4* Vsave = Vprev + (size_t)((sweeps + 1) & 1) * RW * (g.n + 6);
+            const T4* Vsave = Vprev + (size_t)((sweeps + 1) & 1) * RW * nprev;
             v = Vsave[RW * i];
             v.w = (T)0;
             if constexpr (DIM == 3) o = Vsave[RW * i + 1];
@@ -839,7 +969,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
 }
 
 // A plain system: the whole grid is one team.
-template <int DIM, typename T>
+template <int DIM, typename T, bool VIEWS>
 __global__ void __launch_bounds__(FLOW_THREADS, 1)
 k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
 {
@@ -856,7 +986,7 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
         sh.end[k] = w.colour_off[k + 1];
     }
     __syncthreads();
-    if (!flow_solve<DIM, T, false>(g, w, sh, s_rec, rec_cap, tm, K, nc, (T)g.mu, 0, g.n + (g.dyn_walls ? 6 : 0), crit,
+    if (!flow_solve<DIM, T, false, VIEWS>(g, w, sh, s_rec, rec_cap, tm, K, nc, (T)g.mu, 0, g.n + (g.dyn_walls ? 6 : 0), crit,
                                    alpha, max_sweeps))
         return;
     u64 epoch = 0;
@@ -1017,7 +1147,7 @@ k_flow_batch(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec
             sh.end[k] = flow_lower(w, lo, w.colour_off[k + 1], first + count);
         }
         __syncthreads();
-        if (!flow_solve<DIM, T, true>(g, w, sh, s_rec, rec_cap, tm, K, nc, (T)w.pk[b].mu, first, first + count, crit,
+        if (!flow_solve<DIM, T, true, false>(g, w, sh, s_rec, rec_cap, tm, K, nc, (T)w.pk[b].mu, first, first + count, crit,
                                       alpha, max_sweeps))
             return;
         if (tm.blk == 0) {
@@ -1087,24 +1217,31 @@ __global__ void k_flow_totals(CdGeom g, CdWork w)
     }
 }
 
+enum { FLOW_PLAIN = 0, FLOW_BATCH, FLOW_VIEWS };
 struct FlowKernel { const void* fn; int body_bytes, record_bytes; };
-static FlowKernel flow_kernel(int dim, int precision, int batch)
+static FlowKernel flow_kernel(int dim, int precision, int kind)
 {
 #define FLOW_K(D, T) \
-    FlowKernel{batch ? (const void*)k_flow_batch<D, T> : (const void*)k_flow<D, T>, (int)sizeof(FlowBody<D, T>), \
-               FlowRecords<D, T>::BYTES}
+    FlowKernel{kind == FLOW_BATCH ? (const void*)k_flow_batch<D, T> \
+               : kind == FLOW_VIEWS ? (const void*)k_flow<D, T, true> : (const void*)k_flow<D, T, false>, \
+               (int)sizeof(FlowBody<D, T>), FlowRecords<D, T>::BYTES}
     if (dim == 2) return precision == CD_FP64 ? FLOW_K(2, double) : FLOW_K(2, float);
     return precision == CD_FP64 ? FLOW_K(3, double) : FLOW_K(3, float);
 #undef FLOW_K
 }
 
-size_t cd_flow_body_bytes(int dim, int precision) { return (size_t)flow_kernel(dim, precision, 0).body_bytes; }
+size_t cd_flow_body_bytes(int dim, int precision) { return (size_t)flow_kernel(dim, precision, FLOW_PLAIN).body_bytes; }
+
+static int flow_kind(const CdGeom& g)
+{
+    return g.npk > 1 ? FLOW_BATCH : g.ndom_total > 1 ? FLOW_VIEWS : FLOW_PLAIN;
+}
 
 // Contacts a block keeps in shared memory (a multiple of 16, so that every
 // array of the records stays aligned), or -1 if the kernel does not fit.
-int cd_flow_records(int dim, int precision, int batch, int device)
+int cd_flow_records(const CdGeom& g, int precision, int device)
 {
-    const FlowKernel f = flow_kernel(dim, precision, batch);
+    const FlowKernel f = flow_kernel(g.dim, precision, flow_kind(g));
     int most = 0;
     cudaFuncAttributes a;
     if (cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
@@ -1121,13 +1258,13 @@ int cd_flow_records(int dim, int precision, int batch, int device)
     return recs;
 }
 
-static cudaError_t flow_launch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int batch,
-                               int criterion, double alpha, int max_sweeps, cudaStream_t s, int* nl)
+static cudaError_t flow_launch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int criterion,
+                               double alpha, int max_sweeps, cudaStream_t s, int* nl)
 {
     cudaError_t e = cudaMemsetAsync(w.ctrl, 0, 2 * sizeof(u64), s);
     if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(w.fl_mask, 0, sizeof(u64) * (size_t)(g.n + 6), s)) != cudaSuccess) return e;
-    const FlowKernel f = flow_kernel(g.dim, precision, batch);
+    if ((e = cudaMemsetAsync(w.fl_mask, 0, sizeof(u64) * (size_t)w.fl_nrec, s)) != cudaSuccess) return e;
+    const FlowKernel f = flow_kernel(g.dim, precision, flow_kind(g));
     CdGeom ga = g;
     CdWork wa = w;
     int crit = criterion, ms = max_sweeps, rc = records;
@@ -1141,7 +1278,7 @@ static cudaError_t flow_launch(const CdGeom& g, const CdWork& w, int blocks, int
 cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int criterion,
                            double alpha, int max_sweeps, cudaStream_t s, int* nl)
 {
-    return flow_launch(g, w, blocks, records, precision, 0, criterion, alpha, max_sweeps, s, nl);
+    return flow_launch(g, w, blocks, records, precision, criterion, alpha, max_sweeps, s, nl);
 }
 
 cudaError_t cd_launch_flow_batch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision,
@@ -1149,7 +1286,7 @@ cudaError_t cd_launch_flow_batch(const CdGeom& g, const CdWork& w, int blocks, i
 {
     k_flow_plan<<<1, 512, 0, s>>>(g, w, blocks, records);
     ++*nl;
-    cudaError_t e = flow_launch(g, w, blocks, records, precision, 1, criterion, alpha, max_sweeps, s, nl);
+    cudaError_t e = flow_launch(g, w, blocks, records, precision, criterion, alpha, max_sweeps, s, nl);
     if (e != cudaSuccess) return e;
     k_flow_totals<<<1, 256, 0, s>>>(g, w);
     ++*nl;

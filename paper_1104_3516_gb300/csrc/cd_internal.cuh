@@ -189,8 +189,9 @@ struct CdWork {
     int* prep_tot;      // 4 values per block
     int* prep_hist;     // CD_KMAX x blocks: contacts of each colour in each block's range
     // dataflow solve (cd_flow.cu)
-    void* fl_V;         // n + 6 tagged velocity records
-    unsigned long long* fl_mask; // n + 6: colours of each body's contacts
+    int fl_nrec;        // velocity records: n + 6, and the domains' views
+    void* fl_V;         // fl_nrec tagged velocity records
+    unsigned long long* fl_mask; // fl_nrec: colours of each record's contacts
     unsigned* fl_ord;   // cap (colour order): place of the contact among its bodies' contacts
     void* fl_part;      // 4 G tagged block sums
     void* fl_P;         // cap: impulses after the sweeps s with s % 3 = 1 (c_P: 0)
@@ -544,7 +545,7 @@ cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, int blocks, int rec
 cudaError_t cd_launch_flow_batch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision,
                                  int criterion, double alpha, int max_sweeps, cudaStream_t stream, int* nl);
 size_t cd_flow_body_bytes(int dim, int precision);
-int cd_flow_records(int dim, int precision, int batch, int device);
+int cd_flow_records(const CdGeom& g, int precision, int device);
 int cd_sweep_fits(const CdGeom& g, int precision, int threads, int per_sm);
 cudaError_t cd_launch_unpack(const CdGeom& g, const CdWork& w, double* pos, double* vel, double* omega,
                              double* theta, int integrate, int precision, cudaStream_t stream, int* nl);

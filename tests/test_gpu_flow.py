@@ -131,3 +131,35 @@ def test_residual_magnitudes_match_64_bits():
         P = g.contacts()["impulse"].astype(np.longdouble)
         exact = np.sqrt((P * P).sum(1)).mean()
         assert abs(np.longdouble(r) - exact) <= 2e-14 * exact
+
+
+# a particle with two records, corners with four (eight in 3D), and cuts so
+# fine that most particles have several
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("make,domains", [
+    (lambda: W.dense_biaxial_discs(seed=5, n=40), (2, 1, 1)),
+    (lambda: W.dense_biaxial_discs(seed=5, n=4999), (4, 2, 1)),
+    (lambda: W.dense_biaxial_discs(seed=5, n=20011), (70, 70, 1)),
+    (lambda: W.sphere_gas(seed=3, n=4000, floor=20.0, vsig=0.5), (3, 2, 5)),
+])
+def test_domains_are_bit_identical(make, domains, precision):
+    """The domain-wise update, also of short solves (a sweep's tests against
+    the ones started ahead: sweeps 1, 17 and 40), against the barrier schedule,
+    which another block shape keeps."""
+    wl = make()
+    for kw in (dict(criterion=-1, max_sweeps=1), dict(criterion=-1, max_sweeps=17), dict(alpha=1e-2, max_sweeps=400),
+               dict(alpha=1e-5, max_sweeps=40)):
+        kw.update(precision=precision, domains=domains, max_contacts=4 * wl.n + 64)
+        a = gpu_system(wl, sweep_threads=256, sweep_blocks_per_sm=2, **kw)
+        b = gpu_system(wl, **kw)
+        for _ in range(2):
+            x, y = a.step(1)["last"], b.step(1)["last"]
+            for k in ("sweeps", "converged", "n_contacts", "n_colours"):
+                assert x[k] == y[k], k
+            assert abs(x["r_avg"] - y["r_avg"]) <= 1e-13 * x["r_avg"]
+        ca, cb = a.contacts(), b.contacts()
+        for k in ("pairs", "colour", "impulse"):
+            assert np.array_equal(ca[k], cb[k]), k
+        xa, xb = a.state(), b.state()
+        for k in ("x", "v", "w"):
+            assert np.array_equal(xa[k], xb[k]), k
