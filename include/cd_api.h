@@ -442,6 +442,11 @@ cd_status cd_adjoint_step(cd_system* sys, const double* dL_dpos, const double* d
                           const double* dL_dwall_force_host, double* dL_dpos_prev, double* dL_dvel_prev,
                           double* dL_domega_prev, double alpha, int64_t max_sweeps, cd_adjoint_stats* out_host);
 
+/* A number that changes whenever the tape does (a step recorded, a step
+ * consumed, a checkpoint loaded, a workspace set): as long as it is the same, the
+ * recorded steps are. */
+cd_status cd_tape_mark(const cd_system* sys, int64_t* mark);
+
 /* Checkpoints of the full stepping state: positions, velocities, angular
  * velocities, orientations (if the system has them), wall planes, and the
  * contact set with its impulses (the warm start of the next step), so that

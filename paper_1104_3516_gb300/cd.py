@@ -176,6 +176,7 @@ SIGNATURES = [
                                              _P, C.POINTER(C.c_int64), _P]),
     ("cd_adjoint_step", C.c_int, [_P, _P, _P, _P, C.POINTER(C.c_double), _P, _P, _P, C.c_double, C.c_int64,
                                   C.POINTER(cd_adjoint_stats)]),
+    ("cd_tape_mark", C.c_int, [_P, C.POINTER(C.c_int64)]),
     ("cd_checkpoint_size", C.c_int, [_P, C.POINTER(C.c_size_t)]),
     ("cd_save_checkpoint", C.c_int, [_P, _P, C.c_size_t]),
     ("cd_load_checkpoint", C.c_int, [_P, _P, C.c_size_t]),
@@ -353,6 +354,12 @@ def cd_adjoint_step(sysptr, dL_dpos, dL_dvel, dL_domega, dL_dwall_force, out_pos
                                          int(max_sweeps), C.byref(st)),
            allow=(CD_OK, CD_ERR_NOT_CONVERGED))
     return st.as_dict()
+
+
+def cd_tape_mark(sysptr) -> int:
+    m = C.c_int64()
+    _check(sysptr, lib().cd_tape_mark(sysptr, C.byref(m)))
+    return int(m.value)
 
 
 def cd_checkpoint_size(sysptr) -> int:
@@ -555,6 +562,10 @@ class CDSystem:
                 for t in (dL_dpos, dL_dvel, dL_domega)]
         st = cd_adjoint_step(self._h, *args, dL_dwall_force, gx, gv, gw, alpha, max_sweeps)
         return gx, gv, gw, st
+
+    def tape_mark(self) -> int:
+        """Changes whenever the recorded steps do."""
+        return cd_tape_mark(self._h)
 
     def new_checkpoint(self) -> torch.Tensor:
         """A device buffer (256-byte aligned view) for save/load_checkpoint."""

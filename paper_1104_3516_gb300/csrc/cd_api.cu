@@ -43,6 +43,7 @@ struct cd_system {
     int graph_launches;                // kernels in the captured step
     int tape_head;                     // next tape slot a step records into
     int tape_count;                    // recorded steps not yet consumed by cd_adjoint_step
+    int64_t tape_mark;                 // changes of the tape so far
     int adj_blocks;                    // cooperative grid of the adjoint kernel
     // params.merge_last_colour 4: sweeps + 1 of the last solve as last read
     // back (0: none yet), valid while no solve has been launched since; lets
@@ -785,6 +786,7 @@ extern "C" cd_status cd_set_workspace(cd_system* s, void* dev_ptr, size_t bytes)
     s->has_contacts = 0;
     s->tape_head = 0;
     s->tape_count = 0;
+    ++s->tape_mark;
     if (s->step_graph) {
         cudaGraphExecDestroy(s->step_graph);
         s->step_graph = nullptr;
@@ -912,6 +914,7 @@ extern "C" cd_status cd_step(cd_system* s, int64_t n_steps, cd_step_stats* out)
             const int T = (int)s->p.tape_steps;
             s->tape_head = (s->tape_head + 1) % T;
             if (s->tape_count < T) ++s->tape_count;
+            ++s->tape_mark;
         }
     }
     if (n_steps > 0) s->has_contacts = 1;
@@ -1096,6 +1099,7 @@ extern "C" cd_status cd_adjoint_step(cd_system* s, const double* dL_dpos, const 
     if ((st = ctrl_status(s, h)) != CD_OK) return st;
     s->tape_head = slot;
     --s->tape_count;
+    ++s->tape_mark;
     CD_CUDA(s, cd_launch_set_tape_slot(s->w, slot, s->stream, &s->launches));
     if (out_host) {
         out_host->sweeps = h.adj_sweeps;
@@ -1112,6 +1116,13 @@ extern "C" cd_status cd_adjoint_step(cd_system* s, const double* dL_dpos, const 
         out_host->diverged = h.adj_diverged;
     }
     return h.adj_converged ? CD_OK : CD_ERR_NOT_CONVERGED;
+}
+
+extern "C" cd_status cd_tape_mark(const cd_system* s, int64_t* mark)
+{
+    if (!s || !mark) return CD_ERR_INVALID_ARG;
+    *mark = s->tape_mark;
+    return CD_OK;
 }
 
 // Checkpoint sections, each 256-byte aligned: pos, vel, omega, theta (if
@@ -1181,6 +1192,7 @@ static cd_status ckpt_copy(cd_system* s, void* buf, size_t bytes, bool save)
         s->has_contacts = 1;
         s->tape_head = 0;
         s->tape_count = 0;
+        ++s->tape_mark;
         if (s->p.tape_steps > 0) CD_CUDA(s, cd_launch_set_tape_slot(s->w, 0, s->stream, &s->launches));
     }
     return CD_OK;

@@ -255,6 +255,45 @@ def test_checkpointed_rollout_equals_the_full_tape():
         assert np.array_equal(np.asarray(a), np.asarray(b))
 
 
+@pytest.mark.parametrize("between", ["nothing", "step", "checkpoint", "adjoint", "workspace", "other_rollout"])
+def test_backward_uses_the_tape_only_as_the_forward_left_it(between):
+    """Gradients are the same, bit for bit, whether the last segment is read
+    from the tape or stepped again: calls that change the tape between forward
+    and backward, and a second backward pass."""
+    import torch
+    from paper_1104_3516_gb300 import autodiff, cd
+    wl = colliding_gas(n=100, phi=0.62, vsig=3.0, dt=0.02)
+    g = cd.CDSystem(wl, device="cuda:0", criterion=cd.CD_CONV_GLOBAL_REL, alpha=FWD_ALPHA, max_sweeps=MAX_SWEEPS,
+                    tape_steps=4)
+    mu = torch.tensor(wl.mu, dtype=torch.float64, requires_grad=True)
+    start = g.save_checkpoint()   # no contacts: every rollout starts from the same (empty) warm start
+
+    def forward(steps=7):
+        g.load_checkpoint(start)
+        x, v, w = (torch.as_tensor(t, dtype=torch.float64, device="cuda:0").requires_grad_() for t in (wl.x, wl.v, wl.w))
+        xT, vT, wT, FT = autodiff.rollout(g, x, v, w, mu, steps, checkpoint_every=4, alpha=ADJ_ALPHA,
+                                          max_sweeps=MAX_SWEEPS)
+        return (x, v, w, mu), (xT[:, 1].sum() + (vT ** 2).sum() + wT.sum()).cpu() + FT[2] / 15.0
+
+    inputs, L = forward()
+    want = torch.autograd.grad(L, inputs)
+    inputs, L = forward()
+    if between == "step":
+        g.step(1)
+    elif between == "checkpoint":
+        g.load_checkpoint(g.save_checkpoint())
+    elif between == "adjoint":
+        g.adjoint_step(g.pos, g.vel, g.omega)
+    elif between == "workspace":
+        other = torch.empty(cd.cd_workspace_size(g.handle) + 256, dtype=torch.uint8, device="cuda:0")
+        cd.cd_set_workspace(g.handle, other[(-other.data_ptr()) % 256:])
+    elif between == "other_rollout":
+        forward(5)
+    for _ in range(2):
+        got = torch.autograd.grad(L, inputs, retain_graph=True)
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
 def test_gpu_adjoint_settling_10k_against_finite_differences():
     """The differentiated settling rollout at full size: 10,000 discs, 200
     steps, checkpoints every 20; L = floor pressure of the last step + the
