@@ -210,7 +210,7 @@ static size_t layout(cd_system* s, char* base, CdWork* w)
         t.fl_V = L.take<char>(base, fl ? nrec * cd_flow_body_bytes((int)s->p.dim, (int)s->p.precision) : 1);
         t.fl_mask = L.take<unsigned long long>(base, fl ? nrec : 1);
         t.fl_ord = L.take<unsigned>(base, fl ? cap : 1);
-        t.fl_part = L.take<char>(base, fl ? 64 * G : 1);
+        t.fl_part = L.take<char>(base, fl ? 128 * G : 1);
         t.fl_P = L.take<char>(base, fl ? cap * (s->p.dim == 2 ? 2 : 4) * real : 1);
         t.fl_P2 = L.take<char>(base, fl ? cap * (s->p.dim == 2 ? 2 : 4) * real : 1);
         t.fl_Vprev = L.take<char>(base, fl ? 2 * (n + 6) * vrec : 1);

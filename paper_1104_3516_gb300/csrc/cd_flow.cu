@@ -169,7 +169,8 @@ __device__ __forceinline__ double flow_sum_of(const u64 (&e)[2])
 #define FLOW_WORKERS 11                           // warps that update contacts
 #define FLOW_THREADS (32 * (FLOW_WORKERS + 1))    // and one that runs the convergence test
 #define FLOW_LEAST 112                            // contacts that a block of a batched system is given at least
-#define FLOW_ROWS 4                               // rows of tagged block sums
+#define FLOW_ROWS 8                               // rows of tagged block sums: while a block leaves those of pass p
+                                                  // another may still wait for those of p - 5
 #define FLOW_SLOTS 4                              // passes whose residual terms are kept
 #define FLOW_LAG1 16                              // from this pass on one starts before the test of the one before is
 #define FLOW_LAG2 32                              // known, from this one on two do: what they change can be taken back
@@ -271,53 +272,106 @@ __device__ __forceinline__ bool flow_wait(CdCtrl* ctrl, FlowShared& sh, const u6
 
 __device__ __forceinline__ double shfl_pair(double v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
 
-// The control warp's part of a pass: the block's sum, published, every block's
-// sums gathered, the test.  The sums of lanes, then of blocks, are taken in a
-// fixed order, the same in every block.  Returns false when a wait gave up.
-__device__ __forceinline__ bool flow_control(CdCtrl* ctrl, FlowShared& sh, FlowSum* part, const FlowTeam& tm, int pass,
-                                             int nc, int crit, double alpha, int max_sweeps, double& xprev)
+// The sum of N values >= 0 a lane over the warp (in every lane), exact but for
+// the rounding at the end: as integers of 128 bits that share the largest
+// exponent, added a lane and then by limbs of 25 bits.  The FP64 pipe takes 64
+// cycles an instruction, more while the workers use it; a pass's sums and test
+// took 9,000 cycles on it, longer than a pass of two colours (10,000 discs in
+// pyramids, 150 sweeps: 875 us, now 640).
+template <int N>
+__device__ __forceinline__ double flow_sum_warp(const double (&v)[N])
+{
+    typedef unsigned __int128 u128;
+    unsigned top = 0;
+#pragma unroll
+    for (int u = 0; u < N; ++u) top = max(top, (unsigned)((u64)__double_as_longlong(v[u]) >> 32));
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (top == 0u) top = __any_sync(0xffffffffu, [&]() { u64 o = 0; for (int u = 0; u < N; ++u) o |= (u64)__double_as_longlong(v[u]); return o != 0; }());
+    if (top == 0u) return 0.0;
+    const int em = (int)(top >> 20);
+    if (em < 128 || em > 2032) {   // near the ends of the range, infinite, NaN
+        double x = 0.0;
+        for (int u = 0; u < N; ++u) x += v[u];
+        return warp_sum(x);
+    }
+    u128 t = 0;   // bit 116: 2^(em - 1023)
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        const u64 b = (u64)__double_as_longlong(v[u]);
+        const int e = (int)(b >> 52), d = em - e;
+        const u64 m = (b & 0xfffffffffffffULL) | (1ULL << 52);
+        if (e > 0 && d < 117) t += ((u128)m << 64) >> d;
+    }
+    u128 s = 0;
+#pragma unroll
+    for (int q = 4; q >= 0; --q)
+        s = (s << 25) + __reduce_add_sync(0xffffffffu, (unsigned)(t >> (25 * q)) & 0x1ffffffu);
+    const u64 hi = (u64)(s >> 64);   // (not 0: the largest term's bit 52)
+    const int z = __clzll((long long)hi);
+    s <<= z;
+    const u64 m = (u64)(s >> 75) + ((u64)(s >> 74) & 1ULL);
+    return __longlong_as_double((long long)(((u64)(em + 11 - z - 1) << 52) + m));
+}
+
+// The control warp's state: the next pass whose block sum it leaves, and the
+// next one whose test it decides.
+struct FlowControl {
+    int pub = 0, dec = 0;
+    double xprev = 0.0;
+};
+
+// The control warp: leaves the block's sum of a pass when the workers have
+// finished it, and decides the test of the first undecided pass when every
+// block's sum is there (whichever comes first: neither waits for the other).
+// Returns after a decision; false when a wait gave up.  The sums are exact, so
+// the same in every block.
+__device__ __forceinline__ bool flow_control(CdCtrl* ctrl, FlowShared& sh, FlowSum* part, const FlowTeam& tm,
+                                             FlowControl& fc, int nc, int crit, double alpha, int max_sweeps)
 {
     const int lane = threadIdx.x & 31;
-    bool on = true;
-    if (lane == 0) on = flow_wait_shared(ctrl, sh, &sh.arrived[pass % FLOW_SLOTS],
-                                          FLOW_WORKERS * (pass / FLOW_SLOTS + 1));
-    if (!__shfl_sync(0xffffffffu, (int)on, 0)) return false;
-    __syncwarp();
-    double x = 0.0;
-#pragma unroll
-    for (int u = 0; u < FLOW_WORKERS; ++u) {
-        const double y = *(volatile double*)&sh.acc[pass % FLOW_SLOTS][u][lane];
-        if (__any_sync(0xffffffffu, __double_as_longlong(y) != 0)) x += y;
-    }
-    x = warp_sum_nz(x);
     const int nb = tm.nb;
-    FlowSum* row = part + (size_t)(pass % FLOW_ROWS) * gridDim.x + tm.start;
-    const unsigned tag = (unsigned)pass + 1u;
-    if (lane == 0) flow_sum_store(row + tm.blk, x, tag);
-    x = 0.0;
     FlowBound bound;
-    for (int b0 = 0; b0 < nb; b0 += 160) {
-        // five blocks a lane at a time, their loads in flight together
-        u64 f[5][2];
-        bool have = false;
-        while (!__all_sync(0xffffffffu, have)) {
-            have = true;
+    double x = 0.0;
+    for (int b0 = 0; b0 < nb;) {
+        if (__all_sync(0xffffffffu, flow_ld(&sh.arrived[fc.pub % FLOW_SLOTS]) >= FLOW_WORKERS * (fc.pub / FLOW_SLOTS + 1))) {
+            __threadfence_block();
+            __syncwarp();
+            double v[FLOW_WORKERS];
+#pragma unroll
+            for (int u = 0; u < FLOW_WORKERS; ++u)
+                v[u] = *(volatile double*)&sh.acc[fc.pub % FLOW_SLOTS][u][lane];
+            const double y = flow_sum_warp(v);
+            if (lane == 0)
+                flow_sum_store(part + (size_t)(fc.pub % FLOW_ROWS) * gridDim.x + tm.start + tm.blk, y,
+                               (unsigned)fc.pub + 1u);
+            ++fc.pub;
+        }
+        if (fc.dec < fc.pub && (bound.spins & 3u) == 0u) {   // (looks take bandwidth from the workers')
+            // five blocks a lane at a time, their loads in flight together
+            const FlowSum* row = part + (size_t)(fc.dec % FLOW_ROWS) * gridDim.x + tm.start;
+            u64 f[5][2];
+            double v[5];
+            bool have = true;
 #pragma unroll
             for (int u = 0; u < 5; ++u) {
                 const int b = b0 + 32 * u + lane;
                 if (b < nb) flow_load(row[b].e, f[u]);
             }
 #pragma unroll
-            for (int u = 0; u < 5; ++u)
-                if (b0 + 32 * u + lane < nb) have = have && flow_sum_is(f[u], tag);
-            on = bound.go(ctrl) && !flow_ld(&sh.dead);
-            if (!__all_sync(0xffffffffu, on)) return false;
+            for (int u = 0; u < 5; ++u) {
+                const bool in = b0 + 32 * u + lane < nb;
+                have = have && (!in || flow_sum_is(f[u], (unsigned)fc.dec + 1u));
+                v[u] = in ? flow_sum_of(f[u]) : 0.0;
+            }
+            if (__all_sync(0xffffffffu, have)) {
+                const double y = flow_sum_warp(v);
+                x = b0 ? x + y : y;
+                b0 += 160;
+            }
         }
-#pragma unroll
-        for (int u = 0; u < 5; ++u)
-            if (b0 + 32 * u + lane < nb) x += flow_sum_of(f[u]);
+        if (!__all_sync(0xffffffffu, bound.go(ctrl) && !flow_ld(&sh.dead))) return false;
     }
-    x = warp_sum(x);
+    const int pass = fc.dec++;
     if (lane == 0) {
         // the ratio of the test against its threshold by products; only where
         // that is within rounding of the threshold (or at the end) the test
@@ -325,14 +379,14 @@ __device__ __forceinline__ bool flow_control(CdCtrl* ctrl, FlowShared& sh, FlowS
         bool end = pass >= max_sweeps;
         if (pass > 0 && crit != CD_CONV_NONE && !end) {
             const double a = (crit == CD_CONV_GLOBAL_SQ) ? sqrt(alpha) : alpha;
-            const double s = x + xprev, off = fabs(x - xprev) - a * s;
+            const double s = x + fc.xprev, off = fabs(x - fc.xprev) - a * s;
             end = !(off > s * (1e-15 * (1.0 + a)));
         }
         if (end) {
             const double ra = x / (double)nc;
             double rs = 0.0;
             int cv = 0;
-            if (pass > 0) global_test(ra, xprev / (double)nc, crit, alpha, rs, cv);
+            if (pass > 0) global_test(ra, fc.xprev / (double)nc, crit, alpha, rs, cv);
             *(volatile double*)&sh.ravg = ra;
             *(volatile double*)&sh.resid = rs;
             *(volatile int*)&sh.converged = cv;
@@ -340,8 +394,9 @@ __device__ __forceinline__ bool flow_control(CdCtrl* ctrl, FlowShared& sh, FlowS
         }
         __threadfence_block();
         *(volatile int*)&sh.decided = pass;
-        xprev = x;
     }
+    fc.xprev = x;
+    __syncwarp();
     return true;
 }
 
@@ -686,21 +741,20 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
     // 21.3 us), and with one item a warp there is no queue.
     const bool gate = sizeof(T) == 4 && Q > FLOW_WORKERS;
     if (nc > 0 && wid == FLOW_WORKERS) {
-        double xprev = 0.0;
-        for (int pass = 0; ; ++pass) {
-            if (!flow_control(ctrl, sh, part, tm, pass, nc, crit, alpha, max_sweeps, xprev)) {
+        FlowControl fc;
+        do {
+            if (!flow_control(ctrl, sh, part, tm, fc, nc, crit, alpha, max_sweeps)) {
                 *(volatile int*)&sh.dead = 1;
                 break;
             }
-            __syncwarp();
-            if (flow_ld(&sh.stop) >= 0) break;
-        }
+        } while (flow_ld(&sh.stop) < 0);
     } else if (nc > 0) {
         TP pend;   // impulse of the warp's last update whose magnitude is not summed yet
         for (int pass = 0; ; ++pass) {   // pass 0: the starting impulses; pass s: sweep s
             const bool apply_only = (pass == 0);
+            // (pass 0 has no test to wait for)
             const int known = pass - 1 - (pass >= FLOW_LAG1) - (pass >= FLOW_LAG2);
-            bool on = known < 0 || flow_wait_shared(ctrl, sh, &sh.decided, known);
+            bool on = known < 1 || flow_wait_shared(ctrl, sh, &sh.decided, known);
             on = on && pass <= max_sweeps && !flow_ld(&sh.dead);
             // (a stop after `known` is not looked at: every warp of the grid runs the same passes)
             if (on) {

@@ -193,7 +193,7 @@ struct CdWork {
     void* fl_V;         // fl_nrec tagged velocity records
     unsigned long long* fl_mask; // fl_nrec: colours of each record's contacts
     unsigned* fl_ord;   // cap (colour order): place of the contact among its bodies' contacts
-    void* fl_part;      // 4 G tagged block sums
+    void* fl_part;      // 8 G tagged block sums
     void* fl_P;         // cap: impulses after the sweeps s with s % 3 = 1 (c_P: 0)
     void* fl_P2;        // cap: ... = 2
     void* fl_Vprev;     // 2 (n + 6) velocity records from before the latest two sweeps
