@@ -22,7 +22,7 @@
 // so the sweeps begun past the last one are taken back.
 //
 // What bounds it: in FP64 the FP64 pipe (64 cycles a warp instruction on each
-// quarter of an SM, 24 of them a warp of contacts: ~3,200 cycles a colour of the
+// quarter of an SM, 25 of them a warp of contacts: ~3,200 cycles a colour of the
 // 100,000-disc pile) and then the way of the records to the next colour (~1,700)
 // in turn, since neighbouring blocks move in step; in FP32, and in small systems, the way of a record
 // from SM to SM (~500 cycles on a die, ~850 across) once per colour, plus the
@@ -438,15 +438,15 @@ struct FlowRecords {
 // velocities are there: between two FP64 instructions a select or a shuffle
 // costs ~44 cycles beyond their own 64 each.
 struct FlowHalf {
-    double c0, c1, c2, c3, c4, c5, Pold;
+    double c1, c2, c3, c4, c5, bias, Pold;
     __device__ __forceinline__ void choose(bool odd, const Rec<2, double>& r)
     {
         c1 = odd ? -r.geo.y : r.geo.x;
         c2 = odd ? r.geo.x : r.geo.y;
-        c0 = odd ? -0.0 : r.geo.z;   // (adding -0 to a product leaves it as it is)
-        c3 = odd ? -r.sa.y : 0.0;
+        c3 = odd ? -r.sa.y : 1.0;
         c4 = odd ? -r.sb.y : 0.0;
         c5 = odd ? -r.mt : -r.geo.w;
+        bias = r.geo.z;
         Pold = odd ? r.P.y : r.P.x;
     }
     // Returns this lane's impulse component, and in v1 the new velocity record
@@ -459,10 +459,10 @@ struct FlowHalf {
         const double xa = odd ? va.x : va.y, xb = odd ? vb.x : vb.y;
         double Pnew = Pold, d = Pold;
         if (!apply_only) {
-            const double u3 = odd ? va.z : 0.0, u4 = odd ? vb.z : 0.0;
+            const double u3 = odd ? va.z : bias, u4 = odd ? vb.z : 0.0;
             const double dvx = __dsub_rn(vb.x, va.x), dvy = __dsub_rn(vb.y, va.y);
-            double u = __fma_rn(dvy, c2, __fma_rn(dvx, c1, c0));  // b + u_n | (dv x n)
-            u = __fma_rn(c3, u3, u);                              //         | - r_a w_a
+            double u = __fma_rn(dvy, c2, __dmul_rn(dvx, c1));     // u_n     | (dv x n)
+            u = __fma_rn(c3, u3, u);                              // b + u_n | - r_a w_a
             u = __fma_rn(c4, u4, u);                              //         | - r_b w_b
             const double Ps = __fma_rn(c5, u, Pold);
             const double lim = pos_part(shfl_pair(__dmul_rn(r.mu, Ps)));   // mu max(P_n*, 0)

@@ -381,9 +381,10 @@ __device__ __forceinline__ UpdOut core2d(const CdGeom& g, const Rec<2, T>& r, ty
     } else {
         const T b = r.geo.z, mn = r.geo.w;
         const T dvx = sub_of<T>(vb.x, va.x), dvy = sub_of<T>(vb.y, va.y);
-        // b + u_n: in FP64 b enters the first of the fused steps (an instruction less)
-        const T bun = sizeof(T) == 8 ? fma_of<T>(dvy, ny, fma_of<T>(dvx, nx, b))
-                                     : add_of<T>(b, fma_of<T>(dvy, ny, mul_of<T>(dvx, nx)));
+        // (b in the first fused step would save an instruction, but a contact that
+        // carries rounding noise only, under a lid that hangs free for one, is then
+        // open where it was closed, and counts of contacts change)
+        const T bun = add_of<T>(b, fma_of<T>(dvy, ny, mul_of<T>(dvx, nx)));
         // u_t = (dv x n) - (r_a w_a + r_b w_b)
         T ut = fma_of<T>(dvy, nx, -mul_of<T>(dvx, ny));
         ut = fma_of<T>(-r.sa.y, va.z, ut);
