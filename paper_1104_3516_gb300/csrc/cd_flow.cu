@@ -572,6 +572,40 @@ __device__ __forceinline__ bool flow_sum_views(const CdGeom& g, const CdWork& w,
     return true;
 }
 
+// Contact r, open before the update, stays open.
+template <typename T>
+__device__ __forceinline__ bool flow_stays_open(const Rec<2, T>& r, const typename Vec<T>::V4& va,
+                                                const typename Vec<T>::V4&, const typename Vec<T>::V4& vb,
+                                                const typename Vec<T>::V4&)
+{
+    // (FP64 takes an undefined tangential impulse as 0)
+    if (sizeof(T) == 4 && !(tame<T>(exponent_of(va.z), exponent_of(r.sa.y)) &&
+                            tame<T>(exponent_of(vb.z), exponent_of(r.sb.y)))) return false;
+    return stays_open<T>(r.geo.w, gap_rate2d<T>(r.geo.x, r.geo.y, r.geo.z, sub_of<T>(vb.x, va.x),
+                                                sub_of<T>(vb.y, va.y)));
+}
+template <typename T>
+__device__ __forceinline__ bool flow_stays_open(const Rec<3, T>& r, const typename Vec<T>::V4& va,
+                                                const typename Vec<T>::V4& wa, const typename Vec<T>::V4& vb,
+                                                const typename Vec<T>::V4& wb)
+{
+    T gx, gy, gz;
+    const T un = contact_velocity3d<T>(r, va, wa, vb, wb, gx, gy, gz);
+    return tame<T>(max(max(exponent_of(gx), exponent_of(gy)), exponent_of(gz)), exponent_of(r.m.y)) &&
+           stays_open<T>(r.m.x, add_of<T>(r.geo.w, un));
+}
+
+__device__ __forceinline__ bool flow_zero(double2 P) { return ((__double_as_longlong(P.x) | __double_as_longlong(P.y)) << 1) == 0LL; }
+__device__ __forceinline__ bool flow_zero(float2 P) { return P.x == 0.0f && P.y == 0.0f; }
+template <typename V>
+__device__ __forceinline__ bool flow_zero(const V& P)
+{
+    if constexpr (sizeof(V) == 32)
+        return ((__double_as_longlong(P.x) | __double_as_longlong(P.y) | __double_as_longlong(P.z) |
+                 __double_as_longlong(P.w)) << 1) == 0LL;
+    else return P.x == 0.0f && P.y == 0.0f && P.z == 0.0f && P.w == 0.0f;
+}
+
 // The solve of nc contacts by a team of blocks: K colours, colour k at the
 // colour-order positions [sh.lo[k], sh.end[k]) (narrowed to this block's), on
 // the particles body0 .. body1 - 1 (and the force-controlled walls).  Leaves
@@ -848,6 +882,13 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                     r.pk = 0;
                     r.mu = mu;
                 }
+                // In a gas nearly every contact found is open and stays so (of a million
+                // spheres' 912,728, one in 2,000 is not): an item whose contacts all are
+                // takes the normal rate only, 23 of 79 FP64 instructions (2D: 6 of 25), and
+                // nothing in the starting pass.  (Not where pairs of lanes share contacts: there
+                // the votes in the chain cost more, 5,000 packed discs 19.9 -> 21.4 ms, than
+                // a thin gas gains.)
+                const bool shut = !split && __all_sync(0xffffffffu, !act || flow_zero(r.P));
                 FlowHalf half;
                 if constexpr (F64_2D) {
                     if (split) {
@@ -917,6 +958,9 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                     if (!wall) B.unpack(vb, ob);
                     else if constexpr (DIM == 2) wall_vel2<T>(g, w, r.ab.y, vb);
                     else wall_vel3<T>(g, w, r.ab.y, vb, ob);
+                }
+                const bool still = shut && (apply_only || __all_sync(0xffffffffu, !act || flow_stays_open<T>(r, va, oa, vb, ob)));
+                if (act) {
                     if (save) {
                         if ((ord & 255u) == 0u && (!VIEWS || r.ab.x < nprev)) {
                             Vsave[RW * r.ab.x] = va;
@@ -927,23 +971,19 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                             if constexpr (DIM == 3) Vsave[RW * r.ab.y + 1] = ob;
                         }
                     }
-                    TP Pn;
+                    TP Pn = r.P;
                     UpdOut o;
-                    if constexpr (DIM == 2) {
-                        o = core2d<T, true>(g, r, va, vb, wall, apply_only, crit, alpha, 0.0, Pn);
-                        if (!VIEWS && !wall && r.ab.y >= g.n) {
-                            if (((r.ab.y - g.n) >> 1) == 0) vb.y = (T)0; else vb.x = (T)0;
-                            vb.z = (T)0;
-                        }
-                    } else {
-                        o = core3d<T, DEFER>(g, r, va, oa, vb, ob, wall, apply_only, crit, alpha, 0.0, Pn);
-                        if (!VIEWS && !wall && r.ab.y >= g.n) {
-                            const int ax = (r.ab.y - g.n) >> 1;
-                            if (ax != 0) vb.x = (T)0;
-                            if (ax != 1) vb.y = (T)0;
-                            if (ax != 2) vb.z = (T)0;
-                            ob.x = ob.y = ob.z = (T)0;
-                        }
+                    o.pabs = 0.0;
+                    if (!still) {
+                        if constexpr (DIM == 2) o = core2d<T, true>(g, r, va, vb, wall, apply_only, crit, alpha, 0.0, Pn);
+                        else o = core3d<T, DEFER>(g, r, va, oa, vb, ob, wall, apply_only, crit, alpha, 0.0, Pn);
+                    }
+                    if (!VIEWS && !wall && r.ab.y >= g.n) {   // a force-controlled wall moves along its normal only
+                        const int ax = (r.ab.y - g.n) >> 1;
+                        if (ax != 0) vb.x = (T)0;
+                        if (ax != 1) vb.y = (T)0;
+                        if (DIM == 2 || ax != 2) vb.z = (T)0;
+                        if constexpr (DIM == 3) ob.x = ob.y = ob.z = (T)0;
                     }
                     A.pack(va, oa, ta + 1u);
                     A.store(pa);
@@ -958,7 +998,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                     settle();
                     if constexpr (DEFER) {
                         pend = Pn;
-                        owed = true;
+                        owed = !still;
                     } else {
                         acc += o.pabs;
                     }

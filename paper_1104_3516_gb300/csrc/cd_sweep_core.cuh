@@ -364,6 +364,37 @@ __device__ __forceinline__ double abs_of_pair(double pn, double pt)
     return __longlong_as_double((long long)(r + ((u64)(long long)(em - 1023) << 52)));
 }
 
+// 2D: b + u_n.  (b in the first fused step would save an instruction, but a
+// contact that carries rounding noise only, under a lid that hangs free for
+// one, is then open where it was closed, and counts of contacts change.)
+template <typename T>
+__device__ __forceinline__ T gap_rate2d(T nx, T ny, T b, T dvx, T dvy)
+{
+    return add_of<T>(b, fma_of<T>(dvy, ny, mul_of<T>(dvx, nx)));
+}
+
+// Biased exponent of x, and whether x y is finite by those of the two with room
+// for a few sums.
+__device__ __forceinline__ int exponent_of(double x) { return (int)(__double_as_longlong(x) >> 52) & 0x7ff; }
+__device__ __forceinline__ int exponent_of(float x) { return (__float_as_int(x) >> 23) & 0xff; }
+template <typename T>
+__device__ __forceinline__ bool tame(int ex, int ey)
+{
+    constexpr int top = sizeof(T) == 8 ? 0x7ff : 0xff;
+    return max(ex, ey) < top - 8 && ex + ey < top / 2 + top - 8;
+}
+
+// A contact that was open (P = 0) stays so: its new normal impulse is 0, by the
+// operations of the update.  (Where something is infinite or undefined, or
+// might be in the tangential part, the update itself has to tell.)
+template <typename T>
+__device__ __forceinline__ bool stays_open(T mn, T bun)
+{
+    const T Pn = pos_part(fma_of<T>(-mn, bun, (T)0));
+    if constexpr (sizeof(T) == 8) return exponent_of(bun) != 0x7ff && __double_as_longlong(Pn) == 0LL;   // (off the FP64 pipe)
+    else return exponent_of(bun) != 0xff && Pn == (T)0;
+}
+
 // 2D: P_n = max(0, P_n,old - m_n (b + u_n)); P_t = clamp(P_t,old - m_t u_t, +-mu P_n).
 template <typename T, bool SQ = false>
 __device__ __forceinline__ UpdOut core2d(const CdGeom& g, const Rec<2, T>& r, typename Vec<T>::V4& va,
@@ -381,10 +412,7 @@ __device__ __forceinline__ UpdOut core2d(const CdGeom& g, const Rec<2, T>& r, ty
     } else {
         const T b = r.geo.z, mn = r.geo.w;
         const T dvx = sub_of<T>(vb.x, va.x), dvy = sub_of<T>(vb.y, va.y);
-        // (b in the first fused step would save an instruction, but a contact that
-        // carries rounding noise only, under a lid that hangs free for one, is then
-        // open where it was closed, and counts of contacts change)
-        const T bun = add_of<T>(b, fma_of<T>(dvy, ny, mul_of<T>(dvx, nx)));
+        const T bun = gap_rate2d<T>(nx, ny, b, dvx, dvy);
         // u_t = (dv x n) - (r_a w_a + r_b w_b)
         T ut = fma_of<T>(dvy, nx, -mul_of<T>(dvx, ny));
         ut = fma_of<T>(-r.sa.y, va.z, ut);
@@ -507,6 +535,23 @@ __device__ __forceinline__ UpdOut apply2d(const CdGeom& g, const CdWork& w, int 
     return o;
 }
 
+// 3D: relative velocity of the contact points, (vb - va) - (ra wa + rb wb) x n;
+// returns its normal part.
+template <typename T>
+__device__ __forceinline__ T contact_velocity3d(const Rec<3, T>& r, const typename Vec<T>::V4& va,
+                                                const typename Vec<T>::V4& wa, const typename Vec<T>::V4& vb,
+                                                const typename Vec<T>::V4& wb, T& gx, T& gy, T& gz)
+{
+    const T nx = r.geo.x, ny = r.geo.y, nz = r.geo.z;
+    const T lx = fma_of<T>(r.sb.y, wb.x, mul_of<T>(r.sa.y, wa.x));
+    const T ly = fma_of<T>(r.sb.y, wb.y, mul_of<T>(r.sa.y, wa.y));
+    const T lz = fma_of<T>(r.sb.y, wb.z, mul_of<T>(r.sa.y, wa.z));
+    gx = sub_of<T>(sub_of<T>(vb.x, va.x), fma_of<T>(ly, nz, -mul_of<T>(lz, ny)));
+    gy = sub_of<T>(sub_of<T>(vb.y, va.y), fma_of<T>(lz, nx, -mul_of<T>(lx, nz)));
+    gz = sub_of<T>(sub_of<T>(vb.z, va.z), fma_of<T>(lx, ny, -mul_of<T>(ly, nx)));
+    return fma_of<T>(gz, nz, fma_of<T>(gy, ny, mul_of<T>(gx, nx)));
+}
+
 // 3D: the same with the tangential impulse a vector, scaled onto the cone.
 template <typename T, bool SQ = false>
 __device__ __forceinline__ UpdOut core3d(const CdGeom& g, const Rec<3, T>& r, typename Vec<T>::V4& va,
@@ -522,14 +567,8 @@ __device__ __forceinline__ UpdOut core3d(const CdGeom& g, const Rec<3, T>& r, ty
         dPn = Pn; dtx = Ptx; dty = Pty; dtz = Ptz;
     } else {
         const T mn = r.m.x, mt = r.m.y, b = r.geo.w;
-        // relative velocity of the contact points: (vb - va) - (ra wa + rb wb) x n
-        const T lx = fma_of<T>(r.sb.y, wb.x, mul_of<T>(r.sa.y, wa.x));
-        const T ly = fma_of<T>(r.sb.y, wb.y, mul_of<T>(r.sa.y, wa.y));
-        const T lz = fma_of<T>(r.sb.y, wb.z, mul_of<T>(r.sa.y, wa.z));
-        const T gx = sub_of<T>(sub_of<T>(vb.x, va.x), fma_of<T>(ly, nz, -mul_of<T>(lz, ny)));
-        const T gy = sub_of<T>(sub_of<T>(vb.y, va.y), fma_of<T>(lz, nx, -mul_of<T>(lx, nz)));
-        const T gz = sub_of<T>(sub_of<T>(vb.z, va.z), fma_of<T>(lx, ny, -mul_of<T>(ly, nx)));
-        const T un = fma_of<T>(gz, nz, fma_of<T>(gy, ny, mul_of<T>(gx, nx)));
+        T gx, gy, gz;
+        const T un = contact_velocity3d<T>(r, va, wa, vb, wb, gx, gy, gz);
         const T tx = fma_of<T>(-un, nx, gx), ty = fma_of<T>(-un, ny, gy), tz = fma_of<T>(-un, nz, gz);
         Pn = pos_part(fma_of<T>(-mn, add_of<T>(b, un), r.P.x));
         Ptx = fma_of<T>(-mt, tx, r.P.y);

@@ -163,3 +163,25 @@ def test_domains_are_bit_identical(make, domains, precision):
         xa, xb = a.state(), b.state()
         for k in ("x", "v", "w"):
             assert np.array_equal(xa[k], xb[k]), k
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("value", [0.0, 3e38, np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_open_contacts_next_to_a_wild_velocity(dim, value, precision):
+    """Items whose contacts are all open and stay so are passed by; one with an
+    infinite or undefined rate is not."""
+    wl = (W.settling_discs(seed=2, n=40000, vsig=0.1) if dim == 2 else
+          W.sphere_gas(seed=2, n=20000, floor=40.0, vsig=0.1))
+    kw = dict(precision=precision, criterion=-1, max_sweeps=131, max_contacts=4 * wl.n)
+    a, b = gpu_system(wl, merge_last_colour=1, **kw), gpu_system(wl, **kw)
+    for s in (a, b):
+        s.detect_contacts()
+        s.vel.reshape(wl.n, dim)[::977] = value
+        s.solve_contacts()
+    ca, cb = a.contacts(), b.contacts()
+    assert len(ca["impulse"]) > 1000
+    assert np.array_equal(ca["impulse"], cb["impulse"], equal_nan=True)
+    xa, xb = a.state(), b.state()
+    for k in ("v", "w"):
+        assert np.array_equal(xa[k], xb[k], equal_nan=True), k
