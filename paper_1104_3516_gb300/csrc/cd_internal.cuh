@@ -213,10 +213,11 @@ struct CdWork {
     // adjoint (params.tape_steps > 0)
     char* tape;         // tape_steps slots of CdTapeHdr + one step's records
     double2* adj_Y;     // cap: adjoint multipliers (Y_n, Y_t) of the contacts
-    double4_16a* adj_B; // 2 n: per particle Gamma (x, y, w, 0) then Lambda (x, y, w, 0)
+    unsigned long long* adj_rec;  // n 96-byte records (cd_adjoint.cu)
     double4_16a* adj_lam; // n: dL/dv of the step's velocities (x, y, w, 0)
-    double2* adj_gx;    // n: dL/dx being accumulated
-    int* adj_mark;      // n: 1 if the particle has a non-open contact
+    unsigned long long* adj_mask; // n: colours of each particle's non-open contacts
+    unsigned* adj_ord;  // cap: a contact's places among them
+    void* adj_part;     // 4 G tagged block sums
 };
 
 // One recorded time step for the adjoint (2D, FP64): the colour-order
