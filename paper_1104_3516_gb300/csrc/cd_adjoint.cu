@@ -210,10 +210,18 @@ __device__ __forceinline__ double adj_geometry(const CdGeom& g, const CdTape& t,
     return dmu;
 }
 
-__global__ void k_tape_record(CdWork w, int n, int64_t cap)
+// Records the step in the tape's next slot (of T); the last block to have read
+// the slot advances it.
+__global__ void k_tape_record(CdWork w, int n, int64_t cap, int T)
 {
-    const CdCtrl* ctrl = w.ctrl;
-    const CdTape t = cd_tape_slot(w.tape, n, cap, ctrl->tape_slot);
+    CdCtrl* ctrl = w.ctrl;
+    const int slot = ctrl->tape_slot;
+    const CdTape t = cd_tape_slot(w.tape, n, cap, slot);
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&ctrl->tape_ticket, 1) == (int)gridDim.x - 1) {
+        ctrl->tape_ticket = 0;
+        ctrl->tape_slot = (slot + 1) % T;
+    }
     const int nc = ctrl->nc;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
@@ -230,11 +238,6 @@ __global__ void k_tape_record(CdWork w, int n, int64_t cap)
         t.P[c] = ((const double2*)w.c_P)[c];
     }
     for (int i = tid; i < n; i += stride) t.V[i] = ((const double4_16a*)w.V)[i];
-}
-
-__global__ void k_tape_advance(CdCtrl* ctrl, int T)
-{
-    ctrl->tape_slot = (ctrl->tape_slot + 1) % T;
 }
 
 __global__ void k_set_tape_slot(CdCtrl* ctrl, int slot)
@@ -587,6 +590,7 @@ k_adjoint(CdGeom g, CdWork w, CdTape t, CdAdjIO io, double alpha, int max_sweeps
             ctrl->adj_nslide = (long long)r[2];
             ctrl->adj_nbodies = (long long)r[3];
             ctrl->adj_diverged = sh.state == 2;
+            ctrl->tape_slot = io.slot;   // the step is consumed
         }
     }
 }
@@ -598,9 +602,8 @@ cudaError_t cd_launch_tape_record(const CdGeom& g, const CdWork& w, int64_t cap,
     int blocks = (g.n + CD_BLOCK - 1) / CD_BLOCK;
     if (blocks < 64) blocks = 64;
     if (blocks > 4096) blocks = 4096;
-    k_tape_record<<<blocks, CD_BLOCK, 0, s>>>(w, g.n, cap);
-    k_tape_advance<<<1, 1, 0, s>>>(w.ctrl, T);
-    *nl += 2;
+    k_tape_record<<<blocks, CD_BLOCK, 0, s>>>(w, g.n, cap, T);
+    ++*nl;
     return cudaGetLastError();
 }
 

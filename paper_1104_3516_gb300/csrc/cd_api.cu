@@ -383,9 +383,14 @@ static cd_status launch_detect_chain(cd_system* s, int timed, int pack)
     return launch_after_colour(s);
 }
 
+// The dataflow kernel of a plain system writes the caller's arrays itself
+// (unless each phase is timed by itself).
+static bool solve_unpacks(const cd_system* s) { return s->g.flow && s->g.npk == 1 && !s->p.timing; }
+
 static cd_status launch_solve(cd_system* s, int free_flight, int timed)
 {
     cd_status st;
+    const CdState io{s->pos, s->vel, s->omega, s->theta, free_flight};   // a step integrates
     s->mg_hint_valid = false;   // this solve's sweeps are unknown to the host until read back
     // (a step's velocities are packed by the one-kernel preparation)
     if (!(free_flight && s->prep.blocks))
@@ -399,7 +404,8 @@ static cd_status launch_solve(cd_system* s, int free_flight, int timed)
         return CD_OK;
     }
     if (s->g.flow) {
-        CD_CUDA(s, cd_launch_flow(s->g, s->w, s->num_sms, s->flow_records, (int)s->p.precision, (int)s->p.criterion, s->p.alpha,
+        CD_CUDA(s, cd_launch_flow(s->g, s->w, solve_unpacks(s) ? io : CdState{nullptr, nullptr, nullptr, nullptr, 0},
+                                  s->num_sms, s->flow_records, (int)s->p.precision, (int)s->p.criterion, s->p.alpha,
                                   (int)s->p.max_sweeps, s->stream, &s->launches));
         return CD_OK;
     }
@@ -839,8 +845,9 @@ extern "C" cd_status cd_solve_contacts(cd_system* s, cd_solve_stats* out)
     if (!s->has_contacts) return fail(s, CD_ERR_STATE, "no contact set: call cd_detect_contacts or cd_set_contacts");
     k_begin_call<<<1, 1, 0, s->stream>>>(s->w.ctrl, 1);
     if ((st = launch_solve(s, 0, 0)) != CD_OK) return st;
-    CD_CUDA(s, cd_launch_unpack(s->g, s->w, s->pos, s->vel, s->omega, s->theta, 0, (int)s->p.precision, s->stream,
-                                &s->launches));
+    if (!solve_unpacks(s))
+        CD_CUDA(s, cd_launch_unpack(s->g, s->w, s->pos, s->vel, s->omega, s->theta, 0, (int)s->p.precision, s->stream,
+                                    &s->launches));
     if (!out) return CD_OK;
     CdCtrl h;
     if ((st = read_ctrl(s, &h)) != CD_OK) return st;
@@ -858,8 +865,9 @@ static cd_status launch_step(cd_system* s, int timed)
     if ((st = launch_detect_chain(s, timed, 1)) != CD_OK) return st;
     if ((st = launch_solve(s, 1, timed)) != CD_OK) return st;
     if (timed && (st = mark(s)) != CD_OK) return st;
-    CD_CUDA(s, cd_launch_unpack(s->g, s->w, s->pos, s->vel, s->omega, s->theta, 1, (int)s->p.precision, s->stream,
-                                &s->launches));
+    if (!solve_unpacks(s))
+        CD_CUDA(s, cd_launch_unpack(s->g, s->w, s->pos, s->vel, s->omega, s->theta, 1, (int)s->p.precision, s->stream,
+                                    &s->launches));
     if (timed && (st = mark(s)) != CD_OK) return st;
     if (s->p.tape_steps > 0)
         CD_CUDA(s, cd_launch_tape_record(s->g, s->w, s->p.max_contacts, (int)s->p.tape_steps, s->stream,
@@ -1088,6 +1096,7 @@ extern "C" cd_status cd_adjoint_step(cd_system* s, const double* dL_dpos, const 
     io.ox = dL_dpos_prev; io.ov = dL_dvel_prev; io.ow = dL_domega_prev;
     io.inv_I = s->inv_I;
     io.eps = s->p.adjoint_compliance;
+    io.slot = slot;
     for (int k = 0; k < 6; ++k) {
         const double f = dL_dwall_force_host ? dL_dwall_force_host[k] : 0.0;
         if (!std::isfinite(f)) return fail(s, CD_ERR_INVALID_ARG, "dL_dwall_force not finite");
@@ -1101,7 +1110,6 @@ extern "C" cd_status cd_adjoint_step(cd_system* s, const double* dL_dpos, const 
     s->tape_head = slot;
     --s->tape_count;
     ++s->tape_mark;
-    CD_CUDA(s, cd_launch_set_tape_slot(s->w, slot, s->stream, &s->launches));
     if (out_host) {
         out_host->sweeps = h.adj_sweeps;
         out_host->converged = h.adj_converged;

@@ -37,6 +37,7 @@
 // regions a block on four warps each, to run one while the other waits (they
 // fall into step: FP64 10% slower, FP32 19%).
 #include "cd_flow_core.cuh"
+#include "cd_pack_core.cuh"
 
 #define FLOW_WORKERS 11                           // warps that update contacts
 #define FLOW_THREADS (32 * (FLOW_WORKERS + 1))    // and one that runs the convergence test
@@ -411,7 +412,7 @@ __device__ __forceinline__ bool flow_zero(const V& P)
 // 20,000 discs in 4 x 4 domains at FP64, this 13.2.)
 template <int DIM, typename T, bool BATCH, bool VIEWS>
 __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, FlowShared& sh, char* s_rec, int rec_cap,
-                                           const FlowTeam& tm, int K, int nc, T mu, int body0, int body1, int crit,
+                                           const FlowTeam& tm, const CdState& io, int K, int nc, T mu, int body0, int body1, int crit,
                                            double alpha, int max_sweeps)
 {
     typedef FlowBody<DIM, T> Body;
@@ -450,9 +451,11 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                 const int lo = k < K ? sh.lo[k] : 0, hi = k < K ? sh.end[k] : nview;
                 const int half = F64_2D && k < K && hi - lo <= FLOW_SPLIT * nb;
                 const int sh_item = half ? 4 : 5;
-                const long long items = (hi - lo + (1 << sh_item) - 1) >> sh_item;
-                const int r = (int)(((long long)k * 5 * nb >> 3) % nb);
-                const int i0 = (int)((items * tm.blk + r) / nb), i1 = (int)((items * (tm.blk + 1) + r) / nb);
+                const unsigned items = (unsigned)(hi - lo + (1 << sh_item) - 1) >> sh_item;
+                const unsigned r = (unsigned)(k * 5 * nb >> 3) % (unsigned)nb;
+                const unsigned each = items / (unsigned)nb, rest = items % (unsigned)nb;   // (32-bit: items * nb might not fit)
+                const int i0 = (int)(each * tm.blk + (rest * tm.blk + r) / (unsigned)nb);
+                const int i1 = (int)(each * (tm.blk + 1) + (rest * (tm.blk + 1) + r) / (unsigned)nb);
                 sh.lo[k] = min(lo + (i0 << sh_item), hi);
                 sh.end[k] = min(lo + (i1 << sh_item), hi);
                 sh.half[k] = half;
@@ -849,6 +852,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
         }
         V[RW * i] = v;
         if constexpr (DIM == 3) V[RW * i + 1] = o;
+        if (!BATCH && io.vel && i < g.n) unpack_particle<DIM, T>(g, io, i, v, o);
     }
     return true;
 }
@@ -856,12 +860,11 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
 // A plain system: the whole grid is one team.
 template <int DIM, typename T, bool VIEWS>
 __global__ void __launch_bounds__(FLOW_THREADS, 1)
-k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
+k_flow(CdGeom g, CdWork w, CdState io, int crit, double alpha, int max_sweeps, int rec_cap)
 {
     extern __shared__ __align__(128) char s_rec[];
     __shared__ FlowShared sh;
     __shared__ double s_red[FLOW_WORKERS + 1][3];
-    __shared__ double s_bc;
     CdCtrl* ctrl = w.ctrl;
     if (ctrl->skip) return;
     const int nc = ctrl->nc, K = ctrl->ncolours, nb = gridDim.x;
@@ -871,12 +874,16 @@ k_flow(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec_cap)
         sh.end[k] = w.colour_off[k + 1];
     }
     __syncthreads();
-    if (!flow_solve<DIM, T, false, VIEWS>(g, w, sh, s_rec, rec_cap, tm, K, nc, (T)g.mu, 0, g.n + (g.dyn_walls ? 6 : 0), crit,
-                                   alpha, max_sweeps))
+    if (!flow_solve<DIM, T, false, VIEWS>(g, w, sh, s_rec, rec_cap, tm, io, K, nc, (T)g.mu, 0,
+                                          g.n + (g.dyn_walls ? 6 : 0), crit, alpha, max_sweeps))
         return;
     u64 epoch = 0;
     finish_solve<DIM, T>(g, w, nc, nb, blockIdx.x * blockDim.x + threadIdx.x, nb * blockDim.x, epoch, sh.stop,
-                         sh.converged, sh.resid, sh.ravg, s_red, s_bc);
+                         sh.converged, sh.resid, sh.ravg, s_red);
+    if (io.vel && blockIdx.x == 0 && threadIdx.x == 0) {
+        if (g.dyn_walls) unpack_walls<DIM, T>(g, w);   // (their records are written before the barrier in finish_solve)
+        if (io.integrate) move_walls<DIM>(g, w, 0);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1032,7 +1039,7 @@ k_flow_batch(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec
             sh.end[k] = flow_lower(w, lo, w.colour_off[k + 1], first + count);
         }
         __syncthreads();
-        if (!flow_solve<DIM, T, true, false>(g, w, sh, s_rec, rec_cap, tm, K, nc, (T)w.pk[b].mu, first, first + count, crit,
+        if (!flow_solve<DIM, T, true, false>(g, w, sh, s_rec, rec_cap, tm, CdState{nullptr, nullptr, nullptr, nullptr, 0}, K, nc, (T)w.pk[b].mu, first, first + count, crit,
                                       alpha, max_sweeps))
             return;
         if (tm.blk == 0) {
@@ -1143,7 +1150,7 @@ int cd_flow_records(const CdGeom& g, int precision, int device)
     return recs;
 }
 
-static cudaError_t flow_launch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int criterion,
+static cudaError_t flow_launch(const CdGeom& g, const CdWork& w, const CdState* io, int blocks, int records, int precision, int criterion,
                                double alpha, int max_sweeps, cudaStream_t s, int* nl)
 {
     cudaError_t e = cudaMemsetAsync(w.ctrl, 0, 2 * sizeof(u64), s);
@@ -1154,16 +1161,18 @@ static cudaError_t flow_launch(const CdGeom& g, const CdWork& w, int blocks, int
     CdWork wa = w;
     int crit = criterion, ms = max_sweeps, rc = records;
     double al = alpha;
-    void* args[] = {&ga, &wa, &crit, &al, &ms, &rc};
+    CdState st = io ? *io : CdState{nullptr, nullptr, nullptr, nullptr, 0};
+    void* plain[] = {&ga, &wa, &st, &crit, &al, &ms, &rc};
+    void* batch[] = {&ga, &wa, &crit, &al, &ms, &rc};
     ++*nl;
-    return cudaLaunchCooperativeKernel(f.fn, dim3(blocks), dim3(FLOW_THREADS), args,
+    return cudaLaunchCooperativeKernel(f.fn, dim3(blocks), dim3(FLOW_THREADS), io ? plain : batch,
                                        (size_t)(records * f.record_bytes), s);
 }
 
-cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int criterion,
+cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, const CdState& io, int blocks, int records, int precision, int criterion,
                            double alpha, int max_sweeps, cudaStream_t s, int* nl)
 {
-    return flow_launch(g, w, blocks, records, precision, criterion, alpha, max_sweeps, s, nl);
+    return flow_launch(g, w, &io, blocks, records, precision, criterion, alpha, max_sweeps, s, nl);
 }
 
 cudaError_t cd_launch_flow_batch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision,
@@ -1171,7 +1180,7 @@ cudaError_t cd_launch_flow_batch(const CdGeom& g, const CdWork& w, int blocks, i
 {
     k_flow_plan<<<1, 512, 0, s>>>(g, w, blocks, records);
     ++*nl;
-    cudaError_t e = flow_launch(g, w, blocks, records, precision, criterion, alpha, max_sweeps, s, nl);
+    cudaError_t e = flow_launch(g, w, nullptr, blocks, records, precision, criterion, alpha, max_sweeps, s, nl);
     if (e != cudaSuccess) return e;
     k_flow_totals<<<1, 256, 0, s>>>(g, w);
     ++*nl;

@@ -45,6 +45,7 @@ struct CdCtrl {
     long long max_sweeps_step;
     long long n_not_conv;
     // last adjoint step
+    int tape_ticket;                // blocks of k_tape_record that have read tape_slot
     long long adj_sweeps;
     long long adj_converged;
     double adj_residual;
@@ -523,6 +524,13 @@ cudaError_t cd_launch_orient(const CdGeom& g, const CdWork& w, int nbins, unsign
 // replayed).
 cudaError_t cd_launch_tape_record(const CdGeom& g, const CdWork& w, int64_t cap, int T, cudaStream_t stream, int* nl);
 cudaError_t cd_launch_set_tape_slot(const CdWork& w, int slot, cudaStream_t stream, int* nl);
+// Where a solve's velocities go: the caller's arrays; with integrate the
+// positions (and 2D orientations, if any) follow.  vel null: nowhere.
+struct CdState {
+    double *pos, *vel, *omega, *theta;
+    int integrate;
+};
+
 struct CdAdjIO {
     const double* dLx;      // n*2: dL/dx' of the step's output positions
     const double* dLv;      // n*2: dL/dv'
@@ -533,6 +541,7 @@ struct CdAdjIO {
     const double* inv_I;    // n
     double wq[6];           // dL/d(wall force k) / dt: weight of the normal impulse of a contact with wall k
     double eps;             // relative compliance of the rows (params.adjoint_compliance)
+    int slot;               // the step's tape slot
 };
 cudaError_t cd_launch_adjoint(const CdGeom& g, const CdWork& w, const CdTape& t, const CdAdjIO& io, double alpha,
                               int max_sweeps, int coop_blocks, cudaStream_t stream, int* nl);
@@ -541,7 +550,7 @@ cudaError_t cd_launch_stress(const CdGeom& g, const CdWork& w, const double* pos
                              double lo, double width, int ns, double* sig, cudaStream_t stream, int* nl);
 cudaError_t cd_launch_sweep(const CdGeom& g, const CdWork& w, int coop_blocks, int threads, int precision,
                             int criterion, double alpha, int max_sweeps, int pw, cudaStream_t stream, int* nl);
-cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, int blocks, int records, int precision, int criterion,
+cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, const CdState& io, int blocks, int records, int precision, int criterion,
                            double alpha, int max_sweeps, cudaStream_t stream, int* nl);
 cudaError_t cd_launch_flow_batch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision,
                                  int criterion, double alpha, int max_sweeps, cudaStream_t stream, int* nl);

@@ -64,3 +64,56 @@ __device__ __forceinline__ void pack_velocities(const CdGeom& g, const CdWork& w
         }
     }
 }
+
+// Particle i's velocities (v, o: its record) to the caller's arrays; with
+// integrate its position (and 2D orientation) follows Eq. 2.
+template <int DIM, typename T>
+__device__ __forceinline__ void unpack_particle(const CdGeom& g, const CdState& io, int i, const typename Vec<T>::V4& s,
+                                                const typename Vec<T>::V4& o)
+{
+    const double v[3] = {(double)s.x, (double)s.y, DIM == 3 ? (double)s.z : 0.0};
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        io.vel[i * DIM + k] = v[k];
+        if (io.integrate) {
+            double xn = __dadd_rn(io.pos[i * DIM + k], __dmul_rn(v[k], g.dt));
+            if (g.periodic[k]) {
+                if (xn >= g.hi[k]) xn = __dsub_rn(xn, g.L[k]);
+                else if (xn < g.lo[k]) xn = __dadd_rn(xn, g.L[k]);
+            }
+            io.pos[i * DIM + k] = xn;
+        }
+    }
+    if (DIM == 2) {
+        const double om = (double)s.z;
+        io.omega[i] = om;
+        if (io.integrate && io.theta) io.theta[i] = __dadd_rn(io.theta[i], __dmul_rn(om, g.dt));
+    } else {
+        io.omega[3 * i] = (double)o.x; io.omega[3 * i + 1] = (double)o.y; io.omega[3 * i + 2] = (double)o.z;
+    }
+}
+
+// Force-controlled walls: their velocity after the solve becomes the wall velocity.
+template <int DIM, typename T>
+__device__ __forceinline__ void unpack_walls(const CdGeom& g, const CdWork& w)
+{
+    typedef typename Vec<T>::V4 T4;
+    const T4* V = (const T4*)w.V;
+    for (int k = 0; k < 2 * DIM; ++k) {
+        if (!((g.dyn_walls >> k) & 1)) continue;
+        const T4 s = (DIM == 2) ? V[g.n + k] : V[2 * (g.n + k)];
+        const double u[3] = {(double)s.x, (double)s.y, (double)s.z};
+        w.pk[0].wall_vel[3 * k + (k >> 1)] = u[k >> 1];
+    }
+}
+
+// The walls of packing b move (Eq. 2).
+template <int DIM>
+__device__ __forceinline__ void move_walls(const CdGeom& g, const CdWork& w, int b)
+{
+    const CdPack& pb = w.pk[b];
+    for (int k = 0; k < 2 * DIM; ++k)
+        if ((pb.wall_mask >> k) & 1)
+            w.pk_wall_pos[6 * b + k] =
+                __dadd_rn(w.pk_wall_pos[6 * b + k], __dmul_rn(pb.wall_vel[3 * k + (k >> 1)], g.dt));
+}

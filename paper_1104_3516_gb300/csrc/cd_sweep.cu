@@ -86,58 +86,19 @@ template <int DIM, typename T>
 __global__ void k_unpack(CdGeom g, CdWork w, double* __restrict__ pos, double* __restrict__ vel,
                          double* __restrict__ omega, double* __restrict__ theta, int integrate)
 {
-    CdCtrl* ctrl = w.ctrl;
-    if (ctrl->skip) return;
+    if (w.ctrl->skip) return;
     typedef typename Vec<T>::V4 T4;
     const T4* V = (const T4*)w.V;
+    const CdState io{pos, vel, omega, theta, integrate};
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.n; i += gridDim.x * blockDim.x) {
-        double v[3], om[3];
-        if (DIM == 2) {
-            T4 s = V[i];
-            v[0] = (double)s.x; v[1] = (double)s.y; v[2] = 0.0;
-            om[0] = (double)s.z;
-        } else {
-            T4 s = V[2 * i], o = V[2 * i + 1];
-            v[0] = (double)s.x; v[1] = (double)s.y; v[2] = (double)s.z;
-            om[0] = (double)o.x; om[1] = (double)o.y; om[2] = (double)o.z;
-        }
-#pragma unroll
-        for (int k = 0; k < DIM; ++k) {
-            vel[i * DIM + k] = v[k];
-            if (integrate) {
-                double xn = __dadd_rn(pos[i * DIM + k], __dmul_rn(v[k], g.dt));
-                if (g.periodic[k]) {
-                    if (xn >= g.hi[k]) xn = __dsub_rn(xn, g.L[k]);
-                    else if (xn < g.lo[k]) xn = __dadd_rn(xn, g.L[k]);
-                }
-                pos[i * DIM + k] = xn;
-            }
-        }
-        if (DIM == 2) {
-            omega[i] = om[0];
-            if (integrate && theta) theta[i] = __dadd_rn(theta[i], __dmul_rn(om[0], g.dt));
-        } else {
-            omega[3 * i] = om[0]; omega[3 * i + 1] = om[1]; omega[3 * i + 2] = om[2];
-        }
+        if constexpr (DIM == 2) unpack_particle<2, T>(g, io, i, V[i], V[i]);
+        else unpack_particle<3, T>(g, io, i, V[2 * i], V[2 * i + 1]);
     }
-    if (g.dyn_walls && blockIdx.x == 0 && threadIdx.x == 0) {
-        // force-controlled walls: their velocity after the solve becomes the wall velocity
-        for (int k = 0; k < 2 * DIM; ++k) {
-            if (!((g.dyn_walls >> k) & 1)) continue;
-            const T4 s = (DIM == 2) ? V[g.n + k] : V[2 * (g.n + k)];
-            const double u[3] = {(double)s.x, (double)s.y, (double)s.z};
-            w.pk[0].wall_vel[3 * k + (k >> 1)] = u[k >> 1];
-        }
-    }
+    if (g.dyn_walls && blockIdx.x == 0 && threadIdx.x == 0) unpack_walls<DIM, T>(g, w);
     if (integrate) {
         if (g.dyn_walls) __syncthreads();   // block 0 moves the walls after their velocities are written
-        for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < g.npk; b += gridDim.x * blockDim.x) {
-            const CdPack& pb = w.pk[b];
-            for (int k = 0; k < 2 * DIM; ++k)
-                if ((pb.wall_mask >> k) & 1)
-                    w.pk_wall_pos[6 * b + k] = __dadd_rn(w.pk_wall_pos[6 * b + k],
-                                                         __dmul_rn(pb.wall_vel[3 * k + (k >> 1)], g.dt));
-        }
+        for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < g.npk; b += gridDim.x * blockDim.x)
+            move_walls<DIM>(g, w, b);
     }
 }
 
@@ -564,7 +525,7 @@ k_sweep(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps)
         }
     }
 
-    finish_solve<DIM, T>(g, w, nc, nb, tid, stride, epoch, sweeps, converged, resid, ravg, s_red, s_bc);
+    finish_solve<DIM, T>(g, w, nc, nb, tid, stride, epoch, sweeps, converged, resid, ravg, s_red);
 }
 
 // ---------------------------------------------------------------------------

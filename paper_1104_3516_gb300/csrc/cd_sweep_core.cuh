@@ -676,7 +676,7 @@ __device__ __forceinline__ UpdOut apply_rec(const CdGeom& g, const CdWork& w, in
 template <int DIM, typename T>
 __device__ __forceinline__ void finish_solve(const CdGeom& g, const CdWork& w, int nc, int nb, int tid, int stride,
                                              unsigned long long& epoch, int sweeps, int converged, double resid,
-                                             double ravg, double (*s_red)[3], double& s_bc)
+                                             double ravg, double (*s_red)[3])
 {
     CdCtrl* ctrl = w.ctrl;
     double wsum[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
@@ -717,10 +717,16 @@ __device__ __forceinline__ void finish_solve(const CdGeom& g, const CdWork& w, i
     }
     if (!cd_grid_sync(ctrl, nb, epoch)) return;
     if (blockIdx.x == 0) {
-        double wf[6];
-        for (int q = 0; q < 6; ++q) wf[q] = grid_total(w.wpart + q * nb, nb, &s_bc);
+        // a warp a wall (one warp for all six after another, and the divisions one
+        // after another, kept the last block 10 us longer)
+        const int lane = threadIdx.x & 31;
+        for (int q = threadIdx.x >> 5; q < 6; q += blockDim.x >> 5) {
+            double x = 0.0;
+            for (int b = lane; b < nb; b += 32) x += w.wpart[q * nb + b];
+            x = warp_sum_nz(x);
+            if (lane == 0) ctrl->wall_force[q] = x / g.dt;
+        }
         if (threadIdx.x == 0) {
-            for (int q = 0; q < 6; ++q) ctrl->wall_force[q] = wf[q] / g.dt;
             ctrl->sweeps = sweeps;
             ctrl->mg_prev = sweeps + 1;
             ctrl->converged = converged;
