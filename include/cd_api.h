@@ -365,7 +365,7 @@ cd_status cd_download_state(cd_system* sys, double* pos_host, double* vel_host, 
  * Work is enqueued on cuda_stream, and every call synchronises that stream
  * (it reads the largest radius and the contact count back to the host).
  *
- * Scratch lives in a fixed device array of about 4.1 MB inside the library,
+ * Scratch lives in a fixed device array of about 4.4 MB inside the library,
  * held by every GPU that loads it until the process exits; limits: n <= 16384
  * particles, at most 65536 cells of side 2 r_max + delta, max_contacts <=
  * 65536.  Larger sizes return CD_ERR_INVALID_ARG (message via

@@ -47,34 +47,52 @@
 #define NA_CAND (NA_PK + NA_ALIGN(sizeof(double) * 4 * CD_NOALLOC_MAX_CONTACTS))
 #define NA_RMAX (NA_CAND + NA_I32((size_t)CD_NOALLOC_MAX_N * CD_CAND))
 #define NA_TOT (NA_RMAX + 256)
-#define NA_BYTES (NA_TOT + NA_I32(4 * CD_PREP_MAX_BLOCKS))
+#define NA_PF (NA_TOT + NA_I32(4 * CD_PREP_MAX_BLOCKS))
+#define NA_BYTES (NA_PF + NA_ALIGN(sizeof(float4) * CD_NOALLOC_MAX_N))
 
 static __device__ __align__(256) unsigned char cd_noalloc_scratch[NA_BYTES];
 
 static std::mutex na_mutex;
 static void* na_addr[CD_NOALLOC_MAX_DEVICES];
 
-// Largest radius (as ordered bits of a positive double) and a flag for any
-// radius that is not positive and finite.
-__global__ void k_noalloc_radii(int n, const double* __restrict__ radius, unsigned long long* out)
+// Clears the control block; the largest radius (as ordered bits of a positive
+// double) into out[0], and into out[1] whether one is not positive and finite.
+// One block: n is small, and an atomic a particle on one address took 8 us of
+// 5,000 particles' 112.
+__global__ void __launch_bounds__(1024) k_noalloc_begin(CdCtrl* ctrl, int n, const double* __restrict__ radius,
+                                                        unsigned long long* out, double w0, double w1, double w2,
+                                                        double w3, double w4, double w5)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double r = radius[i];
-        if (!(r > 0.0) || !isfinite(r)) atomicMax(&out[1], 1ULL);
-        else atomicMax(&out[0], (unsigned long long)__double_as_longlong(r));
+    __shared__ unsigned long long s_top[32];
+    __shared__ int s_bad;
+    if (threadIdx.x == 0) s_bad = 0;
+    __syncthreads();
+    unsigned long long top = 0ULL;
+    bool bad = false;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const double r = radius[i];
+        if (!(r > 0.0) || !isfinite(r)) bad = true;
+        else top = max(top, (unsigned long long)__double_as_longlong(r));
     }
-}
-
-__global__ void k_noalloc_begin(CdCtrl* ctrl, unsigned long long* rmax_bits, double w0, double w1, double w2, double w3,
-                                double w4, double w5)
-{
-    CdCtrl c;
-    memset(&c, 0, sizeof c);
-    c.wall_pos[0] = w0; c.wall_pos[1] = w1; c.wall_pos[2] = w2;
-    c.wall_pos[3] = w3; c.wall_pos[4] = w4; c.wall_pos[5] = w5;
-    *ctrl = c;
-    rmax_bits[0] = 0ULL;
-    rmax_bits[1] = 0ULL;
+    if (bad) s_bad = 1;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    if ((threadIdx.x & 31) == 0) s_top[threadIdx.x >> 5] = top;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        top = s_top[threadIdx.x];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    }
+    if (threadIdx.x == 0) {
+        CdCtrl c;
+        memset(&c, 0, sizeof c);
+        c.wall_pos[0] = w0; c.wall_pos[1] = w1; c.wall_pos[2] = w2;
+        c.wall_pos[3] = w3; c.wall_pos[4] = w4; c.wall_pos[5] = w5;
+        *ctrl = c;
+        out[0] = top;
+        out[1] = s_bad ? 1ULL : 0ULL;
+    }
 }
 
 // Message of a failure, read back with cd_last_error(NULL).
@@ -136,12 +154,10 @@ extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t
 
     CdCtrl* ctrl = (CdCtrl*)(base + NA_CTRL);
     unsigned long long* rbits = (unsigned long long*)(base + NA_RMAX);
-    k_noalloc_begin<<<1, 1, 0, s>>>(ctrl, rbits, p.wall_pos[0], p.wall_pos[1], p.wall_pos[2], p.wall_pos[3],
-                                    p.wall_pos[4], p.wall_pos[5]);
+    k_noalloc_begin<<<1, 1024, 0, s>>>(ctrl, (int)n, radius, rbits, p.wall_pos[0], p.wall_pos[1], p.wall_pos[2],
+                                       p.wall_pos[3], p.wall_pos[4], p.wall_pos[5]);
     const CdPrepPlan plan = cd_prepare_plan((int)p.dim, CD_FP64, n, dev);
     if (!plan.blocks) return na_error(CD_ERR_CUDA, "the detection kernel does not fit on this device");
-    int gb = (int)((n + CD_BLOCK - 1) / CD_BLOCK);
-    k_noalloc_radii<<<gb, CD_BLOCK, 0, s>>>((int)n, radius, rbits);
     unsigned long long hb[2] = {0ULL, 0ULL};
     if ((e = cudaMemcpyAsync(hb, rbits, sizeof hb, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
         return na_cuda(e, "reading the largest radius");
@@ -198,6 +214,7 @@ extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t
     w.pcnt = (int*)(base + NA_PCNT);
     w.poff = (int*)(base + NA_POFF);
     w.cand = (int*)(base + NA_CAND);
+    w.pf = (float4*)(base + NA_PF);
     w.scan_tmp = (int*)(base + NA_SCAN);
     w.mn = (double*)(base + NA_MN);
     w.mt = (double*)(base + NA_MT);
