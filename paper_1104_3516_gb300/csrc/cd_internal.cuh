@@ -488,6 +488,16 @@ cudaError_t cd_launch_set_contacts(const CdGeom& g, const CdWork& w, const doubl
 cudaError_t cd_launch_colour(const CdGeom& g, const CdWork& w, int coop_blocks, int precision, int pw,
                              cudaStream_t stream, int* nl, const double* pos);
 // What the one-kernel preparation reads (cd_prepare.cu).
+// A cell grid laid out on the device (detection without workspace): the largest
+// radius is known there first.
+enum { CDG_OK = 0, CDG_RADIUS, CDG_PERIODIC, CDG_CELLS };
+struct CdGridSpec {
+    double cs[3], inv_cs[3];
+    int ncell[3];
+    int total;
+    int status;   // CDG_*: what the grid is refused for
+};
+
 struct CdPrepIO {
     const double* pos;
     const double* radius;
@@ -497,9 +507,9 @@ struct CdPrepIO {
     const double* omega;
     const double* f_ext;
     int warm, pw;
-    int detect_only;    // stop once the contact set is current
     int pack;           // 1: the velocities too, free_flight as cd_launch_pack
     int free_flight;
+    const CdGridSpec* grid;   // with the detection-only kernel: the grid (null: that of the CdGeom)
 };
 #define CD_PREP_MAX_BLOCKS 256
 cudaError_t cd_launch_prepare(const CdGeom& g, const CdWork& w, const CdPrepIO& io, int blocks, int cluster,
@@ -507,7 +517,8 @@ cudaError_t cd_launch_prepare(const CdGeom& g, const CdWork& w, const CdPrepIO& 
 // Blocks of the one-kernel preparation for n particles (0: it does not fit the
 // device), and whether they form one cluster.
 struct CdPrepPlan { int blocks, cluster; };
-CdPrepPlan cd_prepare_plan(int dim, int precision, int64_t n, int device);
+int cd_prepare_cluster_n(int dim);   // particles up to which the plan is one cluster of blocks
+CdPrepPlan cd_prepare_plan(int dim, int precision, int detect_only, int64_t n, int device);
 #define CD_PREP_MAX_N 500000   // see cd_prepare.cu
 cudaError_t cd_launch_pack(const CdGeom& g, const CdWork& w, const double* vel, const double* omega,
                            const double* radius, const double* inv_m, const double* inv_I, const double* f_ext,

@@ -33,7 +33,8 @@
 #define NA_ALIGN(x) ((((size_t)(x)) + 255) & ~(size_t)255)
 #define NA_CTRL 0
 #define NA_I32(count) NA_ALIGN(sizeof(int) * (size_t)(count))
-#define NA_CELL_OF (NA_CTRL + NA_ALIGN(sizeof(CdCtrl)))
+#define NA_GRID (NA_CTRL + NA_ALIGN(sizeof(CdCtrl)))   // (read back with the control block)
+#define NA_CELL_OF (NA_GRID + NA_ALIGN(sizeof(CdGridSpec)))
 #define NA_CELL_CNT (NA_CELL_OF + NA_I32(CD_NOALLOC_MAX_N))
 #define NA_CELL_START (NA_CELL_CNT + NA_I32(CD_NOALLOC_MAX_CELLS + 1))
 #define NA_CELL_FILL (NA_CELL_START + NA_I32(CD_NOALLOC_MAX_CELLS + 1))
@@ -45,31 +46,35 @@
 #define NA_MT (NA_MN + NA_ALIGN(sizeof(double) * CD_NOALLOC_MAX_CONTACTS))
 #define NA_PK (NA_MT + NA_ALIGN(sizeof(double) * CD_NOALLOC_MAX_CONTACTS))
 #define NA_CAND (NA_PK + NA_ALIGN(sizeof(double) * 4 * CD_NOALLOC_MAX_CONTACTS))
-#define NA_RMAX (NA_CAND + NA_I32((size_t)CD_NOALLOC_MAX_N * CD_CAND))
-#define NA_TOT (NA_RMAX + 256)
+#define NA_TOT (NA_CAND + NA_I32((size_t)CD_NOALLOC_MAX_N * CD_CAND))
 #define NA_PF (NA_TOT + NA_I32(4 * CD_PREP_MAX_BLOCKS))
 #define NA_BYTES (NA_PF + NA_ALIGN(sizeof(float4) * CD_NOALLOC_MAX_N))
 
 static __device__ __align__(256) unsigned char cd_noalloc_scratch[NA_BYTES];
 
+// Of each device: the scratch array, and the launch plans (2D and 3D, by the
+// size class of cd_prepare_plan).
 static std::mutex na_mutex;
 static void* na_addr[CD_NOALLOC_MAX_DEVICES];
+static CdPrepPlan na_plan[CD_NOALLOC_MAX_DEVICES][2][2];
 
-// Clears the control block; the largest radius (as ordered bits of a positive
-// double) into out[0], and into out[1] whether one is not positive and finite.
-// One block: n is small, and an atomic a particle on one address took 8 us of
-// 5,000 particles' 112.
-__global__ void __launch_bounds__(1024) k_noalloc_begin(CdCtrl* ctrl, int n, const double* __restrict__ radius,
-                                                        unsigned long long* out, double w0, double w1, double w2,
-                                                        double w3, double w4, double w5)
+// Clears the control block, takes the largest radius (as ordered bits of a
+// positive double; a flag if one is not positive and finite) and lays out the
+// cell grid, by the operations of cd_create_system.  One block: n is small, and
+// an atomic a particle on one address took 8 us of 5,000 particles' 112.  The
+// grid used to be the host's, which had to wait for the radius first.
+__global__ void __launch_bounds__(1024) k_noalloc_begin(CdCtrl* ctrl, CdGridSpec* grid, CdGeom g, double w0, double w1,
+                                                        double w2, double w3, double w4, double w5,
+                                                        const double* __restrict__ radius)
 {
     __shared__ unsigned long long s_top[32];
     __shared__ int s_bad;
+    __shared__ int s_m[3];
     if (threadIdx.x == 0) s_bad = 0;
     __syncthreads();
     unsigned long long top = 0ULL;
     bool bad = false;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i = threadIdx.x; i < g.n; i += blockDim.x) {
         const double r = radius[i];
         if (!(r > 0.0) || !isfinite(r)) bad = true;
         else top = max(top, (unsigned long long)__double_as_longlong(r));
@@ -83,15 +88,39 @@ __global__ void __launch_bounds__(1024) k_noalloc_begin(CdCtrl* ctrl, int n, con
         top = s_top[threadIdx.x];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+        const double ell = __dmul_rn(__dadd_rn(__dmul_rn(2.0, __longlong_as_double((long long)top)), g.delta), 1.0 + 1e-9);
+        const int k = threadIdx.x;
+        if (k < 3) {
+            double m = 1.0;
+            if (k < g.dim) {
+                m = floor(__ddiv_rn(g.L[k], ell));
+                if (!(m >= 1.0)) m = 1.0;
+                if (m > (double)CD_NOALLOC_MAX_CELLS) m = (double)CD_NOALLOC_MAX_CELLS;
+                grid->cs[k] = __ddiv_rn(g.L[k], m);
+                grid->inv_cs[k] = __ddiv_rn(1.0, grid->cs[k]);
+            } else {
+                grid->cs[k] = 1.0;
+                grid->inv_cs[k] = 1.0;
+            }
+            grid->ncell[k] = s_m[k] = (int)m;
+        }
+        __syncwarp();
     }
     if (threadIdx.x == 0) {
+        int status = s_bad ? CDG_RADIUS : CDG_OK;
+        long long total = 1;
+        for (int k = 0; k < 3; ++k) {
+            if (g.periodic[k] && s_m[k] < 3 && status == CDG_OK) status = CDG_PERIODIC;
+            total *= s_m[k];
+        }
+        if (total > CD_NOALLOC_MAX_CELLS && status == CDG_OK) status = CDG_CELLS;
+        grid->total = total > CD_NOALLOC_MAX_CELLS ? CD_NOALLOC_MAX_CELLS : (int)total;
+        grid->status = status;
         CdCtrl c;
         memset(&c, 0, sizeof c);
         c.wall_pos[0] = w0; c.wall_pos[1] = w1; c.wall_pos[2] = w2;
         c.wall_pos[3] = w3; c.wall_pos[4] = w4; c.wall_pos[5] = w5;
         *ctrl = c;
-        out[0] = top;
-        out[1] = s_bad ? 1ULL : 0ULL;
     }
 }
 
@@ -141,6 +170,7 @@ extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t
     if (e != cudaSuccess) return na_cuda(e, "cudaGetDevice");
     if (dev < 0 || dev >= CD_NOALLOC_MAX_DEVICES) return na_error(CD_ERR_INVALID_ARG, "device index out of range");
     unsigned char* base = nullptr;
+    CdPrepPlan plan;
     {
         std::lock_guard<std::mutex> lock(na_mutex);
         if (!na_addr[dev]) {
@@ -150,22 +180,14 @@ extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t
             na_addr[dev] = ptr;
         }
         base = (unsigned char*)na_addr[dev];
+        CdPrepPlan& known = na_plan[dev][p.dim - 2][n <= cd_prepare_cluster_n((int)p.dim) ? 1 : 0];
+        if (!known.blocks) known = cd_prepare_plan((int)p.dim, CD_FP64, 1, n, dev);
+        plan = known;
     }
+    if (!plan.blocks) return na_error(CD_ERR_CUDA, "the detection kernel does not fit on this device");
 
     CdCtrl* ctrl = (CdCtrl*)(base + NA_CTRL);
-    unsigned long long* rbits = (unsigned long long*)(base + NA_RMAX);
-    k_noalloc_begin<<<1, 1024, 0, s>>>(ctrl, (int)n, radius, rbits, p.wall_pos[0], p.wall_pos[1], p.wall_pos[2],
-                                       p.wall_pos[3], p.wall_pos[4], p.wall_pos[5]);
-    const CdPrepPlan plan = cd_prepare_plan((int)p.dim, CD_FP64, n, dev);
-    if (!plan.blocks) return na_error(CD_ERR_CUDA, "the detection kernel does not fit on this device");
-    unsigned long long hb[2] = {0ULL, 0ULL};
-    if ((e = cudaMemcpyAsync(hb, rbits, sizeof hb, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-        return na_cuda(e, "reading the largest radius");
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return na_cuda(e, "cudaStreamSynchronize");
-    if (hb[1]) return na_error(CD_ERR_INVALID_ARG, "radius must be positive and finite");
-    double rmax;
-    memcpy(&rmax, &hb[0], sizeof rmax);
-
+    CdGridSpec* grid = (CdGridSpec*)(base + NA_GRID);
     CdGeom g;
     memset(&g, 0, sizeof g);
     g.dim = (int)p.dim;
@@ -178,30 +200,14 @@ extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t
     g.rotations = (int)p.rotations;
     g.seed = p.seed;
     g.npk = 1;
-    const double ell = (2.0 * rmax + p.delta) * (1.0 + 1e-9);   // as in cd_create_system
-    long long ncell = 1;
     for (int k = 0; k < 3; ++k) {
         g.periodic[k] = (k < p.dim) ? (int)p.periodic[k] : 0;
-        if (k < p.dim) {
-            g.lo[k] = p.box_lo[k];
-            g.hi[k] = p.box_hi[k];
-            g.L[k] = p.box_hi[k] - p.box_lo[k];
-            double m = std::floor(g.L[k] / ell);
-            if (m < 1.0) m = 1.0;
-            if (m > (double)CD_NOALLOC_MAX_CELLS) m = (double)CD_NOALLOC_MAX_CELLS;
-            g.ncell[k] = (int)m;
-            g.cs[k] = g.L[k] / m;
-            g.inv_cs[k] = 1.0 / g.cs[k];
-            if (g.periodic[k] && g.ncell[k] < 3)
-                return na_error(CD_ERR_INVALID_ARG, "a periodic axis needs at least 3 cells (box >= 3 l)");
-        } else {
-            g.lo[k] = 0.0; g.hi[k] = 1.0; g.L[k] = 1.0; g.ncell[k] = 1; g.cs[k] = 1.0; g.inv_cs[k] = 1.0;
-        }
-        ncell *= g.ncell[k];
+        g.lo[k] = (k < p.dim) ? p.box_lo[k] : 0.0;
+        g.hi[k] = (k < p.dim) ? p.box_hi[k] : 1.0;
+        g.L[k] = (k < p.dim) ? p.box_hi[k] - p.box_lo[k] : 1.0;
     }
-    if (ncell > CD_NOALLOC_MAX_CELLS)
-        return na_error(CD_ERR_INVALID_ARG, "the box needs more than 65536 cells for the no-allocation entry point");
-    g.ncell_total = (int)ncell;
+    k_noalloc_begin<<<1, 1024, 0, s>>>(ctrl, grid, g, p.wall_pos[0], p.wall_pos[1], p.wall_pos[2], p.wall_pos[3],
+                                       p.wall_pos[4], p.wall_pos[5], radius);
 
     CdWork w;
     memset(&w, 0, sizeof w);
@@ -231,13 +237,22 @@ extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t
     CdPrepIO io = {};
     io.pos = pos; io.radius = radius; io.inv_m = inv_mass; io.inv_I = inv_inertia;
     io.pw = pw;
-    io.detect_only = 1;
+    io.grid = grid;
     if ((e = cd_launch_prepare(g, w, io, plan.blocks, plan.cluster, CD_FP64, s, &nl)) != cudaSuccess)
         return na_cuda(e, "detection launch");
-    CdCtrl h;
-    if ((e = cudaMemcpyAsync(&h, ctrl, sizeof h, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+    alignas(16) unsigned char back[NA_GRID + sizeof(CdGridSpec)];
+    if ((e = cudaMemcpyAsync(back, base, sizeof back, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
         return na_cuda(e, "reading the contact count");
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return na_cuda(e, "cudaStreamSynchronize");
+    CdCtrl h;
+    CdGridSpec hg;
+    memcpy(&h, back + NA_CTRL, sizeof h);
+    memcpy(&hg, back + NA_GRID, sizeof hg);
+    if (hg.status == CDG_RADIUS) return na_error(CD_ERR_INVALID_ARG, "radius must be positive and finite");
+    if (hg.status == CDG_PERIODIC)
+        return na_error(CD_ERR_INVALID_ARG, "a periodic axis needs at least 3 cells (box >= 3 l)");
+    if (hg.status == CDG_CELLS)
+        return na_error(CD_ERR_INVALID_ARG, "the box needs more than 65536 cells for the no-allocation entry point");
     *n_contacts = h.nc_needed;
     if (h.error == CDE_PER_PARTICLE) return na_error(CD_ERR_CAPACITY, "a particle has more than 64 contact candidates");
     if (h.overflow) return na_error(CD_ERR_CAPACITY, "more contacts than max_contacts; *n_contacts holds the number needed");

@@ -126,13 +126,11 @@ __host__ __device__ __forceinline__ int prep_shift(int count, int nb)
     return s;
 }
 
-template <int DIM, typename T>
-__global__ void __launch_bounds__(PREP_THREADS, 1) k_prepare(CdGeom g, CdWork w, CdPrepIO io, int cluster)
+template <int DIM, typename T, bool DETECT_ONLY>
+__device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const CdPrepIO& io, int cluster, int* s_dyn,
+                                        PrepShared& sh)
 {
-    extern __shared__ int s_dyn[];   // the counting pass's queues and runs
-    __shared__ PrepShared sh;
     CdCtrl* ctrl = w.ctrl;
-    if (ctrl->skip) return;
     const int nb = gridDim.x, blk = blockIdx.x;
     const int tid = blk * PREP_THREADS + (int)threadIdx.x, stride = nb * PREP_THREADS;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -152,7 +150,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 1) k_prepare(CdGeom g, CdWork w,
         w.cell_cnt[i] = 0;
         if (i < ncell) w.cell_fill[i] = 0;
     }
-    if (!io.detect_only) {
+    if (!DETECT_ONLY) {
         for (int i = tid; i <= nbody; i += stride) {
             w.p2c_cnt[i] = 0;
             if (i < nbody) w.p2c_fill[i] = 0;
@@ -162,7 +160,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 1) k_prepare(CdGeom g, CdWork w,
 
     // cell lists (in no order)
     for (int i = tid; i < n; i += stride) count_cell<DIM>(g, w, io.pos, io.radius, i, w.cell_of, w.cell_cnt);
-    if (!io.detect_only && io.pack)
+    if (!DETECT_ONLY && io.pack)
         pack_velocities<DIM, T>(g, w, io.vel, io.omega, io.inv_m, io.f_ext, io.free_flight, tid, stride, blk == 0);
     if (!sync()) return;
     {
@@ -208,14 +206,14 @@ __global__ void __launch_bounds__(PREP_THREADS, 1) k_prepare(CdGeom g, CdWork w,
         const int o = w.poff[a] + c0;
         w.poff[a] = o;
         emit_pairs<DIM, false>(g, w, io.pos, io.radius, a, o, start);
-        if (!io.detect_only) atomicAdd(&w.p2c_cnt[a], w.pcnt[a]);
+        if (!DETECT_ONLY) atomicAdd(&w.p2c_cnt[a], w.pcnt[a]);
     }
     if (blk == nb - 1 && threadIdx.x == 0) w.poff[n] = nc;
     __syncthreads();
     for (int c = c0 + (int)threadIdx.x; c < c1; c += PREP_THREADS) {
         geometry_warm<DIM>(g, w, c, nold, by_particle, io.pos, io.radius, io.inv_m, io.inv_I, io.warm, io.pw);
         const int b = w.pairs_nx[c].y;
-        if (!io.detect_only && cd_is_body(g, b)) atomicAdd(&w.p2c_cnt[b], 1);
+        if (!DETECT_ONLY && cd_is_body(g, b)) atomicAdd(&w.p2c_cnt[b], 1);
     }
     if (!sync()) return;
 
@@ -232,7 +230,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 1) k_prepare(CdGeom g, CdWork w,
         ctrl->nc = nc;
         ctrl->prev_offsets = (w.poff_prev != nullptr);
     }
-    if (io.detect_only) return;
+    if (DETECT_ONLY) return;
 
     // contacts of each body in ascending order: those in which it is body b,
     // then its own
@@ -378,8 +376,38 @@ __global__ void __launch_bounds__(PREP_THREADS, 1) k_prepare(CdGeom g, CdWork w,
     }
 }
 
-static const void* prep_fn(int dim, int precision)
+template <int DIM, typename T>
+__global__ void __launch_bounds__(PREP_THREADS, 1) k_prepare(CdGeom g, CdWork w, CdPrepIO io, int cluster)
 {
+    extern __shared__ int s_dyn[];   // the counting pass's queues and runs
+    __shared__ PrepShared sh;
+    if (w.ctrl->skip) return;
+    prepare<DIM, T, false>(g, w, io, cluster, s_dyn, sh);
+}
+
+// The contact set alone, on a grid that the device laid out.
+template <int DIM>
+__global__ void __launch_bounds__(PREP_THREADS, 1) k_detect(CdGeom given, CdWork w, CdPrepIO io, int cluster)
+{
+    extern __shared__ int s_dyn[];
+    __shared__ PrepShared sh;
+    __shared__ CdGeom g;   // (a changed copy in registers would go to local memory)
+    if (w.ctrl->skip || io.grid->status != CDG_OK) return;
+    if (threadIdx.x == 0) g = given;
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        g.cs[threadIdx.x] = io.grid->cs[threadIdx.x];
+        g.inv_cs[threadIdx.x] = io.grid->inv_cs[threadIdx.x];
+        g.ncell[threadIdx.x] = io.grid->ncell[threadIdx.x];
+    }
+    if (threadIdx.x == 3) g.ncell_total = io.grid->total;
+    __syncthreads();
+    prepare<DIM, double, true>(g, w, io, cluster, s_dyn, sh);
+}
+
+static const void* prep_fn(int dim, int precision, int detect_only)
+{
+    if (detect_only) return dim == 2 ? (const void*)k_detect<2> : (const void*)k_detect<3>;
     if (dim == 2) return precision == CD_FP64 ? (const void*)k_prepare<2, double> : (const void*)k_prepare<2, float>;
     return precision == CD_FP64 ? (const void*)k_prepare<3, double> : (const void*)k_prepare<3, float>;
 }
@@ -415,15 +443,17 @@ static cudaLaunchConfig_t prep_config(int dim, int blocks, int cluster, cudaLaun
 // kernels: 2D 1,000 discs 105 / 115 / 155 us, 5,000 111 / 118 / 165, 10,000
 // 129 / 127 / 175, 40,000 185 / 144 / 191; 3D 1,000 spheres 162 / 169 / 222,
 // 5,000 188 / 192 / 242, 20,000 307 / 205 / 261, 50,000 544 / 228 / 290.
-CdPrepPlan cd_prepare_plan(int dim, int precision, int64_t n, int device)
+int cd_prepare_cluster_n(int dim) { return dim == 2 ? 7000 : 5000; }
+
+CdPrepPlan cd_prepare_plan(int dim, int precision, int detect_only, int64_t n, int device)
 {
     CdPrepPlan plan = {0, 0};
-    const void* f = prep_fn(dim, precision);
+    const void* f = prep_fn(dim, precision, detect_only);
     const size_t bytes = prep_shared_bytes(dim);
     cudaLaunchAttribute a[1];
     int b = 0, sms = 0;
     if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return plan;
-    if (n <= (dim == 2 ? 7000 : 5000) &&
+    if (n <= cd_prepare_cluster_n(dim) &&
         cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
         const cudaLaunchConfig_t c = prep_config(dim, PREP_CLUSTER, 1, a);
         if (cudaOccupancyMaxActiveClusters(&b, f, &c) == cudaSuccess && b >= 1) return {PREP_CLUSTER, 1};
@@ -451,5 +481,5 @@ cudaError_t cd_launch_prepare(const CdGeom& g, const CdWork& w, const CdPrepIO& 
     cudaLaunchConfig_t c = prep_config(g.dim, blocks, cluster, a);
     c.stream = s;
     ++*nl;
-    return cudaLaunchKernelExC(&c, prep_fn(g.dim, precision), args);
+    return cudaLaunchKernelExC(&c, prep_fn(g.dim, precision, io.grid != nullptr), args);
 }
