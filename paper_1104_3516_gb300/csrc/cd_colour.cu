@@ -112,12 +112,35 @@ __device__ __forceinline__ void warp_atomic_max(int* dst, int key, int v, bool a
     if (active && (threadIdx.x & 31) == __ffs(grp) - 1) atomicMax(&dst[key], m);
 }
 
+// The largest v >= -1 of the block, one atomicMax for it.
+__device__ __forceinline__ void block_atomic_max(int* dst, int v)
+{
+    __shared__ int s_max;
+    if (threadIdx.x == 0) s_max = -1;
+    __syncthreads();
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_max, v);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(dst, s_max);
+}
+
+// The highest colour and the most contacts at a body, of each packing.  (A
+// plain system knows the colour already, and takes an atomic a block: one a
+// warp on one address took 25 us of a million spheres' step.)
 __global__ void k_rep_scan_colours(CdGeom g, CdWork w)
 {
     if (w.ctrl->skip) return;
     const int nc = w.ctrl->nc;
     const int nbody = g.n + (g.dyn_walls ? 6 : 0);
     const int st = gridDim.x * blockDim.x;
+    if (g.npk == 1) {
+        int d = 0;
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nbody; i += st)
+            d = max(d, w.p2c_off[i + 1] - w.p2c_off[i]);
+        block_atomic_max(w.rep_dmax, d);
+        if (blockIdx.x == 0 && threadIdx.x == 0) w.rep_top[0] = w.ctrl->ncolours - 1;
+        return;
+    }
     // whole warps iterate together (the warp collectives need every lane)
     for (int c0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); c0 < nc; c0 += st) {
         const int c = c0 + (threadIdx.x & 31);
@@ -168,21 +191,27 @@ __global__ void k_rep_run(CdGeom g, CdWork w)
     if (rep_wanted(c1 - c0, t, w.rep_dmax[b], l1 - l0)) rep_run(g, w, t, l0, l1, c1 - c0, w.rep_path + c0);
 }
 
-__global__ void k_rep_ncolours_reset(CdCtrl* ctrl)
+// Whether the repair ran on the plain system (whose colours then are counted anew).
+__device__ __forceinline__ bool rep_ran(const CdWork& w, int nc)
 {
-    if (!ctrl->skip) ctrl->ncolours = 0;
+    return rep_wanted(nc, w.rep_top[0], w.rep_dmax[0], w.rep_pos[nc] - w.rep_pos[0]);
 }
 
-__global__ void k_rep_ncolours(CdWork w)
+__global__ void k_rep_ncolours_reset(CdGeom g, CdWork w)
+{
+    if (w.ctrl->skip) return;
+    if (g.npk > 1 || rep_ran(w, w.ctrl->nc)) w.ctrl->ncolours = 0;
+}
+
+__global__ void k_rep_ncolours(CdGeom g, CdWork w)
 {
     if (w.ctrl->skip) return;
     const int nc = w.ctrl->nc;
-    // warps step together (uniform bound); one atomic per warp
-    for (int c0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); c0 < nc; c0 += gridDim.x * blockDim.x) {
-        const int c = c0 + (threadIdx.x & 31);
-        const int top = __reduce_max_sync(0xffffffffu, c < nc ? w.colour[c] + 1 : 0);
-        if ((threadIdx.x & 31) == 0) atomicMax(&w.ctrl->ncolours, top);
-    }
+    if (g.npk == 1 && !rep_ran(w, nc)) return;
+    int top = 0;
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x)
+        top = max(top, w.colour[c] + 1);
+    block_atomic_max(&w.ctrl->ncolours, top);
 }
 
 static cudaError_t launch_repair(const CdGeom& g, const CdWork& w, int gc, cudaStream_t s, int* nl)
@@ -203,8 +232,8 @@ static cudaError_t launch_repair(const CdGeom& g, const CdWork& w, int gc, cudaS
     k_rep_fill<<<gc, CD_BLOCK, 0, s>>>(w);
     // one warp per packing: a plain system's repair is one sequential walk
     k_rep_run<<<(g.npk + 1) / 2, 64, 0, s>>>(g, w);
-    k_rep_ncolours_reset<<<1, 1, 0, s>>>(w.ctrl);
-    k_rep_ncolours<<<gc, CD_BLOCK, 0, s>>>(w);
+    k_rep_ncolours_reset<<<1, 1, 0, s>>>(g, w);
+    k_rep_ncolours<<<gc, CD_BLOCK, 0, s>>>(g, w);
     *nl += 4;
     return cudaGetLastError();
 }
