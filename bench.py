@@ -165,12 +165,21 @@ def host_cpu():
     return {"cpu": model or platform.processor() or platform.machine(), "nproc": os.cpu_count()}
 
 
+def solve_kernel(dim, precision, max_sweeps, merge_last_colour=4, shape=None):
+    """The kernel that solves a plain system (cd_create_system's rule)."""
+    shape = shape or {}
+    flow = (max_sweeps > 128 and merge_last_colour in (0, 4) and shape.get("sweep_threads", 512) == 512
+            and shape.get("sweep_blocks_per_sm", 1) == 1)
+    return f"{'k_flow' if flow else 'k_sweep'}<{dim},{'double' if precision == 'f64' else 'float'}>"
+
+
 def profiled_traffic(kernel, precision, n):
     """DRAM bytes per launch from the committed ncu summary, or None if the
-    sweep kernel's source changed since the counters were taken."""
+    kernel's source changed since the counters were taken."""
     import hashlib
     try:
-        src = open(os.path.join(ROOT, "paper_1104_3516_gb300", "csrc", "cd_sweep.cu"), "rb").read()
+        name = "cd_flow.cu" if kernel.startswith("k_flow") else "cd_sweep.cu"
+        src = open(os.path.join(ROOT, "paper_1104_3516_gb300", "csrc", name), "rb").read()
         sha = hashlib.sha256(src).hexdigest()[:16]
         for line in open(os.path.join(ROOT, "profiles", "k_sweep_traffic.txt")):
             if line.startswith("#") or not line.strip():
@@ -456,10 +465,9 @@ def run_ours(args):
     steps_per_s = steps_sum / (dev_ms_max / 1e3)
 
     peak, peak_kind = peaks()
-    kname = "k_sweep"
+    kname = solve_kernel(wl.dim, args.precision, wl.max_sweeps, args.merge_last_colour, shape)
     if list(args.domains) != [1, 1, 1]:
-        kname = "k_sweep_domains"
-    kname += f"<{wl.dim},{'double' if args.precision == 'f64' else 'float'}>"
+        kname = kname.replace("k_sweep", "k_flow").replace("<", "_domains<")   # by dataflow, whatever the cap
     sweep_s = ph["sweep"] / 1e3
     gbs = sweep_bytes / sweep_s / 1e9 if sweep_s > 0 else 0.0
     hbm_view = {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
@@ -559,7 +567,8 @@ def run_fp32(args, wl, device, flush, shape):
            "mean_phases_per_sweep": float(np.mean(t["phases"])),
            "phase_ms_per_step": {k: v / args.steps for k, v in t["ph"].items()},
            "roofline": {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
-                        "kernel": "k_sweep<2,float>", "peak_source": f"{peak_kind} HBM copy bandwidth",
+                        "kernel": solve_kernel(2, "f32", wl.max_sweeps, args.merge_last_colour, shape),
+                        "peak_source": f"{peak_kind} HBM copy bandwidth",
                         "bytes_model": f"per sweep {bpc} B x contacts + {bpp} B x particles",
                         "note": "the pile is L2-resident: the sweep is bound by the latency of its colour phases, "
                                 "not by HBM"},
@@ -725,7 +734,7 @@ def run_sphere_gas(args, device, flush):
     tf = FLOPS_PER_UPDATE_3D * upd / sweep_s / 1e12 if sweep_s > 0 else 0.0
     bpc, bpp = sweep_bytes_model(3, "f64")
     roofline = {"bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": tf / FP64_PEAK_TFLOPS, "kernel": "k_sweep<3,double>",
+                "frac": tf / FP64_PEAK_TFLOPS, "kernel": solve_kernel(3, "f64", wl.max_sweeps),
                 "peak_source": "FP64 unit count x clock (152 SMs x 2 FMA/clk x 2 x 2.07 GHz)",
                 "flops_model": f"{FLOPS_PER_UPDATE_3D} FP64 flops per contact update",
                 "avg_launch_ms": ph["sweep"] / args.sphere_steps,

@@ -122,6 +122,15 @@ __device__ __forceinline__ double two(double a, double x, double c, double y)
     return __fma_rn(a, x, __dmul_rn(c, y));
 }
 
+// |(x, y)| for the sweep's sums: off the FP64 pipe, except where a square
+// leaves the range or a component is not finite.  There the square root, with
+// its overflow and NaN, tells the test that the iteration diverged.
+__device__ __forceinline__ double adj_abs(double x, double y)
+{
+    const int e = max(exponent_of(x), exponent_of(y));
+    return (e < 543 || e > 1500) && e != 0 ? sqrt(x * x + y * y) : abs_of_pair(x, y);
+}
+
 // A non-open contact's data that no sweep changes.
 struct AdjContact {
     int2 ab;
@@ -464,8 +473,8 @@ k_adjoint(CdGeom g, CdWork w, CdTape t, CdAdjIO io, double alpha, int max_sweeps
                     B.store(pb);
                 }
                 w.adj_Y[p] = Y;
-                ay += abs_of_pair(Y.x, Y.y);
-                ad += abs_of_pair(dY.x, dY.y);
+                ay += adj_abs(Y.x, Y.y);
+                ad += adj_abs(dY.x, dY.y);
             }
             // Lambda follows in its own record, which nobody else waits for now
             pa = act ? adj_lambda(w, c.ab.x) : nullptr;

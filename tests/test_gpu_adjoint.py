@@ -294,6 +294,21 @@ def test_backward_uses_the_tape_only_as_the_forward_left_it(between):
         assert all(torch.equal(a, b) for a, b in zip(got, want))
 
 
+@pytest.mark.parametrize("value", [np.nan, -np.nan, np.inf])
+def test_gradients_that_are_not_finite_are_reported_as_diverged(value):
+    """And those of the steps before, which then are not finite either."""
+    from paper_1104_3516_gb300 import cd
+    wl = colliding_gas(n=100, phi=0.62, vsig=3.0, dt=0.02)
+    g = cd.CDSystem(wl, device="cuda:0", criterion=cd.CD_CONV_GLOBAL_REL, alpha=FWD_ALPHA, max_sweeps=MAX_SWEEPS,
+                    tape_steps=3)
+    g.step(3)
+    gx, gv, gw = g.pos * 0.0, g.vel * 0.0 + value, g.omega * 0.0
+    for _ in range(3):
+        gx, gv, gw, st = g.adjoint_step(gx, gv, gw, ADJ_ALPHA, 1000)
+        if st["n_stick"] + st["n_slide"] > 0:
+            assert st["diverged"] == 1 and st["converged"] == 0
+
+
 def test_gpu_adjoint_settling_10k_against_finite_differences():
     """The differentiated settling rollout at full size: 10,000 discs, 200
     steps, checkpoints every 20; L = floor pressure of the last step + the
