@@ -649,14 +649,9 @@ def run_batched(args, device, rank, flush, ws=1):
         b.max_sweeps = args.max_sweeps
         b.alpha = args.alpha
     prec = cd.CD_FP64 if args.precision == "f64" else cd.CD_FP32
+    # the default block shape, whose schedule is chosen for each solve: the tuner times solves of 40 sweeps, of
+    # which laying out the teams is a quarter
     shape, tuned = {}, None
-    if not args.no_autotune:
-        from paper_1104_3516_gb300 import autotune
-        shape, table = autotune.tune(batch[0], batch=batch, precision=prec, device=device, steps=1,
-                                     max_contacts=6 * sum(b.n for b in batch),
-                                     candidates=[dict(sweep_threads=t, sweep_blocks_per_sm=b)
-                                                 for t, b in autotune.BLOCK_SHAPES])
-        tuned = {"choice": shape, "ms_per_sweep": [[c, m] for c, m in table]}
     # steps replayed from a captured CUDA graph (use_graph needs its own stream and timing 0);
     # the batch's working set (~1 GB) is larger than L2, so the steps run back to back
     stream = torch.cuda.Stream(device=device)

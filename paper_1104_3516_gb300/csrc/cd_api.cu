@@ -401,14 +401,13 @@ static cd_status launch_solve(cd_system* s, int free_flight, int timed)
         CD_CUDA(s, cd_launch_flow_batch(s->g, s->w, s->num_sms, s->flow_records, (int)s->p.precision,
                                         (int)s->p.criterion, s->p.alpha, (int)s->p.max_sweeps, s->stream,
                                         &s->launches));
-        return CD_OK;
-    }
-    if (s->g.flow) {
+    } else if (s->g.flow) {
         CD_CUDA(s, cd_launch_flow(s->g, s->w, solve_unpacks(s) ? io : CdState{nullptr, nullptr, nullptr, nullptr, 0},
                                   s->num_sms, s->flow_records, (int)s->p.precision, (int)s->p.criterion, s->p.alpha,
                                   (int)s->p.max_sweeps, s->stream, &s->launches));
         return CD_OK;
     }
+    // (for a batch with dataflow: the solves that its plan leaves to the barriers)
     CD_CUDA(s, cd_launch_sweep(s->g, s->w, s->sweep_blocks, s->sweep_threads, (int)s->p.precision,
                                (int)s->p.criterion, s->p.alpha,
                                (int)s->p.max_sweeps, s->pw, s->stream, &s->launches));

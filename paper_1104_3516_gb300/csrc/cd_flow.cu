@@ -42,6 +42,7 @@
 #define FLOW_WORKERS 11                           // warps that update contacts
 #define FLOW_THREADS (32 * (FLOW_WORKERS + 1))    // and one that runs the convergence test
 #define FLOW_LEAST 112                            // contacts that a block of a batched system is given at least
+#define FLOW_BARRIER_CONTACTS 30000               // see flow_leaves_batch
 #define FLOW_ROWS 8                               // rows of tagged block sums: while a block leaves those of pass p
                                                   // another may still wait for those of p - 5
 #define FLOW_SLOTS 4                              // passes whose residual terms are kept
@@ -897,9 +898,11 @@ k_flow(CdGeom g, CdWork w, CdState io, int crit, double alpha, int max_sweeps, i
 // blocks as any packing left asks for: none is left over.)  One step from zero
 // forces against the barrier schedule, which swept all packings together and
 // summed each one's |P| in a single block: 8 packings 45.5 -> 12.8 ms, 23 57.8
-// -> 18.0, 64 94 -> 53, 128 144 -> 102, 300 352 -> 238; from 64 on the FP64 pipe
+// -> 18.0, 64 94 -> 54, 128 144 -> 102, 300 352 -> 238; from 64 on the FP64 pipe
 // bounds it (128: 67 ms).  Cut always, or only for a whole half: 300 packings
-// 370 and 252 ms, 128 106 and 110.
+// 370 and 252 ms, 128 106 and 110.  A reserve of 32 contacts for every colour in
+// place of 128 for all: the fourth step of 64 packings, whose most crowded disc
+// has 29 contacts, 379 ms against 173 (285 with barriers).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int flow_ask(const CdWork& w, int b, int target, int blocks)
 {
@@ -908,16 +911,33 @@ __device__ __forceinline__ int flow_ask(const CdWork& w, int b, int target, int 
     return ask < 1 ? 1 : (ask > blocks ? blocks : ask);
 }
 
+// Whether a batch is left to the barrier schedule.  A block works on one packing
+// at a time, so with many colours (a disc squeezed between many: piles whose
+// solves hit the sweep cap) it has too few contacts of each to fill the FP64
+// pipe; a large batch has enough of all packings together.  One step,
+// dataflow / barriers: 512 packings (70,000 contacts a block) of 8 colours 379 /
+// 559 ms, 14 colours 759 / 832, 23 colours 1,386 / 1,048, 38 colours 1,386 /
+// 1,039; 128 packings (17,500 a block) of 23 colours 307 / 361, 36 colours 302 /
+// 410; 16 packings of 29 colours 46 / 189.
+__device__ __forceinline__ bool flow_leaves_batch(int K, int nc, int blocks)
+{
+    return K > 16 && nc > FLOW_BARRIER_CONTACTS * blocks;
+}
+
 __global__ void k_flow_plan(CdGeom g, CdWork w, int blocks, int records)
 {
     __shared__ int s_at[FLOW_MAX_BLOCKS + 1];   // packings that ask for i blocks, then the next place of theirs
     if (w.ctrl->skip) return;
     FlowPlan* plan = w.fl_plan;
+    const bool barriers = flow_leaves_batch(w.ctrl->ncolours, w.ctrl->nc, blocks);
+    if (threadIdx.x == 0) plan->barriers = barriers;
+    if (barriers) return;
     // all packings at once if the blocks' records can hold them so
     const int room = blocks > 2 * g.npk ? blocks - g.npk : blocks / 2;
     int target = (w.ctrl->nc + room - 1) / room;
-    // (dealt in warp items, a block may get one more than its share of every colour)
-    if (target > records - 32 * w.ctrl->ncolours) target = records - 32 * w.ctrl->ncolours;
+    // (dealt in warp items, remainders from another block on for each colour, a block may get a few
+    // more than its share; one that got too many would read them from memory)
+    if (target > records - 128) target = records - 128;
     if (target < FLOW_LEAST) target = FLOW_LEAST;
     for (int i = threadIdx.x; i < 2 * g.npk + 1; i += blockDim.x) w.fl_word[i] = 0u;
     for (int i = threadIdx.x; i <= blocks; i += blockDim.x) s_at[i] = 0;
@@ -990,7 +1010,7 @@ k_flow_batch(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec
     __shared__ FlowShared sh;
     __shared__ double s_red[FLOW_WORKERS + 1][3];
     CdCtrl* ctrl = w.ctrl;
-    if (ctrl->skip) return;
+    if (ctrl->skip || w.fl_plan->barriers) return;
     FlowPlan* plan = w.fl_plan;
     const int K = ctrl->ncolours, me = blockIdx.x, target = plan->target, placed = plan->placed;
     // the block's first team
@@ -1082,7 +1102,7 @@ __global__ void k_flow_totals(CdGeom g, CdWork w)
     __shared__ long long s_sum, s_upd, s_open;
     __shared__ int s_max;
     CdCtrl* ctrl = w.ctrl;
-    if (ctrl->skip || ctrl->error != CDE_NONE) return;
+    if (ctrl->skip || ctrl->error != CDE_NONE || w.fl_plan->barriers) return;
     if (threadIdx.x == 0) { s_sum = 0; s_upd = 0; s_open = 0; s_max = 0; }
     __syncthreads();
     for (int b = threadIdx.x; b < g.npk; b += blockDim.x) {

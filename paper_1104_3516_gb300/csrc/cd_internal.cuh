@@ -89,6 +89,7 @@ struct CdPack {
 // Batched systems by dataflow (cd_flow.cu): how the blocks form teams.
 #define FLOW_MAX_BLOCKS 512
 struct FlowPlan {
+    int barriers;               // 1: this solve is left to k_sweep_batch
     int target;                     // contacts a block is given
     int placed;                     // packings whose teams are laid out in advance
     int head[FLOW_MAX_BLOCKS + 1];  // packings that ask for g blocks: the next one of them to be taken,

@@ -727,7 +727,7 @@ k_sweep_batch(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps)
     __shared__ int s_off[CD_KMAX + 1];
     __shared__ double s_red[CD_SWEEP_THREADS / 32][3];
     CdCtrl* ctrl = w.ctrl;
-    if (ctrl->skip) return;
+    if (ctrl->skip || (g.flow && !w.fl_plan->barriers)) return;   // (solved by dataflow)
     const int nc = ctrl->nc;
     const int K = ctrl->ncolours;
     const int nb = gridDim.x;

@@ -185,3 +185,23 @@ def test_open_contacts_next_to_a_wild_velocity(dim, value, precision):
     xa, xb = a.state(), b.state()
     for k in ("v", "w"):
         assert np.array_equal(xa[k], xb[k], equal_nan=True), k
+
+
+@pytest.mark.parametrize("count", [100, 230])
+def test_batches_of_many_colours_are_bit_identical(count):
+    """A large disc among small ones: more than 16 colours.  230 packings
+    (5,000,000 contacts) are then left to the barrier schedule, 100 are not."""
+    wl = W.dense_biaxial_discs(seed=3, n=10000)
+    wl.r[5000] = 6.0
+    kw = dict(batch=[wl] * count, alpha=1e-6, max_sweeps=30, max_contacts=24000 * count)
+    a = gpu_system(wl, sweep_threads=256, sweep_blocks_per_sm=2, **kw)
+    b = gpu_system(wl, **kw)
+    sa, sb = a.step(1), b.step(1)
+    assert sb["last"]["n_colours"] > 16 and (sb["last"]["n_contacts"] > 30000 * 152) == (count == 230)
+    for k in ("total_sweeps", "total_contact_updates", "max_sweeps_in_step", "n_not_converged"):
+        assert sa[k] == sb[k], k
+    ca, cb = a.contacts(), b.contacts()
+    assert np.array_equal(ca["impulse"], cb["impulse"])
+    xa, xb = a.state(), b.state()
+    for k in ("x", "v", "w"):
+        assert np.array_equal(xa[k], xb[k]), k
