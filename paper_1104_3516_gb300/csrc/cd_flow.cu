@@ -1,5 +1,6 @@
 // cd_flow.cu -- the impulse solve as a dataflow over the contacts (plain
-// systems): the colour order without a grid barrier per colour.
+// systems, their domain-wise update, batches): the colour order without a grid
+// barrier per colour.
 //
 // The colour order says, for every body, in which order its contacts update
 // it.  Nothing else orders the updates: an update may run as soon as both its
@@ -15,8 +16,8 @@
 // A block keeps its contacts' records (impulse included) in shared memory for
 // the whole solve where they fit; a system too large for that reads them
 // through L1.  One more warp takes the block's residual terms, publishes their
-// sum, gathers the other blocks' and runs the convergence test.  Its ~5,000
-// cycles stay off the path: after the first sweeps a sweep starts before the
+// sum, gathers the other blocks' and runs the convergence test.  That stays off
+// the path: after the first sweeps a sweep starts before the
 // test of the one (then two) before it is known.  The impulses of the last
 // three sweeps are kept in turn, and the velocities from before the last two,
 // so the sweeps begun past the last one are taken back.
@@ -29,8 +30,8 @@
 // update (FP64: ~1,700 cycles for a whole warp of contacts; ~1,100 for 16
 // contacts split over lane pairs, where a block has few).  Per sweep, against
 // the barrier schedule (grid barrier 2,900 cycles a colour, then the velocity
-// loads): 100,000-disc pile FP64 28.4 -> 17.2 us, FP32 18.0 -> 10.2 us;
-// 5,000 discs FP64 20.6 -> 9.9 us; 2,000 discs 20.9 -> 10.1 us.  Tried and not kept: one lane
+// loads): 100,000-disc pile FP64 28.4 -> 17.3 us, FP32 18.0 -> 9.5 us;
+// 5,000 discs FP64 20.6 -> 9.7 us; 2,000 discs 18.0 -> 8.3 us.  Tried and not kept: one lane
 // looking for its warp (FP32 7% slower, 5,000 discs 12%), pauses between looks
 // (5,000 discs 2 to 15% slower), 15 or 7 updating warps in place of 11 (FP64 2
 // and 17% slower), records through L1 (FP64 pile 24.3 us a sweep), two far-apart

@@ -130,7 +130,7 @@ struct CdWork {
     int* p2c_fill;      // n
     int* p2c;           // 2 * cap
     unsigned long long* prio;  // cap colouring priorities
-    int* round_cnt;     // 3 counters of the colouring rounds
+    int* round_cnt;     // 3 change flags of the chain labelling (cd_merge.cu)
     int* chunk_cnt;     // CD_KMAX * nchunk_cap + 1; used as [colour][live chunk]
     int* colour_off;    // CD_KMAX + 1
     int* perm;          // colour position -> key index

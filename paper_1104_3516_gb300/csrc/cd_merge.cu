@@ -97,7 +97,7 @@ __global__ void k_mg_mark(CdGeom g, CdWork w, int M)
 
 // Minimum propagation along the links, one round per grid barrier, until no
 // label moves (labels only decrease, so reading a neighbour's label while it
-// changes is harmless).  round_cnt (free after the colouring) holds three
+// changes is harmless).  round_cnt holds three
 // rotating "moved" flags.
 __global__ void k_mg_label(CdGeom g, CdWork w, int* flag, int M)
 {

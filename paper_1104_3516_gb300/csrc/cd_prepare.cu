@@ -12,9 +12,9 @@
 // are a range of the key order and only those in which it is body b are
 // gathered and sorted; cell lists stay unsorted.
 //
-// Step of a 1,000-disc rollout 180 -> 101 us (of it this kernel 57 us, the
-// solve 47), 10,000 discs 175 -> 127, detection without workspace 151 -> 112
-// us.  The largest size that takes it: 3D step (150,000 / 400,000 / 1,000,000
+// Step of a 1,000-disc rollout 180 -> 101 us (of it this kernel 57 us; 84 us with
+// the shorter solve since), 10,000 discs 175 -> 127, detection without workspace
+// 151 -> 112 us (90 with the grid laid out on the device).  The largest size that takes it: 3D step (150,000 / 400,000 / 1,000,000
 // spheres) 393 -> 336, 1,018 -> 1,003, 2,319 -> 2,378 us: the walks of a
 // million spheres want the occupancy of kernels of their own.
 #include "cd_colour_core.cuh"

@@ -1,7 +1,8 @@
 // cd_sweep.cu -- the iterative contact-impulse solve (paper Sec. 2.1, Fig. 2)
 // and the Euler update (Eqs. 1-2).
 //
-// Long solves of plain systems run as a dataflow instead (cd_flow.cu).
+// Long solves of plain systems, the domain-wise update and most batches run as a
+// dataflow instead (cd_flow.cu).
 //
 // k_sweep is one cooperative persistent launch per solve: it applies the
 // starting impulses, then repeats sweeps over the colour classes (one grid
