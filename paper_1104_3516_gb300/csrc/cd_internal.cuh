@@ -361,9 +361,10 @@ __device__ __forceinline__ bool cd_is_parallel(double p, unsigned long long seed
 // below 2^31 within a round) and the low bits return to their old value.
 // Waiters compare the top bit with the value their own add returned.  The
 // spin is bounded by %globaltimer (CD_WAIT_NS) and also stops early when
-// another block has flagged an error; then it returns false (all threads of
-// the block) and the caller must leave the kernel.  The word must be zero at
-// launch (the launchers clear it).
+// another block's wait has run out; then it returns false (all threads of
+// the block) and the caller must leave the kernel.  (Other errors end no wait:
+// whoever flags one still arrives, and all blocks leave together behind the
+// barrier.)  The word must be zero at launch (the launchers clear it).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned long long cd_globaltimer()
 {
@@ -416,7 +417,7 @@ __device__ __forceinline__ bool cd_bar_wait(CdCtrl* ctrl, const unsigned* word, 
                     ok = 0;
                     break;
                 }
-                if (cd_ld_volatile_int(&ctrl->error) != CDE_NONE) { ok = 0; break; }
+                if (cd_ld_volatile_int(&ctrl->error) == CDE_TIMEOUT) { ok = 0; break; }
             }
         }
         // the acquire load that saw the flip orders thread 0's later accesses;

@@ -126,8 +126,9 @@ __host__ __device__ __forceinline__ int prep_shift(int count, int nb)
     return s;
 }
 
+// False when a barrier gave up: the step must not go on.
 template <int DIM, typename T, bool DETECT_ONLY>
-__device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const CdPrepIO& io, int cluster, int* s_dyn,
+__device__ __forceinline__ bool prepare(const CdGeom& g, const CdWork& w, const CdPrepIO& io, int cluster, int* s_dyn,
                                         PrepShared& sh)
 {
     CdCtrl* ctrl = w.ctrl;
@@ -156,25 +157,25 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
             if (i < nbody) w.p2c_fill[i] = 0;
         }
     }
-    if (!sync()) return;
+    if (!sync()) return false;
 
     // cell lists (in no order)
     for (int i = tid; i < n; i += stride) count_cell<DIM>(g, w, io.pos, io.radius, i, w.cell_of, w.cell_cnt);
     if (!DETECT_ONLY && io.pack)
         pack_velocities<DIM, T>(g, w, io.vel, io.omega, io.inv_m, io.f_ext, io.free_flight, tid, stride, blk == 0);
-    if (!sync()) return;
+    if (!sync()) return false;
     {
         const int t = prep_scan(w.cell_cnt, w.cell_start, cell0, cell1, sh);
         if (threadIdx.x == 0) tot[PREP_CELLS * nb + blk] = t;
     }
-    if (!sync()) return;
+    if (!sync()) return false;
     prep_before(tot + PREP_CELLS * nb, nb, sh.cells, sh);
     const PrepPrefix start{w.cell_start, sh.cells, cshift};
     for (int i = tid; i < n; i += stride) {
         const int c = w.cell_of[i];
         w.cell_pid[start[c] + atomicAdd(&w.cell_fill[c], 1)] = i;
     }
-    if (!sync()) return;
+    if (!sync()) return false;
 
     // contacts of the block's particles: counted, then written from the sum
     // of the blocks before on
@@ -190,7 +191,7 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
         const int t = prep_scan(w.pcnt, w.poff, part0, part1, sh);
         if (threadIdx.x == 0) tot[PREP_CONTACTS * nb + blk] = t;
     }
-    if (!sync()) return;
+    if (!sync()) return false;
     const int nc = prep_before(tot + PREP_CONTACTS * nb, nb, sh.p2c, sh);
     const int c0 = sh.p2c[blk], c1 = c0 + tot[PREP_CONTACTS * nb + blk];
     const bool fits = nc <= g.cap && cd_ld_volatile_int(&ctrl->error) == CDE_NONE;
@@ -201,7 +202,7 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
             ctrl->skip = 1;
         }
     }
-    if (!fits) return;
+    if (!fits) return true;
     for (int a = part0 + (int)threadIdx.x; a < part1; a += PREP_THREADS) {
         const int o = w.poff[a] + c0;
         w.poff[a] = o;
@@ -215,7 +216,7 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
         const int b = w.pairs_nx[c].y;
         if (!DETECT_ONLY && cd_is_body(g, b)) atomicAdd(&w.p2c_cnt[b], 1);
     }
-    if (!sync()) return;
+    if (!sync()) return false;
 
     // the new set becomes the current one
     for (int c = c0 + (int)threadIdx.x; c < c1; c += PREP_THREADS) {
@@ -230,7 +231,7 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
         ctrl->nc = nc;
         ctrl->prev_offsets = (w.poff_prev != nullptr);
     }
-    if (DETECT_ONLY) return;
+    if (DETECT_ONLY) return true;
 
     // contacts of each body in ascending order: those in which it is body b,
     // then its own
@@ -238,7 +239,7 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
         const int t = prep_scan(w.p2c_cnt, w.p2c_cnt, body0, body1, sh);
         if (threadIdx.x == 0) tot[PREP_P2C * nb + blk] = t;
     }
-    if (!sync()) return;
+    if (!sync()) return false;
     prep_before(tot + PREP_P2C * nb, nb, sh.p2c, sh);
     const PrepPrefix first{w.p2c_cnt, sh.p2c, bshift};
     for (int i = body0 + (int)threadIdx.x; i < body1; i += PREP_THREADS) w.p2c_off[i] = first[i];
@@ -247,7 +248,7 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
         w.p2c[first[ab.x + 1] - (w.poff[ab.x + 1] - c)] = c;
         if (cd_is_body(g, ab.y)) w.p2c[first[ab.y] + atomicAdd(&w.p2c_fill[ab.y], 1)] = c;
     }
-    if (!sync()) return;
+    if (!sync()) return false;
     for (int i = tid; i < nbody; i += stride) {
         const int b = w.p2c_off[i], e = w.p2c_off[i + 1] - ((i < n) ? w.poff[i + 1] - w.poff[i] : 0);
         for (int k = b + 1; k < e; ++k) {
@@ -257,10 +258,10 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
             w.p2c[j + 1] = v;
         }
     }
-    if (!jp_colour(g, w, nc, w.prio, sync)) return;
+    if (!jp_colour(g, w, nc, w.prio, sync)) return false;
     if (cd_ld_volatile_int(&ctrl->error) != CDE_NONE) {
         if (tid == 0) ctrl->skip = 1;
-        return;
+        return true;
     }
 
     // colours of the block's contacts, and whether the highest one is repaired
@@ -280,7 +281,7 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
         __syncthreads();
         for (int k = threadIdx.x; k < CD_KMAX; k += PREP_THREADS) w.prep_hist[k * nb + blk] = sh.hist[k];
         if (round == 0 && threadIdx.x == 0) tot[PREP_DEGREE * nb + blk] = sh.dmax;
-        if (!sync()) return;
+        if (!sync()) return false;
         if (round == 1) break;
         if (wid == 0) {
             int top = 0, dmax = 0;
@@ -320,7 +321,7 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
             __syncthreads();
             if (lane == 0) atomicMax(&ctrl->ncolours, k);
         }
-        if (!sync()) return;
+        if (!sync()) return false;
         K = cd_ld_volatile_int(&ctrl->ncolours);
     }
 
@@ -374,6 +375,7 @@ __device__ __forceinline__ void prepare(const CdGeom& g, const CdWork& w, const 
         }
         __syncthreads();
     }
+    return true;
 }
 
 template <int DIM, typename T>
@@ -382,7 +384,8 @@ __global__ void __launch_bounds__(PREP_THREADS, 1) k_prepare(CdGeom g, CdWork w,
     extern __shared__ int s_dyn[];   // the counting pass's queues and runs
     __shared__ PrepShared sh;
     if (w.ctrl->skip) return;
-    prepare<DIM, T, false>(g, w, io, cluster, s_dyn, sh);
+    // (any block that gave up says so: the one that reports the errors may have left first)
+    if (!prepare<DIM, T, false>(g, w, io, cluster, s_dyn, sh) && threadIdx.x == 0) w.ctrl->skip = 1;
 }
 
 // The contact set alone, on a grid that the device laid out.
@@ -402,7 +405,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 1) k_detect(CdGeom given, CdWork
     }
     if (threadIdx.x == 3) g.ncell_total = io.grid->total;
     __syncthreads();
-    prepare<DIM, double, true>(g, w, io, cluster, s_dyn, sh);
+    if (!prepare<DIM, double, true>(g, w, io, cluster, s_dyn, sh) && threadIdx.x == 0) w.ctrl->skip = 1;
 }
 
 static const void* prep_fn(int dim, int precision, int detect_only)

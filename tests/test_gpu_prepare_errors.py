@@ -1,0 +1,70 @@
+"""What the one-kernel preparation cannot take ends the step before the solve:
+more than 64 candidates at a disc, more than 64 colours, on one cluster of blocks
+and on the grid.  The state stays as it was, on the first step and after a good
+one, and the system steps on, equal to the separate kernels (timing = 1)."""
+import numpy as np
+import pytest
+
+from gpu_common import gpu_system, needs_gpu
+from paper_1104_3516_gb300 import cd, workloads as W
+
+pytestmark = [pytest.mark.gpu, needs_gpu]
+
+
+def ringed(n, large_first):
+    """n - 71 small discs apart from each other, and a large one (the first or
+    the last disc) in a ring of 70: on it in the second set of positions."""
+    ring = 70
+    ang = np.linspace(0.0, 2.0 * np.pi, ring, endpoint=False)
+    circle = np.stack([np.cos(ang), np.sin(ang)], 1)
+    side = int(np.ceil(np.sqrt(n)))
+    k = np.arange(n - ring - 1)
+    field = np.stack([30.0 + 1.3 * (k % side), 1.0 + 1.3 * (k // side)], 1)
+    centre = np.array([[12.0, 12.0]])
+    sets = [np.concatenate([centre, 12.0 + rad * circle, field]) for rad in (6.5, 5.3)]
+    r = np.concatenate([[5.0], np.full(ring, 0.2), np.full(len(field), 0.4)])
+    if not large_first:
+        sets, r = [np.roll(x, -1, axis=0) for x in sets], np.roll(r, -1)
+    inv_m, inv_I = W.masses(2, r)
+    wl = W.Workload(name="ringed", dim=2, x=sets[0], v=W.normal(1, 2 * n, 0.1).reshape(n, 2), w=np.zeros(n), r=r,
+                    inv_m=inv_m, inv_I=inv_I, box_hi=(1.3 * side + 40.0, 1.3 * side + 40.0, 1.0), wall_mask=0b0100)
+    return wl, sets
+
+
+def put(g, x, v):
+    import torch
+    for dst, a in ((g.pos, x), (g.vel, v)):
+        dst.copy_(torch.as_tensor(np.ascontiguousarray(a).reshape(-1), device=dst.device))
+
+
+def whole(g):
+    s = g.state()
+    return [s["x"], s["v"], s["w"], g.walls()]
+
+
+@pytest.mark.parametrize("n", [500, 20000])
+@pytest.mark.parametrize("large_first", [True, False])
+@pytest.mark.parametrize("kw", [{"max_sweeps": 20}, {"max_sweeps": 200}, {"max_sweeps": 200, "domains": (2, 2, 1)}])
+@pytest.mark.parametrize("good_first", [False, True])
+def test_a_step_that_cannot_be_prepared_leaves_the_state(n, large_first, kw, good_first):
+    wl, (good, bad) = ringed(n, large_first)
+    words = "64 contact candidates" if large_first else "64 colours"
+    one, apart = gpu_system(wl, **kw), gpu_system(wl, timing=1, **kw)
+    for g in (one, apart):
+        if good_first:
+            g.step(1)
+        put(g, bad, wl.v)
+        before = whole(g)
+        for _ in range(2):
+            with pytest.raises(cd.CDError, match=words) as e:
+                g.step(2)
+            assert e.value.status == cd.CD_ERR_CAPACITY
+        for a, b in zip(before, whole(g)):
+            assert np.array_equal(a, b)
+        put(g, good, wl.v)
+        g.step(2)
+    for a, b in zip(whole(one), whole(apart)):
+        assert np.array_equal(a, b)
+    a, b = one.contacts(), apart.contacts()
+    for k in a:
+        assert np.array_equal(a[k], b[k]), k
