@@ -242,11 +242,16 @@ static size_t layout(cd_system* s, char* base, CdWork* w)
 // ---------------------------------------------------------------------------
 // Helpers
 // ---------------------------------------------------------------------------
-__global__ void k_begin_call(CdCtrl* ctrl, int reset_accum)
+// solve: the call uses the colour order as it is.
+__global__ void k_begin_call(CdCtrl* ctrl, int reset_accum, int solve = 0)
 {
     ctrl->skip = 0;
     ctrl->overflow = 0;
     ctrl->error = CDE_NONE;
+    if (solve && (ctrl->order_lost || ctrl->order_nc != ctrl->nc)) {
+        ctrl->skip = 1;
+        ctrl->error = CDE_ORDER;
+    }
     if (reset_accum) {
         ctrl->steps_done = 0;
         ctrl->total_sweeps = 0;
@@ -259,6 +264,7 @@ __global__ void k_begin_call(CdCtrl* ctrl, int reset_accum)
 __global__ void k_error_gate(CdCtrl* ctrl)
 {
     if (ctrl->error != CDE_NONE) ctrl->skip = 1;
+    else if (!ctrl->skip) ctrl->order_nc = ctrl->nc;   // (the launches of the colour order end here)
 }
 
 // Records the next phase event on the system's stream (params.timing).
@@ -312,6 +318,8 @@ static cd_status ctrl_status(cd_system* s, const CdCtrl& h)
     if (h.error == CDE_TIMEOUT) return fail(s, CD_ERR_TIMEOUT, "a bounded device-side wait ran out");
     if (h.error == CDE_COLOURS) return fail(s, CD_ERR_CAPACITY, "the contact graph needs more than 64 colours");
     if (h.error == CDE_PER_PARTICLE) return fail(s, CD_ERR_CAPACITY, "a particle has more than 64 contact candidates");
+    if (h.error == CDE_ORDER)
+        return fail(s, CD_ERR_STATE, "the contact set has no colour order: detect or set the contacts again");
     if (h.error == CDE_TAPE) return fail(s, CD_ERR_STATE, "the recorded step had failed (contact overflow or timeout)");
     return CD_OK;
 }
@@ -842,7 +850,7 @@ extern "C" cd_status cd_solve_contacts(cd_system* s, cd_solve_stats* out)
     cd_status st = need_ready(s);
     if (st != CD_OK) return st;
     if (!s->has_contacts) return fail(s, CD_ERR_STATE, "no contact set: call cd_detect_contacts or cd_set_contacts");
-    k_begin_call<<<1, 1, 0, s->stream>>>(s->w.ctrl, 1);
+    k_begin_call<<<1, 1, 0, s->stream>>>(s->w.ctrl, 1, 1);
     if ((st = launch_solve(s, 0, 0)) != CD_OK) return st;
     if (!solve_unpacks(s))
         CD_CUDA(s, cd_launch_unpack(s->g, s->w, s->pos, s->vel, s->omega, s->theta, 0, (int)s->p.precision, s->stream,

@@ -314,6 +314,8 @@ __global__ void k_set_nc(CdCtrl* ctrl, int by_particle)
     if (ctrl->skip) return;
     ctrl->nc = ctrl->nc_needed;
     ctrl->prev_offsets = by_particle;
+    ctrl->order_nc = -1;
+    ctrl->order_lost = 0;
 }
 
 static int grid_for(int n, int per_block = CD_BLOCK)

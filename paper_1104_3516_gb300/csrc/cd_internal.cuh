@@ -18,7 +18,7 @@
 #define CD_MG_MIN_SWEEPS 64   // params.merge_last_colour 4: merge after solves of at least this many sweeps
 
 // Device error codes written into CdCtrl::error.
-enum { CDE_NONE = 0, CDE_TIMEOUT = 1, CDE_COLOURS = 2, CDE_PER_PARTICLE = 3, CDE_TAPE = 4 };
+enum { CDE_NONE = 0, CDE_TIMEOUT = 1, CDE_COLOURS = 2, CDE_PER_PARTICLE = 3, CDE_TAPE = 4, CDE_ORDER = 5 };
 
 // Control block at the start of the workspace.
 struct CdCtrl {
@@ -64,6 +64,10 @@ struct CdCtrl {
     int mg_prev;                    // sweeps + 1 of the last solve (0: none yet), for params.merge_last_colour 4
     int chunk_last;                 // colour partition: CD_KMAX x live chunks - 1 (the scan's extent)
     int chunk_pad;
+    // the colour order belongs to the current set: both, so that a solve by itself
+    // does not run on an order that was never finished
+    int order_nc;                   // contacts of the set that was ordered last (-1: the current one was not)
+    int order_lost;                 // 1: a block gave up while it was being prepared
 };
 
 // Parameters of one packing of a batched system (a plain system is a batch of

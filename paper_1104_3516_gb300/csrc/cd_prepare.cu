@@ -230,6 +230,8 @@ __device__ __forceinline__ bool prepare(const CdGeom& g, const CdWork& w, const 
     if (tid == 0) {
         ctrl->nc = nc;
         ctrl->prev_offsets = (w.poff_prev != nullptr);
+        ctrl->order_nc = -1;
+        ctrl->order_lost = 0;
     }
     if (DETECT_ONLY) return true;
 
@@ -354,6 +356,7 @@ __device__ __forceinline__ bool prepare(const CdGeom& g, const CdWork& w, const 
     __syncthreads();
     if (blk == 0)
         for (int k = threadIdx.x; k <= CD_KMAX; k += PREP_THREADS) w.colour_off[k] = sh.coff[k];
+    if (tid == 0) ctrl->order_nc = nc;   // (no barrier follows; a block that gave up at the last one has set order_lost)
     for (int i0 = c0; i0 < c1; i0 += PREP_THREADS) {
         for (int i = threadIdx.x; i < PREP_WARPS * CD_KMAX; i += PREP_THREADS) (&sh.wcnt[0][0])[i] = 0;
         __syncthreads();
@@ -384,8 +387,11 @@ __global__ void __launch_bounds__(PREP_THREADS, 1) k_prepare(CdGeom g, CdWork w,
     extern __shared__ int s_dyn[];   // the counting pass's queues and runs
     __shared__ PrepShared sh;
     if (w.ctrl->skip) return;
-    // (any block that gave up says so: the one that reports the errors may have left first)
-    if (!prepare<DIM, T, false>(g, w, io, cluster, s_dyn, sh) && threadIdx.x == 0) w.ctrl->skip = 1;
+    const bool ok = prepare<DIM, T, false>(g, w, io, cluster, s_dyn, sh);
+    if (threadIdx.x == 0 && !ok) {   // (any block that gave up says so: the one that reports the errors may have left first)
+        w.ctrl->skip = 1;
+        w.ctrl->order_lost = 1;
+    }
 }
 
 // The contact set alone, on a grid that the device laid out.

@@ -1,7 +1,8 @@
 """What the one-kernel preparation cannot take ends the step before the solve:
 more than 64 candidates at a disc, more than 64 colours, on one cluster of blocks
 and on the grid.  The state stays as it was, on the first step and after a good
-one, and the system steps on, equal to the separate kernels (timing = 1)."""
+one, and the system steps on, equal to the separate kernels (timing = 1).  A solve
+by itself refuses the set that was left without a colour order."""
 import numpy as np
 import pytest
 
@@ -68,3 +69,35 @@ def test_a_step_that_cannot_be_prepared_leaves_the_state(n, large_first, kw, goo
     a, b = one.contacts(), apart.contacts()
     for k in a:
         assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("n", [500, 20000])
+@pytest.mark.parametrize("timing", [0, 1])
+@pytest.mark.parametrize("max_sweeps", [20, 200])
+def test_a_set_without_a_colour_order_is_not_solved(n, timing, max_sweeps):
+    wl, (good, bad) = ringed(n, large_first=False)
+    g = gpu_system(wl, timing=timing, max_sweeps=max_sweeps)
+    put(g, bad, wl.v)
+    for fail in (lambda: g.step(1), g.detect_contacts):
+        with pytest.raises(cd.CDError, match="64 colours"):
+            fail()
+    before = whole(g)
+    g.load_checkpoint(g.save_checkpoint())   # counts as a set, and has no order either
+    with pytest.raises(cd.CDError, match="colour order") as e:
+        g.solve_contacts()
+    assert e.value.status == cd.CD_ERR_STATE
+    for a, b in zip(before, whole(g)):
+        assert np.array_equal(a, b)
+    # a checkpoint with more contacts than the set that was ordered last
+    put(g, good, wl.v)
+    more = g.detect_contacts()
+    saved = g.save_checkpoint()
+    put(g, np.concatenate([[[3.0, 25.0]], good[1:]]), wl.v)   # a disc of the ring alone
+    assert 0 < g.detect_contacts() < more
+    g.load_checkpoint(saved)
+    with pytest.raises(cd.CDError, match="colour order"):
+        g.solve_contacts()
+    assert g.detect_contacts() == more
+    g.solve_contacts()
+    g.load_checkpoint(saved)   # of the set that is in order
+    g.solve_contacts()
