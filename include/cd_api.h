@@ -365,7 +365,9 @@ cd_status cd_download_state(cd_system* sys, double* pos_host, double* vel_host, 
  * max_contacts*3 doubles, gap max_contacts doubles (may be NULL when
  * max_contacts is 0: a size query); *n_contacts (host) the number found.
  * Work is enqueued on cuda_stream, and every call synchronises that stream
- * (it reads the largest radius and the contact count back to the host).
+ * (it reads the contact count back to the host).  The kernel's blocks wait for
+ * one another with a bound: CD_ERR_TIMEOUT if it ran out, *n_contacts then as
+ * it was.
  *
  * Scratch lives in a fixed device array of about 4.4 MB inside the library,
  * held by every GPU that loads it until the process exits; limits: n <= 16384

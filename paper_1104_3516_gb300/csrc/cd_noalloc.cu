@@ -141,6 +141,26 @@ static cd_status na_cuda(cudaError_t e, const char* where)
     return CD_ERR_CUDA;
 }
 
+// What the call answers for what the device left behind (of the grid: CDG_*; of
+// the control block: CDE_*, overflow, the count).  Not in the public header:
+// apart from the call because the kernel's barriers have a bound, and what
+// follows when one runs out is checked without making one run out.  The count
+// is written where it is one.
+extern "C" cd_status cd_noalloc_outcome(int grid, int error, int overflow, int nc_needed, int64_t* n_contacts)
+{
+    if (grid == CDG_RADIUS) return na_error(CD_ERR_INVALID_ARG, "radius must be positive and finite");
+    if (grid == CDG_PERIODIC)
+        return na_error(CD_ERR_INVALID_ARG, "a periodic axis needs at least 3 cells (box >= 3 l)");
+    if (grid == CDG_CELLS)
+        return na_error(CD_ERR_INVALID_ARG, "the box needs more than 65536 cells for the no-allocation entry point");
+    if (error == CDE_TIMEOUT) return na_error(CD_ERR_TIMEOUT, "a bounded device-side wait ran out");
+    *n_contacts = nc_needed;
+    if (error == CDE_PER_PARTICLE) return na_error(CD_ERR_CAPACITY, "a particle has more than 64 contact candidates");
+    if (error != CDE_NONE) return na_error(CD_ERR_STATE, "the detection failed on the device");
+    if (overflow) return na_error(CD_ERR_CAPACITY, "more contacts than max_contacts; *n_contacts holds the number needed");
+    return CD_OK;
+}
+
 extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t n, const double* pos,
                                                 const double* radius, const double* inv_mass,
                                                 const double* inv_inertia, int64_t max_contacts, int32_t* pairs,
@@ -248,13 +268,5 @@ extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t
     CdGridSpec hg;
     memcpy(&h, back + NA_CTRL, sizeof h);
     memcpy(&hg, back + NA_GRID, sizeof hg);
-    if (hg.status == CDG_RADIUS) return na_error(CD_ERR_INVALID_ARG, "radius must be positive and finite");
-    if (hg.status == CDG_PERIODIC)
-        return na_error(CD_ERR_INVALID_ARG, "a periodic axis needs at least 3 cells (box >= 3 l)");
-    if (hg.status == CDG_CELLS)
-        return na_error(CD_ERR_INVALID_ARG, "the box needs more than 65536 cells for the no-allocation entry point");
-    *n_contacts = h.nc_needed;
-    if (h.error == CDE_PER_PARTICLE) return na_error(CD_ERR_CAPACITY, "a particle has more than 64 contact candidates");
-    if (h.overflow) return na_error(CD_ERR_CAPACITY, "more contacts than max_contacts; *n_contacts holds the number needed");
-    return CD_OK;
+    return cd_noalloc_outcome(hg.status, h.error, h.overflow, h.nc_needed, n_contacts);
 }

@@ -101,3 +101,16 @@ def test_a_set_without_a_colour_order_is_not_solved(n, timing, max_sweeps):
     g.solve_contacts()
     g.load_checkpoint(saved)   # of the set that is in order
     g.solve_contacts()
+
+
+@pytest.mark.parametrize("n", [500, 16000])
+def test_detection_without_workspace_counts_what_it_refuses(n):
+    from test_zz_no_alloc import _noalloc
+    wl, (good, bad) = ringed(n, large_first=True)
+    wl.x = bad
+    for _ in range(3):
+        with pytest.raises(cd.CDError, match="64 contact candidates") as e:
+            _noalloc(wl, 1000)
+        assert e.value.status == cd.CD_ERR_CAPACITY and e.value.needed == 140   # 70 on the large disc, 70 along the ring
+    wl.x = good
+    assert len(_noalloc(wl, 1000)[0]) == 70
