@@ -122,13 +122,12 @@ __device__ __forceinline__ double two(double a, double x, double c, double y)
     return __fma_rn(a, x, __dmul_rn(c, y));
 }
 
-// |(x, y)| for the sweep's sums: off the FP64 pipe, except where a square
-// leaves the range or a component is not finite.  There the square root, with
-// its overflow and NaN, tells the test that the iteration diverged.
+// |(x, y)| for the sweep's sums.  The square root (the forward solve's integer
+// form is up to 7.3e-15 off, which the residual would carry); its overflow and NaN
+// tell the test that the iteration diverged.
 __device__ __forceinline__ double adj_abs(double x, double y)
 {
-    const int e = max(exponent_of(x), exponent_of(y));
-    return (e < 543 || e > 1500) && e != 0 ? sqrt(x * x + y * y) : abs_of_pair(x, y);
+    return sqrt(x * x + y * y);
 }
 
 // A non-open contact's data that no sweep changes.

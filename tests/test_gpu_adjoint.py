@@ -524,3 +524,32 @@ def test_graph_replayed_steps_equal_direct_launches():
                     st["total_sweeps"]))
     for a, b in zip(out[0], out[1]):
         assert np.array_equal(np.asarray(a), np.asarray(b))
+
+
+def test_residual_of_one_contact_is_rounded_only():
+    """After one sweep of a sticking contact the residual is |Y| over the scale
+    m_n (|Gamma| + r |Gamma_w|).  To first order in u = 2^-53: Gamma 1 each, Y 4
+    (products, the difference, no cancellation), its magnitude 2 more, the scale 5,
+    the quotient 1: 12 u."""
+    import torch
+    from paper_1104_3516_gb300 import cd
+    wl = resting_disc(radius=1.3)
+    g = cd.CDSystem(wl, device="cuda:0", criterion=cd.CD_CONV_GLOBAL_REL, alpha=FWD_ALPHA, max_sweeps=MAX_SWEEPS,
+                    tape_steps=1)
+    start = g.save_checkpoint()
+    rng = np.random.default_rng(8)
+    L = np.longdouble
+    im, iI, r = float(wl.inv_m[0]), float(wl.inv_I[0]), float(wl.r[0])
+    mn, mt = 1.0 / im, 1.0 / (im + (r * r) * iI)
+    for _ in range(200):
+        cx, cy, cw = rng.uniform(0.1, 3.0, 3)
+        g.load_checkpoint(start)
+        g.step(1)
+        grads = [torch.tensor(c, dtype=torch.float64, device="cuda:0") for c in ([0.0, 0.0], [cx, cy], [cw])]
+        _, _, _, st = g.adjoint_step(*grads, 1e-300, 1)
+        assert st["n_stick"] == 1 and st["sweeps"] == 1
+        gx, gy, gw = L(im) * L(cx), L(im) * L(cy), L(iI) * L(cw)
+        Y = np.sqrt((L(mn) * gy) ** 2 + (L(mt) * (gx + L(r) * gw)) ** 2)
+        scale = L(mn) * (np.sqrt(gx * gx + gy * gy) + L(r) * gw)
+        ref = Y / max(Y, scale)
+        assert abs(L(st["residual"]) - ref) <= 12 * 2.0 ** -53 * ref, (cx, cy, cw, float(L(st["residual"]) / ref - 1))
