@@ -56,10 +56,11 @@
 #define FLOW_SPLIT 64
 
 // The blocks that solve a system (or a packing) together: nb of the grid from
-// block `start` on, this one the blk-th, with a barrier word of their own.
+// block `start` on, this one the blk-th, with a barrier word of their own.  The
+// first `work` of them have contacts; the others take part in the tests only.
 struct FlowTeam {
     unsigned* word;
-    int start, nb, blk;
+    int start, nb, blk, work;
     __device__ __forceinline__ bool sync(CdCtrl* ctrl) const
     {
         if (nb == 1) {
@@ -428,8 +429,8 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
     // |P| of an update is taken while the warp's next one waits (3D FP64 has no registers left for it)
     constexpr bool DEFER = (DIM == 2) || std::is_same<T, float>::value;
     CdCtrl* ctrl = w.ctrl;
-    const int nb = tm.nb;
-    const int tid = tm.blk * blockDim.x + threadIdx.x, stride = nb * blockDim.x;
+    const int nw = tm.work;
+    const int tid = tm.blk * blockDim.x + threadIdx.x, stride = tm.nb * blockDim.x;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     u64* VT = (u64*)w.fl_V;
     FlowSum* part = (FlowSum*)w.fl_part;
@@ -451,13 +452,14 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
                 // whole warp items, dealt so that the blocks' totals over the colours
                 // are even: colour k's remainder starts at another block
                 const int lo = k < K ? sh.lo[k] : 0, hi = k < K ? sh.end[k] : nview;
-                const int half = F64_2D && k < K && hi - lo <= FLOW_SPLIT * nb;
+                const int half = F64_2D && k < K && hi - lo <= FLOW_SPLIT * nw;
                 const int sh_item = half ? 4 : 5;
                 const unsigned items = (unsigned)(hi - lo + (1 << sh_item) - 1) >> sh_item;
-                const unsigned r = (unsigned)(k * 5 * nb >> 3) % (unsigned)nb;
-                const unsigned each = items / (unsigned)nb, rest = items % (unsigned)nb;   // (32-bit: items * nb might not fit)
-                const int i0 = (int)(each * tm.blk + (rest * tm.blk + r) / (unsigned)nb);
-                const int i1 = (int)(each * (tm.blk + 1) + (rest * (tm.blk + 1) + r) / (unsigned)nb);
+                const unsigned r = (unsigned)(k * 5 * nw >> 3) % (unsigned)nw;
+                const unsigned each = items / (unsigned)nw, rest = items % (unsigned)nw;   // (32-bit: items * nw might not fit)
+                const unsigned b = min(tm.blk, nw), e = min(tm.blk + 1, nw);
+                const int i0 = (int)(each * b + (rest * b + r) / (unsigned)nw);
+                const int i1 = (int)(each * e + (rest * e + r) / (unsigned)nw);
                 sh.lo[k] = min(lo + (i0 << sh_item), hi);
                 sh.end[k] = min(lo + (i1 << sh_item), hi);
                 sh.half[k] = half;
@@ -870,7 +872,7 @@ k_flow(CdGeom g, CdWork w, CdState io, int crit, double alpha, int max_sweeps, i
     CdCtrl* ctrl = w.ctrl;
     if (ctrl->skip) return;
     const int nc = ctrl->nc, K = ctrl->ncolours, nb = gridDim.x;
-    const FlowTeam tm{reinterpret_cast<unsigned*>(&ctrl->bar_count), 0, nb, (int)blockIdx.x};
+    const FlowTeam tm{reinterpret_cast<unsigned*>(&ctrl->bar_count), 0, nb, (int)blockIdx.x, nb};
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         sh.lo[k] = w.colour_off[k];
         sh.end[k] = w.colour_off[k + 1];
@@ -891,17 +893,22 @@ k_flow(CdGeom g, CdWork w, CdState io, int crit, double alpha, int max_sweeps, i
 // ---------------------------------------------------------------------------
 // Batched systems.  Packings share nothing, so each is solved by a team of its
 // own and stops by itself: no barrier and no residual pass over the others.  A
-// packing asks for a block per `target` contacts.  The largest packings' teams
-// are laid out in advance until the grid is full; a team that is done takes
-// the largest packing left that asks for no more blocks than it has, with as
-// many as that asks for, and what is left of the team the one after, if that
-// is half as many or more.  (The first part of a team so keeps at least as many
-// blocks as any packing left asks for: none is left over.)  One step from zero
+// packing asks for a block per `target` contacts and is spread over exactly as
+// many, whichever team takes it: the magnitudes are added up lane by lane, so
+// with another number of blocks the mean would end in other digits.  The largest
+// packings' teams are laid out in advance until the grid is full; a team that is
+// done takes the largest packing left that asks for no more blocks than it has.
+// What is left of the team becomes one of its own if it is a third as many or
+// more (the first part so keeps at least as many blocks as any packing left asks
+// for: none is left over); fewer stay, without contacts, since blocks once cut off
+// do not come back together for a large packing.  One step from zero
 // forces against the barrier schedule, which swept all packings together and
-// summed each one's |P| in a single block: 8 packings 45.5 -> 12.8 ms, 23 57.8
-// -> 18.0, 64 94 -> 54, 128 144 -> 102, 300 352 -> 238; from 64 on the FP64 pipe
-// bounds it (128: 67 ms).  Cut always, or only for a whole half: 300 packings
-// 370 and 252 ms, 128 106 and 110.  A reserve of 32 contacts for every colour in
+// summed each one's |P| in a single block: 8 packings 45.4 -> 12.6 ms, 23 57.6
+// -> 17.8, 64 94 -> 55, 128 150 -> 105, 300 356 -> 233, 512 537 -> 394; from 64 on
+// the FP64 pipe bounds it (128: 67 ms).  With the blocks left over given contacts
+// too, which depends on timing: 102, 228 and 379 for the last three.  Cut always:
+// 91, 352, 715; for a half or more: 106, 246, 407; for a whole: 109, 278, 469.  A
+// reserve of 32 contacts for every colour in
 // place of 128 for all: the fourth step of 64 packings, whose most crowded disc
 // has 29 contacts, 379 ms against 173 (285 with barriers).
 // ---------------------------------------------------------------------------
@@ -1029,7 +1036,7 @@ k_flow_batch(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec
     for (;;) {
         while (!given) {
             // the team of `slot` takes the next packing
-            const FlowTeam tm{&w.fl_word[slot], start, nb, me - start};
+            const FlowTeam tm{&w.fl_word[slot], start, nb, me - start, nb};
             if (tm.blk == 0 && threadIdx.x < 32) {
                 const int x = flow_take(plan, nb);
                 if (threadIdx.x == 0) *(volatile int*)&w.fl_mail[slot] = x;
@@ -1037,8 +1044,8 @@ k_flow_batch(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec
             if (!tm.sync(ctrl)) return;
             at = cd_ld_volatile_int(&w.fl_mail[slot]);
             if (at < 0) return;
-            int ask = flow_ask(w, w.fl_list[at], target, (int)gridDim.x);
-            if (2 * nb < 3 * ask) ask = nb;   // not worth a team of its own
+            const int ask = flow_ask(w, w.fl_list[at], target, (int)gridDim.x);
+            if (3 * nb < 4 * ask) break;   // what is left over is not worth a team of its own
             given = me < start + ask;
             if (given) {
                 nb = ask;
@@ -1050,8 +1057,8 @@ k_flow_batch(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec
         }
         given = false;
         slot = at;
-        const FlowTeam tm{&w.fl_word[slot], start, nb, me - start};
         const int b = w.fl_list[at];
+        const FlowTeam tm{&w.fl_word[slot], start, nb, me - start, flow_ask(w, b, target, (int)gridDim.x)};
         const int first = w.pk[b].first, count = w.pk[b].count;
         const int c0 = w.pk_coff[b], nc = w.pk_coff[b + 1] - c0;
         for (int k = threadIdx.x; k < K; k += blockDim.x) {
