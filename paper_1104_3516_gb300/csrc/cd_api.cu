@@ -740,7 +740,7 @@ static cd_status create_impl(const cd_params* params, int64_t npk, const int64_t
     }
     // one-kernel preparation of small plain systems (with timing the phases are
     // launched, and timed, one by one)
-    if (npk == 1 && !p.timing && n <= CD_PREP_MAX_N) s->prep = cd_prepare_plan((int)p.dim, (int)p.precision, 0, n, s->device);
+    if (npk == 1 && !p.timing) s->prep = cd_prepare_plan((int)p.dim, (int)p.precision, 0, n, g.ncell_total, s->device);
     *out = s;
     return CD_OK;
 }

@@ -520,11 +520,12 @@ struct CdPrepIO {
 #define CD_PREP_MAX_BLOCKS 256
 cudaError_t cd_launch_prepare(const CdGeom& g, const CdWork& w, const CdPrepIO& io, int blocks, int cluster,
                               int precision, cudaStream_t stream, int* nl);
-// Blocks of the one-kernel preparation for n particles (0: it does not fit the
-// device), and whether they form one cluster.
+// Blocks of the one-kernel preparation for n particles in a grid of `cells` (0: it
+// does not fit the device, or separate kernels are faster), and whether they
+// form one cluster.
 struct CdPrepPlan { int blocks, cluster; };
-int cd_prepare_cluster_n(int dim);   // particles up to which the plan is one cluster of blocks
-CdPrepPlan cd_prepare_plan(int dim, int precision, int detect_only, int64_t n, int device);
+int cd_prepare_cluster_n(int dim);   // particles up to which the plan for a small grid is one cluster of blocks
+CdPrepPlan cd_prepare_plan(int dim, int precision, int detect_only, int64_t n, int64_t cells, int device);
 #define CD_PREP_MAX_N 500000   // see cd_prepare.cu
 cudaError_t cd_launch_pack(const CdGeom& g, const CdWork& w, const double* vel, const double* omega,
                            const double* radius, const double* inv_m, const double* inv_I, const double* f_ext,

@@ -201,7 +201,7 @@ extern "C" cd_status cd_detect_contacts_noalloc(const cd_params* params, int64_t
         }
         base = (unsigned char*)na_addr[dev];
         CdPrepPlan& known = na_plan[dev][p.dim - 2][n <= cd_prepare_cluster_n((int)p.dim) ? 1 : 0];
-        if (!known.blocks) known = cd_prepare_plan((int)p.dim, CD_FP64, 1, n, dev);
+        if (!known.blocks) known = cd_prepare_plan((int)p.dim, CD_FP64, 1, n, CD_NOALLOC_MAX_CELLS, dev);
         plan = known;
     }
     if (!plan.blocks) return na_error(CD_ERR_CUDA, "the detection kernel does not fit on this device");

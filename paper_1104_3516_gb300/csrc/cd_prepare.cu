@@ -452,17 +452,27 @@ static cudaLaunchConfig_t prep_config(int dim, int blocks, int cluster, cudaLaun
 // kernels: 2D 1,000 discs 105 / 115 / 155 us, 5,000 111 / 118 / 165, 10,000
 // 129 / 127 / 175, 40,000 185 / 144 / 191; 3D 1,000 spheres 162 / 169 / 222,
 // 5,000 188 / 192 / 242, 20,000 307 / 205 / 261, 50,000 544 / 228 / 290.
+//
+// Few particles in a large box: the cells are cleared and scanned all the same,
+// by 16 SMs 512 a block at a time, or by all, against separate kernels that scan
+// 2,048 a block.  Steps of 1,000 discs in a box of 1e5 cells 95 / 94 / 217 us, 3e5 120
+// / 95 / 219, 1e6 159 / 103 / 219, 4e6 377 / 135 / 240, 1e7 1,623 / - / 219; 500,000
+// discs in 4e6 cells - / 463 / 485, 5e6 - / 519 / 490, 1e7 - / 646 / 541 (the chunks
+// of cells are powers of two: beyond 152 x 2^15 half the blocks have none).
+#define PREP_CLUSTER_CELLS (1 << 17)
+#define PREP_MAX_CELLS (1 << 22)
 int cd_prepare_cluster_n(int dim) { return dim == 2 ? 7000 : 5000; }
 
-CdPrepPlan cd_prepare_plan(int dim, int precision, int detect_only, int64_t n, int device)
+CdPrepPlan cd_prepare_plan(int dim, int precision, int detect_only, int64_t n, int64_t cells, int device)
 {
     CdPrepPlan plan = {0, 0};
+    if (n > CD_PREP_MAX_N || cells > PREP_MAX_CELLS) return plan;
     const void* f = prep_fn(dim, precision, detect_only);
     const size_t bytes = prep_shared_bytes(dim);
     cudaLaunchAttribute a[1];
     int b = 0, sms = 0;
     if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return plan;
-    if (n <= cd_prepare_cluster_n(dim) &&
+    if (n <= cd_prepare_cluster_n(dim) && cells <= PREP_CLUSTER_CELLS &&
         cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
         const cudaLaunchConfig_t c = prep_config(dim, PREP_CLUSTER, 1, a);
         if (cudaOccupancyMaxActiveClusters(&b, f, &c) == cudaSuccess && b >= 1) return {PREP_CLUSTER, 1};
