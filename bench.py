@@ -173,14 +173,31 @@ def solve_kernel(dim, precision, max_sweeps, merge_last_colour=4, shape=None):
     return f"{'k_flow' if flow else 'k_sweep'}<{dim},{'double' if precision == 'f64' else 'float'}>"
 
 
+def kernel_source(kernel):
+    """The source that the kernel is compiled from: its .cu file and, in the
+    order of their first mention, the files of csrc that it includes."""
+    import re
+    csrc = os.path.join(ROOT, "paper_1104_3516_gb300", "csrc")
+    todo, done, text = ["cd_flow.cu" if kernel.startswith("k_flow") else "cd_sweep.cu"], set(), b""
+    while todo:
+        name = todo.pop(0)
+        path = os.path.join(csrc, name)
+        if name in done or (done and not os.path.exists(path)):   # (the public header lies elsewhere: no code)
+            continue
+        done.add(name)
+        with open(path, "rb") as f:
+            src = f.read()
+        text += src
+        todo += [m.decode() for m in re.findall(rb'^\s*#\s*include\s+"([^"]+)"', src, flags=re.M)]
+    return text
+
+
 def profiled_traffic(kernel, precision, n):
     """DRAM bytes per launch from the committed ncu summary, or None if the
-    kernel's source changed since the counters were taken."""
+    kernel's source (headers included) changed since the counters were taken."""
     import hashlib
     try:
-        name = "cd_flow.cu" if kernel.startswith("k_flow") else "cd_sweep.cu"
-        src = open(os.path.join(ROOT, "paper_1104_3516_gb300", "csrc", name), "rb").read()
-        sha = hashlib.sha256(src).hexdigest()[:16]
+        sha = hashlib.sha256(kernel_source(kernel)).hexdigest()[:16]
         for line in open(os.path.join(ROOT, "profiles", "k_sweep_traffic.txt")):
             if line.startswith("#") or not line.strip():
                 continue
