@@ -98,7 +98,10 @@ __device__ __forceinline__ bool pair_touches(const GridV& v, double delta, const
 // below s + E; the relative roundings of d2, of s and of the threshold
 // itself are covered by the factors 1 + 2^-20.  An image chosen differently
 // near |d| = L/2 changes nothing: a periodic axis spans at least three cells,
-// so both images are farther apart than any contact distance.
+// so both images are farther apart than any contact distance.  Squares below
+// 2^-126 are rounded to multiples of 2^-149 instead, at most three of them: the
+// 2^-126 added to the threshold covers those (lengths below 1e-19; larger squares
+// than FP32 has are infinite on both sides, or far).
 template <int DIM>
 __device__ __forceinline__ bool pair_far_f32(const GridV& v, const float (&Lf)[3], float delta_f, const float4& pa,
                                              const float4& pb)
@@ -120,7 +123,7 @@ __device__ __forceinline__ bool pair_far_f32(const GridV& v, const float (&Lf)[3
     }
     const float s = pa.w + pb.w + delta_f;
     const float t = fmaf(s, 1.0f + 9.5367432e-7f, E) * (1.0f + 9.5367432e-7f);   // 1 + 2^-20
-    return d2 > t * t;
+    return d2 > fmaf(t, t, 1.1754944e-38f);   // 2^-126
 }
 
 // Gap of the particle at xa to wall k (k = 2 axis + side).  The coordinate is
