@@ -254,7 +254,7 @@ __global__ void k_set_tape_slot(CdCtrl* ctrl, int slot)
 }
 
 // The block's sum of x (lane sums in sh.acc[q]), left for the other blocks and
-// gathered from them: one warp.  The sums are exact, the same in every block.
+// gathered from them: one warp.  Every block adds the same sums in the same order.
 __device__ __forceinline__ bool adj_gather(CdCtrl* ctrl, AdjShared& sh, FlowSum* row, int q, unsigned tag)
 {
     const int lane = threadIdx.x & 31, nb = gridDim.x;

@@ -118,8 +118,8 @@ struct FlowControl {
 // The control warp: leaves the block's sum of a pass when the workers have
 // finished it, and decides the test of the first undecided pass when every
 // block's sum is there (whichever comes first: neither waits for the other).
-// Returns after a decision; false when a wait gave up.  The sums are exact, so
-// the same in every block.
+// Returns after a decision; false when a wait gave up.  Every block adds the same
+// sums in the same order, so all decide alike.
 __device__ __forceinline__ bool flow_control(CdCtrl* ctrl, FlowShared& sh, FlowSum* part, const FlowTeam& tm,
                                              FlowControl& fc, int nc, int crit, double alpha, int max_sweeps)
 {

@@ -9,8 +9,8 @@
 // of velocity and a 16-bit tag, the number of updates its body has had (modulo
 // 2^16).  Every element says by itself which update it belongs to, so a reader
 // that finds the tag it expects in all of them has that update's velocities:
-// no fence, no flag beside the data.  (A reader is at most one pass, 64
-// updates, behind a writer.)  Three numbers make a group: FP64 four elements
+// no fence, no flag beside the data.  (A reader is at most one pass behind a
+// writer: 64 updates, 65 of a particle that domains share.)  Three numbers make a group: FP64 four elements
 // (one 256-bit access), FP32 two (one 128-bit access); 2D has one group
 // (v_x, v_y, omega), 3D two (v, omega).
 // ---------------------------------------------------------------------------
@@ -172,9 +172,11 @@ __device__ __forceinline__ bool flow_wait(CdCtrl* ctrl, int* gave_up, const u64*
     return true;
 }
 
-// The sum of N values >= 0 a lane over the warp (in every lane), exact but for
-// the rounding at the end: as integers of 128 bits that share the largest
-// exponent, added a lane and then by limbs of 25 bits.  The FP64 pipe takes 64
+// The sum of N values >= 0 a lane over the warp (in every lane), as integers of
+// 128 bits that share the largest exponent, added a lane and then by limbs of 25
+// bits: of each term what is below 2^-116 of the largest one's binade is cut
+// off, and the sum is rounded once.  (Near the ends of the range FP64 adds.)  The
+// FP64 pipe takes 64
 // cycles an instruction, more while the workers use it; a pass's sums and test
 // took 9,000 cycles on it, longer than a pass of two colours (10,000 discs in
 // pyramids, 150 sweeps: 875 us, now 640).
