@@ -566,12 +566,14 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
     __syncthreads();
 
     int last = 0;   // last pass this warp has run
-    // FP32 with more items than warps: wait for the block's own colour before
+    // FP32: wait for the block's own colour before
     // looking.  The looks that find nothing fill the L1's request queue and hold
-    // up everything else there (100,000 discs: 15.4 -> 10.9 us a sweep).  FP64
-    // items take longer than that and gain from starting early (gated: 18.7 ->
-    // 21.3 us), and with one item a warp there is no queue.
-    const bool gate = sizeof(T) == 4 && Q > FLOW_WORKERS;
+    // up everything else there (100,000 discs: 15.4 -> 10.9 us a sweep; 20,000 discs, a
+    // warp or none an item: 11.6 -> 9.2; 10,000 spheres on a lattice, 11 contacts each, whose records
+    // are twice as long: 72 -> 31, behind barriers 63).  FP64
+    // items take longer than that and gain from starting early (100,000 discs gated:
+    // 18.7 -> 21.3 us).
+    constexpr bool gate = sizeof(T) == 4;
     if (nc > 0 && wid == FLOW_WORKERS) {
         FlowControl fc;
         do {
