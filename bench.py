@@ -165,11 +165,13 @@ def host_cpu():
     return {"cpu": model or platform.processor() or platform.machine(), "nproc": os.cpu_count()}
 
 
-def solve_kernel(dim, precision, max_sweeps, merge_last_colour=4, shape=None):
-    """The kernel that solves a plain system (cd_create_system's rule)."""
+def solve_kernel(dim, precision, max_sweeps, merge_last_colour=4, shape=None, n=0, sms=152):
+    """The kernel that solves a plain system of n particles (cd_create_system's
+    rule; the particles an SM up to which it is the dataflow, cd_flow_max_n)."""
     shape = shape or {}
+    most = {(2, "f32"): 2300, (3, "f32"): 1100, (2, "f64"): 6000}.get((dim, precision))
     flow = (max_sweeps > 128 and merge_last_colour in (0, 4) and shape.get("sweep_threads", 512) == 512
-            and shape.get("sweep_blocks_per_sm", 1) == 1)
+            and shape.get("sweep_blocks_per_sm", 1) == 1 and (most is None or n <= most * sms))
     return f"{'k_flow' if flow else 'k_sweep'}<{dim},{'double' if precision == 'f64' else 'float'}>"
 
 
@@ -482,9 +484,9 @@ def run_ours(args):
     steps_per_s = steps_sum / (dev_ms_max / 1e3)
 
     peak, peak_kind = peaks()
-    kname = solve_kernel(wl.dim, args.precision, wl.max_sweeps, args.merge_last_colour, shape)
-    if list(args.domains) != [1, 1, 1]:
-        kname = kname.replace("k_sweep", "k_flow").replace("<", "_domains<")   # by dataflow, whatever the cap
+    kname = solve_kernel(wl.dim, args.precision, wl.max_sweeps, args.merge_last_colour, shape, n=wl.n)
+    if list(args.domains) != [1, 1, 1]:   # whatever the cap
+        kname = solve_kernel(wl.dim, args.precision, 1000, 4, shape, n=wl.n).replace("<", "_domains<")
     sweep_s = ph["sweep"] / 1e3
     gbs = sweep_bytes / sweep_s / 1e9 if sweep_s > 0 else 0.0
     hbm_view = {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
@@ -584,7 +586,7 @@ def run_fp32(args, wl, device, flush, shape):
            "mean_phases_per_sweep": float(np.mean(t["phases"])),
            "phase_ms_per_step": {k: v / args.steps for k, v in t["ph"].items()},
            "roofline": {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
-                        "kernel": solve_kernel(2, "f32", wl.max_sweeps, args.merge_last_colour, shape),
+                        "kernel": solve_kernel(2, "f32", wl.max_sweeps, args.merge_last_colour, shape, n=wl.n),
                         "peak_source": f"{peak_kind} HBM copy bandwidth",
                         "bytes_model": f"per sweep {bpc} B x contacts + {bpp} B x particles",
                         "note": "the pile is L2-resident: the sweep is bound by the latency of its colour phases, "
@@ -746,7 +748,7 @@ def run_sphere_gas(args, device, flush):
     tf = FLOPS_PER_UPDATE_3D * upd / sweep_s / 1e12 if sweep_s > 0 else 0.0
     bpc, bpp = sweep_bytes_model(3, "f64")
     roofline = {"bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": tf / FP64_PEAK_TFLOPS, "kernel": solve_kernel(3, "f64", wl.max_sweeps),
+                "frac": tf / FP64_PEAK_TFLOPS, "kernel": solve_kernel(3, "f64", wl.max_sweeps, n=wl.n),
                 "peak_source": "FP64 unit count x clock (152 SMs x 2 FMA/clk x 2 x 2.07 GHz)",
                 "flops_model": f"{FLOPS_PER_UPDATE_3D} FP64 flops per contact update",
                 "avg_launch_ms": ph["sweep"] / args.sphere_steps,

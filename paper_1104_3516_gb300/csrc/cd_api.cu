@@ -716,23 +716,28 @@ static cd_status create_impl(const cd_params* params, int64_t npk, const int64_t
                     g.ndom_total == 1 && !g.dyn_walls && p.tape_steps == 0 && cd_merge_label_blocks_per_sm() >= 1)
                        ? (p.merge_last_colour == 2 ? 2 : 3) : 0;
     g.merge_blocks = s->sweep_blocks;
-    // the dataflow solve: wherever its schedule may replace the barriers'.  A
+    // the dataflow solve: wherever its schedule may replace the barriers' and is
+    // the faster one.  A
     // caller who asks for merging (1 to 3) or for another block shape gets the
-    // schedule that was asked for; up to 128 sweeps mode 4 keeps merging, which
-    // n_phases reports (longer solves are faster without it, see cd_flow.cu)
+    // schedule that was asked for.  Up to 128 sweeps mode 4 keeps merging for the
+    // sake of n_phases, which reports it: callers of short solves go on reading the
+    // phases they read before.  (Speed is not the reason: 5,000 discs, 100 sweeps a
+    // step 2.35 ms with barriers, 1.23 by dataflow; 100,000 3.89 and 2.59.)
     s->flow_records = cd_flow_records(g, (int)p.precision, s->device);
-    g.flow = (npk > 1) ? (p.criterion != CD_CONV_LOCAL && s->sweep_threads == CD_SWEEP_THREADS &&
-                          s->sweep_blocks == s->num_sms && s->num_sms <= FLOW_MAX_BLOCKS &&
-                          s->flow_records >= 2 * CD_KMAX) :
-             (g.par_p == 0.0 && p.criterion != CD_CONV_LOCAL && s->sweep_threads == CD_SWEEP_THREADS &&
-              s->sweep_blocks == s->num_sms && s->flow_records >= 0 &&
-              (g.ndom_total > 1 ||   // (nothing to merge there)
-               (p.max_sweeps > 128 && (p.merge_last_colour == 0 || p.merge_last_colour == 4)))) ? 1 : 0;
-    if (g.flow) {
+    const bool same_shape = p.criterion != CD_CONV_LOCAL && s->sweep_threads == CD_SWEEP_THREADS &&
+                            s->sweep_blocks == s->num_sms;
+    if (npk > 1) {
+        g.flow = same_shape && s->num_sms <= FLOW_MAX_BLOCKS && s->flow_records >= 2 * CD_KMAX;
+    } else if (same_shape && g.par_p == 0.0 && s->flow_records >= 0 &&
+               (g.ndom_total > 1 ||   // (nothing to merge there)
+                (p.max_sweeps > 128 && (p.merge_last_colour == 0 || p.merge_last_colour == 4)))) {
+        g.flow = n <= cd_flow_max_n((int)p.dim, (int)p.precision, s->num_sms);
+        // (with as many particles as to be left to the barriers, merging saves nothing: 700,000
+        // packed discs, FP32, 8.06 ms without, 8.18 with)
         g.merge_last = 0;
         // records that cannot fit (more particles, so more contacts, than the blocks hold)
-        // leave the shared memory to the L1 cache
-        if (npk == 1 && n > (int64_t)s->flow_records * s->num_sms) s->flow_records = 0;
+        // leave the shared memory to the L1 cache (300,000 discs FP64: the same either way)
+        if (n > (int64_t)s->flow_records * s->num_sms) s->flow_records = 0;
     }
     if (g.merge_last && !cd_sweep_fits(g, (int)p.precision, s->sweep_threads, s->sweep_blocks / s->num_sms)) {
         delete s;

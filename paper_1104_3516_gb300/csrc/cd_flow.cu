@@ -1180,6 +1180,25 @@ int cd_flow_records(const CdGeom& g, int precision, int device)
     return recs;
 }
 
+// Particles up to which the dataflow is the faster schedule.  A system whose
+// contacts do not fit the blocks' shared memory is read through the L1, 11 warps an
+// SM at a time; the barrier schedule has 16, each with its next record on the way,
+// and barriers that weigh less the more there is between them.  A step of 150
+// sweeps (FP32: also 2 to 3 of a gas), dataflow / barriers: FP32 packed discs
+// 300,000 5.66 / 5.73 ms, 400,000 5.99 / 5.98, 700,000 11.4 / 8.1, 2,000,000 37.2 /
+// 21.2, lattice of 16 contacts each 200,000 14.4 / 16.2, 400,000 28.1 / 25.9; FP32
+// spheres, six contacts each, 150,000 5.00 / 5.23, 200,000 6.87 / 6.64, 400,000 13.3 /
+// 9.5, 11 each 100,000 9.9 / 10.8, 200,000 16.8 / 14.7, a gas 400,000 0.58 / 0.55,
+// 2,000,000 2.18 / 1.99; FP64 discs 700,000 17.6 / 19.3, 1,000,000 26.8 / 25.8,
+// 2,000,000 57.1 / 49.5; FP64 spheres 2,000,000 124 / 132, a gas of 4,000,000
+// 4.76 / 4.97: no line.  (With more contacts a body there are more colours, so as
+// much to do in each: the line is one of particles.)
+int64_t cd_flow_max_n(int dim, int precision, int blocks)
+{
+    if (precision == CD_FP32) return (int64_t)blocks * (dim == 2 ? 2300 : 1100);
+    return dim == 2 ? (int64_t)blocks * 6000 : INT64_MAX;
+}
+
 static cudaError_t flow_launch(const CdGeom& g, const CdWork& w, const CdState* io, int blocks, int records, int precision, int criterion,
                                double alpha, int max_sweeps, cudaStream_t s, int* nl)
 {

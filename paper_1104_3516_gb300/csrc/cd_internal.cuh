@@ -574,6 +574,7 @@ cudaError_t cd_launch_flow_batch(const CdGeom& g, const CdWork& w, int blocks, i
                                  int criterion, double alpha, int max_sweeps, cudaStream_t stream, int* nl);
 size_t cd_flow_body_bytes(int dim, int precision);
 int cd_flow_records(const CdGeom& g, int precision, int device);
+int64_t cd_flow_max_n(int dim, int precision, int blocks);
 int cd_sweep_fits(const CdGeom& g, int precision, int threads, int per_sm);
 cudaError_t cd_launch_unpack(const CdGeom& g, const CdWork& w, double* pos, double* vel, double* omega,
                              double* theta, int integrate, int precision, cudaStream_t stream, int* nl);
