@@ -43,7 +43,6 @@
 #define FLOW_WORKERS 11                           // warps that update contacts
 #define FLOW_THREADS (32 * (FLOW_WORKERS + 1))    // and one that runs the convergence test
 #define FLOW_LEAST 112                            // contacts that a block of a batched system is given at least
-#define FLOW_BARRIER_CONTACTS 30000               // see flow_leaves_batch
 #define FLOW_ROWS 8                               // rows of tagged block sums: while a block leaves those of pass p
                                                   // another may still wait for those of p - 5
 #define FLOW_SLOTS 4                              // passes whose residual terms are kept
@@ -921,27 +920,55 @@ __device__ __forceinline__ int flow_ask(const CdWork& w, int b, int target, int 
     return ask < 1 ? 1 : (ask > blocks ? blocks : ask);
 }
 
-// Whether a batch is left to the barrier schedule.  A block works on one packing
-// at a time, so with many colours (a disc squeezed between many: piles whose
-// solves hit the sweep cap) it has too few contacts of each to fill the FP64
-// pipe; a large batch has enough of all packings together.  One step,
-// dataflow / barriers: 512 packings (70,000 contacts a block) of 8 colours 379 /
-// 559 ms, 14 colours 759 / 832, 23 colours 1,386 / 1,048, 38 colours 1,386 /
-// 1,039; 128 packings (17,500 a block) of 23 colours 307 / 361, 36 colours 302 /
-// 410; 16 packings of 29 colours 46 / 189.
-__device__ __forceinline__ bool flow_leaves_batch(int K, int nc, int blocks)
+// Whether a batch is left to the barrier schedule: by what a sweep of all packings
+// takes by either, in us.  By dataflow a block has one packing at a time, `rounds` of them
+// one after another (packings that ask for several blocks in proportion), and of
+// each a chain of its colours, whose latency the contacts of one colour in one
+// block hardly fill.  Behind barriers all packings' contacts of a colour fill it
+// together, but every colour is a barrier of the grid, the sums of the tests
+// are a block's per packing, one after another, the largest of them alone at the
+// end, and more contacts than L2 holds come from memory every sweep.  The terms were
+// fitted to 370 batches of 3 to 5,000 equal packings (10 to 40,000 discs or spheres, 4
+// to 25 colours, 2,000 to 13 million contacts in all): to 7 to 14% of the dataflow's times and 3 to
+// 5% of the barriers', and the faster one is taken but in 13, where it is up to 20%
+// (most 6%) faster.  A sweep, dataflow / barriers: 150 packings of 30 discs
+// 9.1 / 29 us, 600 34 / 38, 5,000 259 / 132; FP64, 2,000 of 100 spheres with 7 contacts
+// each 750 / 253, 200 of 2,000 859 / 444; 2,000 of 3,000 discs 1,014 / 1,189.  (A gas, whose
+// contacts stay open, takes the dataflow less than that, but nothing tells beforehand.)
+struct FlowCost {
+    float round, colour, item;                      // dataflow: a round, a colour in it, 32 contacts of it in a block
+    float sweep, phase, contact, packing, largest;  // barriers: a sweep, a colour, a contact and a packing a block,
+    float far, near;                                // a contact of the largest packing, one a block beyond `near`
+};
+static FlowCost flow_cost(int dim, int precision)
 {
-    return K > 16 && nc > FLOW_BARRIER_CONTACTS * blocks;
+    if (dim == 2)
+        return precision == CD_FP64
+                   ? FlowCost{0.55f, 1.11f, 0.222f, 6.0f, 3.35f, 0.0080f, 2.65f, 0.0006f, 0.0059f, 3000.0f}
+                   : FlowCost{1.39f, 0.75f, 0.096f, 5.3f, 2.70f, 0.0034f, 2.76f, 0.0006f, 0.0067f, 9000.0f};
+    return precision == CD_FP64
+               ? FlowCost{0.0f, 2.99f, 0.510f, 4.5f, 4.57f, 0.0193f, 2.65f, 0.0006f, 0.0084f, 3000.0f}
+               : FlowCost{0.59f, 0.78f, 0.233f, 3.3f, 2.87f, 0.0056f, 2.72f, 0.0006f, 0.0062f, 9000.0f};
+}
+// K colours in all, `own` a packing; the packings ask for `asks` blocks.
+__device__ __forceinline__ bool flow_leaves_batch(const FlowCost& c, int K, float own, int nc, int largest, int asks,
+                                                  int npk, int blocks)
+{
+    const float rounds = (float)((asks + blocks - 1) / blocks);
+    const float items = fmaxf((float)nc / ((float)asks * own * 32.0f), 1.0f);
+    const float flow = rounds * (c.round + own * (c.colour + c.item * items));
+    const float each = (float)nc / (float)blocks;
+    const float barriers = c.sweep + (float)K * c.phase + c.largest * (float)largest + c.contact * each +
+                           c.far * fmaxf(each - c.near, 0.0f) + c.packing * (float)npk / (float)blocks;
+    return barriers < flow;
 }
 
-__global__ void k_flow_plan(CdGeom g, CdWork w, int blocks, int records)
+__global__ void k_flow_plan(CdGeom g, CdWork w, int blocks, int records, FlowCost cost)
 {
     __shared__ int s_at[FLOW_MAX_BLOCKS + 1];   // packings that ask for i blocks, then the next place of theirs
+    __shared__ int s_largest;
     if (w.ctrl->skip) return;
     FlowPlan* plan = w.fl_plan;
-    const bool barriers = flow_leaves_batch(w.ctrl->ncolours, w.ctrl->nc, blocks);
-    if (threadIdx.x == 0) plan->barriers = barriers;
-    if (barriers) return;
     // all packings at once if the blocks' records can hold them so
     const int room = blocks > 2 * g.npk ? blocks - g.npk : blocks / 2;
     int target = (w.ctrl->nc + room - 1) / room;
@@ -951,10 +978,28 @@ __global__ void k_flow_plan(CdGeom g, CdWork w, int blocks, int records)
     if (target < FLOW_LEAST) target = FLOW_LEAST;
     for (int i = threadIdx.x; i < 2 * g.npk + 1; i += blockDim.x) w.fl_word[i] = 0u;
     for (int i = threadIdx.x; i <= blocks; i += blockDim.x) s_at[i] = 0;
+    if (threadIdx.x == 0) s_largest = 0;
     __syncthreads();
-    for (int b = threadIdx.x; b < g.npk; b += blockDim.x) atomicAdd(&s_at[flow_ask(w, b, target, blocks)], 1);
+    for (int b = threadIdx.x; b < g.npk; b += blockDim.x) {
+        atomicAdd(&s_at[flow_ask(w, b, target, blocks)], 1);
+        atomicMax(&s_largest, w.pk_coff[b + 1] - w.pk_coff[b]);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
+        // the colours that a packing has of those there are: at most as many as there are contacts of
+        // each for every packing, and one crowded packing's own weigh as much as their
+        // contacts (1.25: in a packing alone the last colours have few)
+        const int K = w.ctrl->ncolours, nc = w.ctrl->nc;
+        float own = 0.0f, weight = 0.0f;
+        for (int k = 0; k < K; ++k) {
+            const float n = (float)(w.colour_off[k + 1] - w.colour_off[k]);
+            own += fminf(1.0f, n / (float)g.npk);
+            weight += fminf(1.0f, n * (float)K / (float)nc);
+        }
+        own = fmaxf(fminf(own, 1.25f * weight), 1.0f);
+        int asks = 0;
+        for (int ask = 1; ask <= blocks; ++ask) asks += ask * s_at[ask];
+        plan->barriers = flow_leaves_batch(cost, K, own, nc, s_largest, asks, g.npk, blocks);
         int i = 0, run = 0, used = 0;
         bool full = false;
         for (int ask = blocks; ask >= 1; --ask) {
@@ -1227,7 +1272,7 @@ cudaError_t cd_launch_flow(const CdGeom& g, const CdWork& w, const CdState& io, 
 cudaError_t cd_launch_flow_batch(const CdGeom& g, const CdWork& w, int blocks, int records, int precision,
                                  int criterion, double alpha, int max_sweeps, cudaStream_t s, int* nl)
 {
-    k_flow_plan<<<1, 512, 0, s>>>(g, w, blocks, records);
+    k_flow_plan<<<1, 512, 0, s>>>(g, w, blocks, records, flow_cost(g.dim, precision));
     ++*nl;
     cudaError_t e = flow_launch(g, w, nullptr, blocks, records, precision, criterion, alpha, max_sweeps, s, nl);
     if (e != cudaSuccess) return e;
