@@ -297,7 +297,8 @@ cd_status cd_set_contacts(cd_system* sys, int64_t nc, const int32_t* pairs, cons
  * synchronised).  Returns CD_ERR_NOT_CONVERGED (informational) when the
  * sweep cap was hit and out was given.  A set without a colour order (its
  * preparation failed, or a loaded checkpoint brought another one) is not
- * solved: CD_ERR_STATE if out was given. */
+ * solved, unless it is a plain system's and empty: CD_ERR_STATE if out was
+ * given. */
 cd_status cd_solve_contacts(cd_system* sys, cd_solve_stats* out);
 
 /* n_steps full time steps (Fig. 3): detection (as cd_detect_contacts), the

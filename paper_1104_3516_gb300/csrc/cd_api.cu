@@ -242,13 +242,14 @@ static size_t layout(cd_system* s, char* base, CdWork* w)
 // ---------------------------------------------------------------------------
 // Helpers
 // ---------------------------------------------------------------------------
-// solve: the call uses the colour order as it is.
+// solve: the call uses the colour order as it is (2: a batch, whose packings'
+// contact ranges belong to it even where there is none).
 __global__ void k_begin_call(CdCtrl* ctrl, int reset_accum, int solve = 0)
 {
     ctrl->skip = 0;
     ctrl->overflow = 0;
     ctrl->error = CDE_NONE;
-    if (solve && (ctrl->order_lost || ctrl->order_nc != ctrl->nc)) {
+    if (solve && (ctrl->nc > 0 || solve == 2) && (ctrl->order_lost || ctrl->order_nc != ctrl->nc)) {
         ctrl->skip = 1;
         ctrl->error = CDE_ORDER;
     }
@@ -855,7 +856,7 @@ extern "C" cd_status cd_solve_contacts(cd_system* s, cd_solve_stats* out)
     cd_status st = need_ready(s);
     if (st != CD_OK) return st;
     if (!s->has_contacts) return fail(s, CD_ERR_STATE, "no contact set: call cd_detect_contacts or cd_set_contacts");
-    k_begin_call<<<1, 1, 0, s->stream>>>(s->w.ctrl, 1, 1);
+    k_begin_call<<<1, 1, 0, s->stream>>>(s->w.ctrl, 1, s->g.npk > 1 ? 2 : 1);
     if ((st = launch_solve(s, 0, 0)) != CD_OK) return st;
     if (!solve_unpacks(s))
         CD_CUDA(s, cd_launch_unpack(s->g, s->w, s->pos, s->vel, s->omega, s->theta, 0, (int)s->p.precision, s->stream,

@@ -437,7 +437,7 @@ __device__ __forceinline__ bool flow_solve(const CdGeom& g, const CdWork& w, Flo
     T4* Vprev = (T4*)w.fl_Vprev;
     constexpr int RW = (DIM == 2) ? 1 : 2;
     const int nprev = g.n + 6;                        // records in Vprev (a view is taken back with its particle)
-    const int nview = VIEWS ? w.view_off[g.n] : 0;    // records of the domains past the particles' own
+    const int nview = VIEWS && nc > 0 ? w.view_off[g.n] : 0;   // records of the domains past the particles' own
     const int vbase = cd_view_base(g);
     const int KX = VIEWS ? K + 1 : K;
 
@@ -872,7 +872,8 @@ k_flow(CdGeom g, CdWork w, CdState io, int crit, double alpha, int max_sweeps, i
     __shared__ double s_red[FLOW_WORKERS + 1][3];
     CdCtrl* ctrl = w.ctrl;
     if (ctrl->skip) return;
-    const int nc = ctrl->nc, K = ctrl->ncolours, nb = gridDim.x;
+    // (a set without contacts may have no colour order: a checkpoint can bring one)
+    const int nc = ctrl->nc, K = nc > 0 ? ctrl->ncolours : 0, nb = gridDim.x;
     const FlowTeam tm{reinterpret_cast<unsigned*>(&ctrl->bar_count), 0, nb, (int)blockIdx.x, nb};
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         sh.lo[k] = w.colour_off[k];

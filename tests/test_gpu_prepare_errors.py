@@ -114,3 +114,33 @@ def test_detection_without_workspace_counts_what_it_refuses(n):
         assert e.value.status == cd.CD_ERR_CAPACITY and e.value.needed == 140   # 70 on the large disc, 70 along the ring
     wl.x = good
     assert len(_noalloc(wl, 1000)[0]) == 70
+
+
+@pytest.mark.parametrize("kw", [{}, {"max_sweeps": 50}, {"domains": (2, 2, 1)}, {"timing": 1}])
+def test_an_empty_set_from_a_checkpoint_is_solved(kw):
+    wl, (good, _) = ringed(500, large_first=True)
+    g = gpu_system(wl, **kw)
+    empty = g.save_checkpoint()
+    for detected in (False, True):
+        if detected:
+            g.detect_contacts()
+        g.load_checkpoint(empty)
+        before = whole(g)
+        st = g.solve_contacts()
+        assert st["converged"] and st["sweeps"] == 0 and st["n_contacts"] == 0
+        for a, b in zip(before, whole(g)):
+            assert np.array_equal(a, b)
+
+
+def test_a_batch_solves_what_it_has_ranges_for():
+    packs = [W.settling_discs(seed=s, n=60, vsig=0.5) for s in (1, 2)]
+    g = gpu_system(packs[0], batch=packs, max_sweeps=200)
+    empty = g.save_checkpoint()
+    assert g.detect_contacts() > 0
+    g.solve_contacts()
+    full = g.save_checkpoint()
+    g.load_checkpoint(empty)
+    with pytest.raises(cd.CDError, match="colour order"):
+        g.solve_contacts()
+    g.load_checkpoint(full)
+    g.solve_contacts()
