@@ -42,6 +42,7 @@
 
 #define FLOW_WORKERS 11                           // warps that update contacts
 #define FLOW_THREADS (32 * (FLOW_WORKERS + 1))    // and one that runs the convergence test
+#define FLOW_TAIL 4                               // rounds of packings left from which teams are cut whatever is left over
 #define FLOW_LEAST 112                            // contacts that a block of a batched system is given at least
 #define FLOW_ROWS 8                               // rows of tagged block sums: while a block leaves those of pass p
                                                   // another may still wait for those of p - 5
@@ -901,16 +902,18 @@ k_flow(CdGeom g, CdWork w, CdState io, int crit, double alpha, int max_sweeps, i
 // packings' teams are laid out in advance until the grid is full; a team that is
 // done takes the largest packing left that asks for no more blocks than it has.
 // What is left of the team becomes one of its own if it is a third as many or
-// more (the first part so keeps at least as many blocks as any packing left asks
-// for: none is left over); fewer stay, without contacts, since blocks once cut off
-// do not come back together for a large packing.  One step from zero
+// more, or near the end (the first part so keeps at least as many blocks as any
+// packing left asks for: none is left over); before that fewer stay, without
+// contacts, since blocks once cut off do not come back together for a large
+// packing.  One step from zero
 // forces against the barrier schedule, which swept all packings together and
 // summed each one's |P| in a single block: 8 packings 45.4 -> 12.6 ms, 23 57.6
-// -> 17.8, 64 94 -> 55, 128 150 -> 105, 300 356 -> 233, 512 537 -> 394; from 64 on
+// -> 17.5, 64 94 -> 55, 128 150 -> 91, 300 356 -> 229, 512 537 -> 394; from 64 on
 // the FP64 pipe bounds it (128: 67 ms).  With the blocks left over given contacts
 // too, which depends on timing: 102, 228 and 379 for the last three.  Cut always:
-// 91, 352, 715; for a half or more: 106, 246, 407; for a whole: 109, 278, 469.  A
-// reserve of 32 contacts for every colour in
+// 91, 352, 715; for a third or more to the end: 105, 233, 395; for a half: 106, 246, 407; for a
+// whole: 109, 278, 469; from 3 rounds before the end 100, 230, 395, from 6 91, 231, 394 (200
+// packings 162 -> 178).  A reserve of 32 contacts for every colour in
 // place of 128 for all: the fourth step of 64 packings, whose most crowded disc
 // has 29 contacts, 379 ms against 173 (285 with barriers).
 // ---------------------------------------------------------------------------
@@ -1018,6 +1021,7 @@ __global__ void k_flow_plan(CdGeom g, CdWork w, int blocks, int records, FlowCos
             plan->end[ask] = run;
         }
         w.fl_start[i] = used;
+        plan->left = asks - used;
         plan->target = target;
         plan->placed = i;
     }
@@ -1087,13 +1091,24 @@ k_flow_batch(CdGeom g, CdWork w, int crit, double alpha, int max_sweeps, int rec
             const FlowTeam tm{&w.fl_word[slot], start, nb, me - start, nb};
             if (tm.blk == 0 && threadIdx.x < 32) {
                 const int x = flow_take(plan, nb);
-                if (threadIdx.x == 0) *(volatile int*)&w.fl_mail[slot] = x;
+                if (threadIdx.x == 0) {
+                    int mail = -1;
+                    if (x >= 0) {
+                        // whether what is left over becomes a team of its own
+                        const int ask = flow_ask(w, w.fl_list[x], target, (int)gridDim.x);
+                        const int left = atomicSub(&plan->left, ask) - ask;
+                        mail = 2 * x + (3 * nb >= 4 * ask || left < FLOW_TAIL * (int)gridDim.x ? 1 : 0);
+                    }
+                    *(volatile int*)&w.fl_mail[slot] = mail;
+                }
             }
             if (!tm.sync(ctrl)) return;
             at = cd_ld_volatile_int(&w.fl_mail[slot]);
             if (at < 0) return;
+            const bool cut = at & 1;
+            at >>= 1;
             const int ask = flow_ask(w, w.fl_list[at], target, (int)gridDim.x);
-            if (3 * nb < 4 * ask) break;   // what is left over is not worth a team of its own
+            if (!cut || nb == ask) break;
             given = me < start + ask;
             if (given) {
                 nb = ask;

@@ -96,6 +96,7 @@ struct FlowPlan {
     int barriers;               // 1: this solve is left to k_sweep_batch
     int target;                     // contacts a block is given
     int placed;                     // packings whose teams are laid out in advance
+    int left;                       // blocks that the packings not taken yet ask for
     int head[FLOW_MAX_BLOCKS + 1];  // packings that ask for g blocks: the next one of them to be taken,
     int end[FLOW_MAX_BLOCKS + 1];   // and the end of them, in fl_list
 };
