@@ -668,8 +668,7 @@ def run_batched(args, device, rank, flush, ws=1):
         b.max_sweeps = args.max_sweeps
         b.alpha = args.alpha
     prec = cd.CD_FP64 if args.precision == "f64" else cd.CD_FP32
-    # the default block shape, whose schedule is chosen for each solve: the tuner times solves of 40 sweeps, of
-    # which laying out the teams is a quarter
+    # the default block shape, whose schedule is chosen for each solve by the batch at hand
     shape, tuned = {}, None
     # steps replayed from a captured CUDA graph (use_graph needs its own stream and timing 0);
     # the batch's working set (~1 GB) is larger than L2, so the steps run back to back
