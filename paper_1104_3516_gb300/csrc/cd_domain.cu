@@ -46,7 +46,11 @@ __device__ __forceinline__ int contact_domain(const CdGeom& g, const CdWork& w, 
 
 __global__ void k_dom_contact(CdGeom g, CdWork w, const double* __restrict__ pos, const double* __restrict__ radius)
 {
-    if (w.ctrl->skip) return;
+    if (w.ctrl->skip) {
+        // (the view counts are cleared all the same: a set that stays current has lost its records)
+        if (blockIdx.x == 0 && threadIdx.x == 0) w.ctrl->order_lost = 1;
+        return;
+    }
     const int nc = w.ctrl->nc;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x)
         w.dom_key[c] = contact_domain(g, w, pos, radius, c);

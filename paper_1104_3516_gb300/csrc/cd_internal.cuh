@@ -67,7 +67,7 @@ struct CdCtrl {
     // the colour order belongs to the current set: both, so that a solve by itself
     // does not run on an order that was never finished
     int order_nc;                   // contacts of the set that was ordered last (-1: the current one was not)
-    int order_lost;                 // 1: a block gave up while it was being prepared
+    int order_lost;                 // 1: a block gave up while it was being prepared, or its domain records are gone
 };
 
 // Parameters of one packing of a batched system (a plain system is a batch of

@@ -144,3 +144,31 @@ def test_a_batch_solves_what_it_has_ranges_for():
         g.solve_contacts()
     g.load_checkpoint(full)
     g.solve_contacts()
+
+
+@pytest.mark.parametrize("timing", [0, 1])
+@pytest.mark.parametrize("domains", [(1, 1, 1), (2, 2, 1)])
+def test_a_set_that_outlives_a_failed_step(timing, domains):
+    """More contacts than room: the set before stays, and is solved with its colour
+    order; not where its domain records went."""
+    wl, (good, _) = ringed(500, large_first=True)
+    more = good.copy()
+    more[71:106] = good[1:36] + 0.05   # 35 discs of the field into the ring
+    kw = dict(timing=timing, domains=domains, max_sweeps=200, max_contacts=100)
+    g, twin = gpu_system(wl, **kw), gpu_system(wl, **kw)
+    for s in (g, twin):
+        assert s.detect_contacts() == 70
+    put(g, more, wl.v)
+    with pytest.raises(cd.CDError, match="capacity 100 exceeded"):
+        g.step(1)
+    put(g, good, wl.v)
+    if domains == (1, 1, 1):
+        assert g.solve_contacts()["n_contacts"] == 70
+        twin.solve_contacts()
+        for a, b in zip(whole(g), whole(twin)):
+            assert np.array_equal(a, b)
+    else:
+        with pytest.raises(cd.CDError, match="colour order"):
+            g.solve_contacts()
+        assert g.detect_contacts() == 70
+        g.solve_contacts()
